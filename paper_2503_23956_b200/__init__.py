@@ -120,6 +120,10 @@ def _ptr(t) -> int | None:
 
 def _stream(stream) -> int | None:
     if stream is None:
+        if torch.cuda.is_initialized():
+            # the raw handle: torch.cuda.current_stream() builds a Stream object around it first (3.4 against 0.4 us
+            # per call of an entry point whose kernel may take 5)
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
         stream = torch.cuda.current_stream()
     if isinstance(stream, int):
         return stream or None
@@ -283,4 +287,4 @@ def aircache_pipeline_host(sh, h_full, full_elems, d_full_k, d_full_v, h_q_windo
 def _nbytes(t) -> int:
     if t is None or isinstance(t, int):
         return 0
-    return t.numel() * t.element_size()
+    return t.nbytes

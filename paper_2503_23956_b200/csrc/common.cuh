@@ -13,6 +13,7 @@ constexpr int kMaxWindow = 128;
 constexpr int kMaxGroup = 16;         // query heads per KV head
 constexpr int kMaxRegions = 1792;     // L * B (the decode kernel keeps the unit prefix of all regions in shared memory)
 constexpr int kMaxDecodeCtas = 256;   // upper bound on the persistent decode grid (sizes the partial slots)
+constexpr int kMaxDevices = 64;       // devices whose properties are kept after the first look
 constexpr int kScoreKeyTile = 128;    // visual keys per CTA of the importance pass
 constexpr float kLog2e = 1.4426950408889634f;
 // status word left by aircache_compact when the device-side budgets / offsets / lists do not fit the buffers
@@ -104,15 +105,11 @@ constexpr int kOnePassMinKeys = 256;
 constexpr int kOnePassMaxKeys = 1024;
 inline int onepass_chunks(int n_visual) { return (n_visual + kOnePassMinKeys - 1) / kOnePassMinKeys; }
 
-// The most (group, chunk) cells of statistics any call on this shape can have (it sizes the workspace).
+// The most (group, chunk) cells of statistics any call on this shape can have (it sizes the workspace).  score_chunks
+// never cuts finer than 256 keys, so the one-pass layout is the larger one for every number of layers.  (Searching
+// the layer counts for the largest product cost 1.6 us of host time per look at the workspace, twice a call.)
 inline int64_t score_chunk_cells(const aircache_shape_t *s) {
-    int64_t most = (int64_t)s->n_layers * s->batch * s->n_kv_heads * onepass_chunks(s->n_visual);
-    for (int layers = 1; layers <= s->n_layers; ++layers) {
-        const int64_t groups = (int64_t)layers * s->batch * s->n_kv_heads;
-        const int64_t cells = groups * score_chunks(s->n_visual, groups);
-        if (cells > most) most = cells;
-    }
-    return most;
+    return (int64_t)s->n_layers * s->batch * s->n_kv_heads * onepass_chunks(s->n_visual);
 }
 
 struct WsLayout {

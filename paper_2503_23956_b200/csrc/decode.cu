@@ -34,6 +34,7 @@
 // workspace, raises a CTA-wide abort flag and the kernel drains and returns.
 #include <cuda.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -1151,10 +1152,13 @@ int make_map(CUtensorMap *tm, const void *base, int D, int Hkv, int64_t rows, in
     return AIRCACHE_OK;
 }
 
-int sm_count(int *out) {
-    int dev = 0;
-    AIRCACHE_CUDA_TRY(cudaGetDevice(&dev));
-    AIRCACHE_CUDA_TRY(cudaDeviceGetAttribute(out, cudaDevAttrMultiProcessorCount, dev));
+// The current device and its number of SMs, asked once per device (the answer never changes).
+int current_device(int *dev, int *sms) {
+    static std::atomic<int> known[kMaxDevices];
+    AIRCACHE_CUDA_TRY(cudaGetDevice(dev));
+    if (*dev >= 0 && *dev < kMaxDevices && (*sms = known[*dev].load(std::memory_order_relaxed)) > 0) return AIRCACHE_OK;
+    AIRCACHE_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev));
+    if (*dev >= 0 && *dev < kMaxDevices) known[*dev].store(*sms, std::memory_order_relaxed);
     return AIRCACHE_OK;
 }
 
@@ -1165,11 +1169,16 @@ int launch_decode_t(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, c
     int rc = make_map(&tm_k, c->k, D, kv_heads, c->total_rows, C::CH);
     if (rc) return rc;
     if ((rc = make_map(&tm_v, c->v, D, kv_heads, c->total_rows, C::CH))) return rc;
-    int sms = 0;
-    if ((rc = sm_count(&sms))) return rc;
+    int dev = 0, sms = 0;
+    if ((rc = current_device(&dev, &sms))) return rc;
     const int ctas = sms < kMaxDecodeCtas ? sms : kMaxDecodeCtas;
-    AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, HKV, G_HI, HS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           C::SMEM_BYTES));
+    // the shared-memory limit is a property of the kernel on a device: set once for each
+    static std::atomic<bool> ready[kMaxDevices];
+    if (dev >= kMaxDevices || !ready[dev].load(std::memory_order_acquire)) {
+        AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, HKV, G_HI, HS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               C::SMEM_BYTES));
+        if (dev < kMaxDevices) ready[dev].store(true, std::memory_order_release);
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(C::THREADS);
@@ -1199,8 +1208,8 @@ int launch_decode_g(const aircache_ragged_t *c, DecodeParams &p, cudaStream_t st
 template <int D>
 int launch_decode_d(const aircache_shape_t *s, const aircache_ragged_t *c, DecodeParams &p, cudaStream_t st) {
     const int hkv = s->n_kv_heads;
-    int sms = 0;
-    int rc = sm_count(&sms);
+    int dev = 0, sms = 0;
+    int rc = current_device(&dev, &sms);
     if (rc) return rc;
     if (p.n_regions * hkv <= (sms < kMaxDecodeCtas ? sms : kMaxDecodeCtas)) {   // also with one KV head: an item is a region
         p.hs = hkv;
@@ -1274,7 +1283,6 @@ int launch_decode(const aircache_shape_t *s, const aircache_ragged_t *c, const v
 static __device__ __align__(256) unsigned char g_static_scratch[AIRCACHE_STATIC_SCRATCH_BYTES];
 
 namespace {
-constexpr int kMaxDevices = 64;
 std::mutex g_static_mutex;
 unsigned char *g_static_ptr[kMaxDevices] = {};
 }  // namespace
@@ -1282,9 +1290,9 @@ unsigned char *g_static_ptr[kMaxDevices] = {};
 int launch_decode_static(const aircache_shape_t *s, const aircache_ragged_t *c, const void *q, float *out,
                          cudaStream_t st) {
     int dev = 0, sms = 0;
-    AIRCACHE_CUDA_TRY(cudaGetDevice(&dev));
+    int rc = current_device(&dev, &sms);
+    if (rc) return rc;
     if (dev < 0 || dev >= kMaxDevices) return AIRCACHE_ERR_UNSUPPORTED;
-    AIRCACHE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t ctas = sms < kMaxDecodeCtas ? sms : kMaxDecodeCtas;
     const int64_t need = kStatusBytes + 2 * ctas * partial_slot_floats(s->n_q_heads, s->head_dim) * 4;
     if (need > (int64_t)AIRCACHE_STATIC_SCRATCH_BYTES) return AIRCACHE_ERR_STATIC_SCRATCH;
