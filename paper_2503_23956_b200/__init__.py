@@ -287,4 +287,4 @@ def aircache_pipeline_host(sh, h_full, full_elems, d_full_k, d_full_v, h_q_windo
 def _nbytes(t) -> int:
     if t is None or isinstance(t, int):
         return 0
-    return t.nbytes
+    return t.numel() * t.element_size()
