@@ -1,7 +1,8 @@
 // aircache_score: importance of every visual token seen from the elite observation window
 // (Section 3.3, Eq. 4-8), all layers and sequences per launch.
 //
-// Kernels on one stream:
+// Sequences of up to 16384 visual tokens are scored by the cluster kernel of score_cluster.cu.  Here is the rest:
+// longer ones, caches that no tensor map describes, and alpha = 0 with 32 window rows or more.  Kernels on one stream:
 //   elite_kernel       one CTA per (layer, sequence, KV head): the W candidate keys and the last text query
 //                      are staged in shared memory; Eq. 4 logits as fp64 dot products in element order (so
 //                      the Eq. 5 decision does not depend on a summation order), the elite set of each
@@ -10,7 +11,7 @@
 //                      It also leaves a gathered copy of the group's first 16 elite query rows.
 //   onepass_kernel     Eq. 7 and Eq. 8 with one read of the visual keys: Q_tk K_v^T on tensor cores (keys on
 //   + group_sum_kernel the M axis, elite rows on N), a chunk's logits kept in shared memory between the
-//                      statistics and the probabilities; see the comment at the kernel.  The normal path.
+//                      statistics and the probabilities; see the comment at the kernel.
 //   stats_kernel       the same in two passes, for sequences too long for the one-pass kernel.  Pass one:
 //   + importance_kernel running (max, sum of exp2) of every elite row over one chunk of visual keys; the CTA
 //                      that finishes a KV group last (ticket) merges the chunks and the text statistics
@@ -25,45 +26,11 @@
 
 #include <mutex>
 
-#include "common.cuh"
-#include "ptx.cuh"
+#include "score.cuh"
 
 namespace aircache {
 
 namespace {
-
-struct ScoreParams {
-    const uint16_t *k;
-    int64_t s_layer, s_batch, s_head, s_token;
-    const uint16_t *qw;  // [L,B,W,Hq,d]
-    float *scores;       // [L,B,Nv]
-    uint64_t *elite_mask;
-    int32_t *row_count;
-    int32_t *row_info;
-    float *row_coef;
-    float2 *row_text;
-    float2 *chunk_stats;
-    float2 *row_final;   // (max, weight / normaliser) per elite row, written by the last stats CTA of a group
-    uint32_t *group_ticket;
-    uint32_t *dispatch;     // one-pass scoring: blocks started so far
-    float *imp_part;        // one-pass scoring: [L*B*Hkv][Nv] importance of one KV group
-    uint16_t *q_block;      // one-pass scoring: [L*B*Hkv][16][d] the first 16 elite query rows, gathered
-    int op_chunks;      // numbers (blocks) per KV group in the one-pass grid
-    int op_tile_cap;    // most 16-key tiles a warp of the one-pass kernel takes: 16, or fewer when the call is small
-    int L, B, Hq, Hkv, G, d, Nv, Nt, W;
-    int lb0, n_lb;   // the launch covers regions lb0 .. lb0 + n_lb - 1 (a range of layers)
-    int per_head;    // scores are kept apart per KV group: [L,B,Hkv,Nv], Eq. 8 averaged over the group's heads only
-    int cap, chunks, chunk_keys;
-    float scale, sl2, ln_alpha;
-    int keep_all;
-    // one stats launch handles the KV groups with rows_lo < elite rows <= rows_hi
-    int rows_lo, rows_hi;
-    // dense (tcgen05) path: position of the token / head / sequence / layer coordinate in the key tensor map
-    int pos_token, pos_head, pos_batch, pos_layer;
-    uint32_t *status;
-};
-
-constexpr float kNegBig = -1.0e30f;
 
 // ---------------------------------------------------------------------------------------------
 // Eq. 4-5 and the elite-row table
@@ -738,6 +705,9 @@ __global__ void __launch_bounds__(128, 5) onepass_kernel(ScoreParams p) {
 __global__ void __launch_bounds__(256) group_sum_kernel(ScoreParams p) {
     const int lb = p.lb0 + blockIdx.y;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    // launched ahead of its predecessor's end: nothing is read before the wait
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (i >= p.Nv) return;
     const float *src = p.imp_part + (int64_t)lb * p.Hkv * p.Nv + i;
     float v = 0.f;
@@ -772,11 +742,7 @@ int launch_onepass(const ScoreParams &p, cudaStream_t st) {
     const int64_t blocks = (int64_t)p.n_lb * p.Hkv * p.op_chunks;
     onepass_kernel<D><<<(unsigned)blocks, 128, 32768, st>>>(p);
     AIRCACHE_LAUNCH_CHECK();
-    if (!p.per_head) {
-        group_sum_kernel<<<dim3((p.Nv + 255) / 256, (unsigned)p.n_lb), 256, 0, st>>>(p);
-        AIRCACHE_LAUNCH_CHECK();
-    }
-    return AIRCACHE_OK;
+    return p.per_head ? AIRCACHE_OK : launch_group_sum(p, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -848,17 +814,6 @@ __device__ __forceinline__ void issue_tile_mma(uint32_t tmem_d, uint32_t a_base,
         const uint32_t off = (kk >> 2) * SUB + (kk & 3) * 32;
         umma_bf16(tmem_d, umma_desc_sw128(a_base + off), umma_desc_sw128(b_base + off), idesc, kk > 0 ? 1u : 0u);
     }
-}
-
-template <int D>
-__device__ __forceinline__ void load_key_tile(uint32_t dst, const CUtensorMap *tm, const ScoreParams &p, int key,
-                                              int g, int b, int l, uint32_t bar) {
-    int c[5] = {0, 0, 0, 0, 0};
-    c[p.pos_token] = key; c[p.pos_head] = g; c[p.pos_batch] = b; c[p.pos_layer] = l;
-    mbar_expect_tx(bar, DenseCfg<D>::TILE_BYTES);
-#pragma unroll
-    for (int sub = 0; sub < DenseCfg<D>::KSUB; ++sub)
-        tma_load_5d(dst + sub * DenseCfg<D>::SUB_BYTES, tm, sub * 64, c[1], c[2], c[3], c[4], bar);
 }
 
 // Both dense kernels are warp-specialised: two sets of four epilogue warps (warps 0-3 and 4-7; a thread owns one
@@ -1236,38 +1191,6 @@ int launch_passes_d(const ScoreParams &p, cudaStream_t st) {
     return nt_max <= 4 ? launch_importance<D, 4>(p, st) : launch_importance<D, 8>(p, st);
 }
 
-// 5-D tensor map over the caller's key cache: channels innermost, then token / head / sequence / layer in
-// the order of their strides (smallest first); one box = 64 channels x 128 tokens.
-int make_key_map(CUtensorMap *tm, ScoreParams &p, const aircache_shape_t *s, const aircache_full_t *f) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return AIRCACHE_ERR_CUDA;
-    struct Dim { int64_t size, stride; int which; };
-    Dim dims[4] = {{(int64_t)s->n_visual + s->n_text, f->stride_token, 0}, {s->n_kv_heads, f->stride_head, 1},
-                   {s->batch, f->stride_batch, 2}, {s->n_layers, f->stride_layer, 3}};
-    for (int i = 0; i < 4; ++i)
-        for (int j = i + 1; j < 4; ++j)
-            if (dims[j].stride < dims[i].stride || (dims[j].stride == dims[i].stride && dims[j].size < dims[i].size)) {
-                const Dim t = dims[i]; dims[i] = dims[j]; dims[j] = t;
-            }
-    cuuint64_t gdim[5] = {(cuuint64_t)s->head_dim, 1, 1, 1, 1};
-    cuuint64_t gstr[4] = {0, 0, 0, 0};
-    cuuint32_t box[5] = {64, 1, 1, 1, 1};
-    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    int pos[4] = {0, 0, 0, 0};
-    for (int i = 0; i < 4; ++i) {
-        gdim[i + 1] = (cuuint64_t)dims[i].size;
-        // a dimension of extent 1 never moves; give it the smallest stride the encoder accepts
-        gstr[i] = (cuuint64_t)(dims[i].stride > 0 ? dims[i].stride : s->head_dim) * 2;
-        pos[dims[i].which] = i + 1;
-        if (dims[i].which == 0) box[i + 1] = 128;
-    }
-    p.pos_token = pos[0]; p.pos_head = pos[1]; p.pos_batch = pos[2]; p.pos_layer = pos[3];
-    const CUresult rc = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(f->k), gdim, gstr, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return rc == CUDA_SUCCESS ? AIRCACHE_OK : AIRCACHE_ERR_CUDA;
-}
-
 template <int D>
 int launch_dense(ScoreParams &p, const CUtensorMap &tm, cudaStream_t st) {
     using C = DenseCfg<D>;
@@ -1278,14 +1201,24 @@ int launch_dense(ScoreParams &p, const CUtensorMap &tm, cudaStream_t st) {
     AIRCACHE_LAUNCH_CHECK();
     dense_importance_kernel<D><<<dim3(p.chunks, (unsigned)((int64_t)p.n_lb * p.Hkv)), kDenseThreads, C::SMEM_IMP, st>>>(tm, p);
     AIRCACHE_LAUNCH_CHECK();
-    if (!p.per_head) {
-        group_sum_kernel<<<dim3((p.Nv + 255) / 256, (unsigned)p.n_lb), 256, 0, st>>>(p);
-        AIRCACHE_LAUNCH_CHECK();
-    }
-    return AIRCACHE_OK;
+    return p.per_head ? AIRCACHE_OK : launch_group_sum(p, st);
 }
 
 }  // namespace
+
+int launch_group_sum(const ScoreParams &p, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((p.Nv + 255) / 256, (unsigned)p.n_lb);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    AIRCACHE_CUDA_TRY(cudaLaunchKernelEx(&cfg, group_sum_kernel, p));
+    return AIRCACHE_OK;
+}
 
 int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void *q_window, float alpha,
                  int layer_begin, int layer_count, float *scores, uint64_t *elite_mask, void *ws, cudaStream_t st) {
@@ -1336,6 +1269,11 @@ int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void
     p.pos_token = p.pos_head = p.pos_batch = p.pos_layer = 0;
     p.status = ws_ptr<uint32_t>(ws, w.status);
 
+    if (!(p.keep_all && p.G * p.W >= 32)) {
+        int taken = 0;
+        const int rc = launch_score_cluster(p, s, f, st, &taken);
+        if (rc || taken) return rc;
+    }
     const int64_t groups = (int64_t)p.n_lb * p.Hkv;
     const size_t elite_smem = (size_t)(p.W + p.G) * (p.d + 8) * 2;
     if (p.keep_all) {

@@ -1,0 +1,36 @@
+"""The cluster scoring kernel at the edges of its range: one tile, tile and block boundaries, the longest sequence it
+takes and the first it does not, several units of 16 elite rows, and logits spread so far that the exponent reference
+of a row has to move.  Against the CPU oracle, element by element, within the suite's 2e-3 (a logit of 100 in the
+log2 domain, summed in fp32 over 128 exact products, is off by some 1e-4 at most)."""
+import numpy as np
+import pytest
+
+from harness import GpuPath, gen_inputs, logical, oracle_dims, rel_elem_err, u16
+from workloads import Workload
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("n_visual,d,window,alpha,sharp,per_head", [
+    (3, 128, 4, 0.9, 1.0, 0), (128, 64, 16, 0.9, 1.0, 0), (129, 128, 16, 0.9, 1.0, 1), (1025, 128, 16, 0.5, 1.0, 0),
+    (2049, 64, 64, 0.3, 1.0, 0), (2500, 128, 16, 0.9, 6.0, 0), (3000, 64, 32, 0.2, 6.0, 1),
+    (16384, 128, 16, 0.9, 1.0, 0), (16385, 128, 16, 0.9, 1.0, 0)])
+def test_scores_at_the_edges(oracle_mod, n_visual, d, window, alpha, sharp, per_head):
+    wl = Workload("edge", 2, 14, 2, d, batch=2, n_visual=n_visual, n_text=70, ratio=0.1, steps=1, window=window,
+                  alpha=alpha)
+    scale = sharp / d ** 0.5
+    k, v, qw = gen_inputs(wl, "cpu")
+    score = oracle_mod.score_groups if per_head else oracle_mod.score
+    ref = score(oracle_dims(oracle_mod, wl), u16(logical(k)), u16(qw), scale, alpha)
+    gp = GpuPath(wl, device=DEV, per_kv_head=per_head)
+    gp.sh.scale = scale
+    gp.set_full(logical(k.to(DEV)), logical(v.to(DEV)))
+    for _ in range(2):   # the second call finds the workspace as the first left it
+        gp.scores.fill_(float("nan"))
+        gp.score(qw.to(DEV), alpha=alpha)
+        assert gp.status() == 0
+        assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
+        err = rel_elem_err(gp.scores.cpu().numpy(), ref["scores"])
+        assert err <= 2e-3, err
+
