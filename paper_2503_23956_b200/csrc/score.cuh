@@ -76,16 +76,27 @@ inline int make_key_map(CUtensorMap *tm, ScoreParams &p, const aircache_shape_t 
 constexpr int kKeySubBytes = 128 * 128;   // 128 keys x 64 channels
 
 #ifdef __CUDACC__
+// Coordinates 1 to 4 of a key in that map.  (Selects: an array indexed by position would live in local memory.)
+__device__ __forceinline__ int4 key_coords(const ScoreParams &p, int key, int g, int b, int l) {
+    auto at = [&](int i) { return p.pos_token == i ? key : p.pos_head == i ? g : p.pos_batch == i ? b : l; };
+    return make_int4(at(1), at(2), at(3), at(4));
+}
 // One tile of 128 keys (D / 64 boxes of 64 channels, 128-byte swizzle) of KV head g of sequence b, layer l.
 template <int D>
 __device__ __forceinline__ void load_key_tile(uint32_t dst, const CUtensorMap *tm, const ScoreParams &p, int key,
                                               int g, int b, int l, uint32_t bar) {
-    int c[5] = {0, 0, 0, 0, 0};
-    c[p.pos_token] = key; c[p.pos_head] = g; c[p.pos_batch] = b; c[p.pos_layer] = l;
+    const int4 c = key_coords(p, key, g, b, l);
     mbar_expect_tx(bar, D / 64 * kKeySubBytes);
 #pragma unroll
     for (int sub = 0; sub < D / 64; ++sub)
-        tma_load_5d(dst + sub * kKeySubBytes, tm, sub * 64, c[1], c[2], c[3], c[4], bar);
+        tma_load_5d(dst + sub * kKeySubBytes, tm, sub * 64, c.x, c.y, c.z, c.w, bar);
+}
+// The same tile asked into L2.
+template <int D>
+__device__ __forceinline__ void prefetch_key_tile(const CUtensorMap *tm, const ScoreParams &p, int key, int g, int b, int l) {
+    const int4 c = key_coords(p, key, g, b, l);
+#pragma unroll
+    for (int sub = 0; sub < D / 64; ++sub) tma_prefetch_5d(tm, sub * 64, c.x, c.y, c.z, c.w);
 }
 
 #endif

@@ -23,8 +23,10 @@
 //
 // What it replaced (elite kernel, one-pass kernel on mma.sync with a wait between blocks, sum kernel) streamed keys
 // during half of a block's life and took three launches.  Measured, 28 layers of 28 query and 4 KV heads of 128
-// channels: 64 sequences of 2916 tokens 1180 -> 952 us (5.6 TB/s of keys); one of 7290 tokens 75 -> 56 us; four of
-// 6272, a call per layer, 33 -> 20 us a call.
+// channels: 64 sequences of 2916 tokens 1180 -> 882 us (6.1 TB/s of keys: at the memory's rate); one of 7290 tokens
+// 75 -> 51 us; four of 6272, a call per layer, 33 -> 17 us a call.  A call of one layer is a chain of latencies: some
+// 7 us until the first query block is ready (2 of them the first rows from memory), 4 us until the last tile has been
+// multiplied, 4 us for the exchange and Eq. 8.
 //
 // With up to eight tiles per block the tensor memory holds two units of work and the tensor core runs ahead of the
 // epilogue; with up to sixteen the other block of the SM fills the gap.  All waits are bounded.
@@ -49,10 +51,12 @@ constexpr int kEliteThreads = 128, kEpiThreads = 128;
 constexpr int kEliteWarp0 = 4, kEpiWarp0 = 8;
 constexpr int kSmemPerBlock = (228 * 1024) / 2 - 1024;   // two blocks per SM, 1 KB each is the system's
 constexpr float kRescale = 24.f;
+constexpr int kPreloadRows = 128;     // window queries of a group that fit a ring stage
+constexpr int kFirstAhead = 5;        // tiles asked into L2 behind the first full ring
 
 struct ClusterSmem {   // small state behind the ring and the query block
     uint64_t full[kMaxStages], empty[kMaxStages];
-    uint64_t q_full[2], meta_empty[2], q_free;
+    uint64_t q_full[2], meta_empty[2], q_free, q_all, q_taken;
     uint64_t acc_full[kSlots], acc_empty[2], exchange[2];
     float2 stats[2][kMaxCluster][kRows];   // (max, sum) of every block of the cluster
     float2 warp_stats[2][4][kRows];
@@ -72,7 +76,7 @@ struct ClusterCfg {
     static constexpr int Q_BYTES = D / 64 * Q_SUB;
     static constexpr int KS = D + 8;   // padded row of the staged candidate keys and last queries
     static int tail_bytes(int W, int G) {
-        return (int)sizeof(ClusterSmem) + (W + G) * KS * 2 + (G * W * 4 + 15) / 16 * 16;
+        return (int)sizeof(ClusterSmem) + (W + G) * KS * 2 + (G * W * 4 + (W + G) * 4 + 15) / 16 * 16;
     }
     static int stages(int W, int G) {
         const int fit = (kSmemPerBlock - Q_BYTES - tail_bytes(W, G)) / TILE_BYTES;
@@ -106,7 +110,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
     uint8_t *s_q = smem + S * C::TILE_BYTES;
     ClusterSmem &sm = *reinterpret_cast<ClusterSmem *>(s_q + C::Q_BYTES);
     uint16_t *s_k = reinterpret_cast<uint16_t *>(&sm + 1);   // [W][KS] candidate keys, then [G][KS] last queries
-    float *s_logit = reinterpret_cast<float *>(s_k + (p.W + p.G) * C::KS);
+    float *s_logit = reinterpret_cast<float *>(s_k + (p.W + p.G) * C::KS);   // [G][W]
+    float *s_norm = s_logit + p.G * p.W;                                     // 2-norm of every staged row
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank();
@@ -122,6 +127,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
             mbar_init(smem_u32(&sm.exchange[i]), 1);
         }
         mbar_init(smem_u32(&sm.q_free), 1);
+        mbar_init(smem_u32(&sm.q_all), 1);
+        mbar_init(smem_u32(&sm.q_taken), 1);
         for (int i = 0; i < kSlots; ++i) mbar_init(smem_u32(&sm.acc_full[i]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sm.abort = 0;
@@ -146,8 +153,11 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
     // Units of work, in the same order in every role: item (the cluster's share), KV group of the item, 16 rows.
     if (warp == 0) {
         // ================================ producer ================================
+        // The keys of all blocks together occupy the memory for microseconds: the few rows that the elite warps need
+        // first come in before them.
+        named_bar(3, kEliteThreads + 32);
         if (lane == 0) {
-            bool ok = true;
+            bool ok = p.W * p.G > kPreloadRows || mbar_wait(smem_u32(&sm.q_all), 0, abort_flag, p.status, 32);
             uint32_t u = 0, it = 0;
             for (int item = cid; ok && item < plan.items; item += n_clusters) {
                 for (int gi = 0; ok && gi < plan.groups_per_item; ++gi) {
@@ -155,8 +165,12 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     const int g = grp % p.Hkv, lb = grp / p.Hkv, l = lb / p.B, b = lb - l * p.B;
                     for (bool last = false; ok && !last; ++u) {
                         for (int t = 0; t < T; ++t, ++it) {
+                            if (it == (uint32_t)S - 1)   // the first query rows are some microseconds away: a few tiles more
+                                for (int t2 = t; t2 < T && t2 < S + kFirstAhead; ++t2)   // come as far as L2 meanwhile
+                                    prefetch_key_tile<D>(&tm_k, p, key0 + t2 * 128, g, b, l);
                             const uint32_t st = it % S;
-                            ok = mbar_wait(smem_u32(&sm.empty[st]), ((it / S) & 1) ^ 1, abort_flag, p.status, 20);
+                            ok = mbar_wait(smem_u32(&sm.empty[st]), ((it / S) & 1) ^ 1, abort_flag, p.status, 20) &&
+                                 (it != (uint32_t)S - 1 || mbar_wait(smem_u32(&sm.q_taken), 0, abort_flag, p.status, 31));
                             if (!ok) break;
                             load_key_tile<D>(smem_u32(s_ring + st * C::TILE_BYTES), &tm_k, p, key0 + t * 128, g, b, l,
                                              smem_u32(&sm.full[st]));
@@ -175,33 +189,41 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
         }
     } else if (warp == 1) {
         // ================================ tensor core ================================
-        if (lane == 0) {
-            bool ok = true;
-            uint32_t u = 0, it = 0;
-            const uint32_t idesc = umma_idesc_bf16(128, kRows);
-            for (int item = cid; ok && item < plan.items; item += n_clusters) {
-                for (int gi = 0; ok && gi < plan.groups_per_item; ++gi) {
-                    for (bool last = false; ok && !last; ++u) {
-                        const uint32_t buf = plan.bufs == 2 ? u & 1 : 0, use = plan.bufs == 2 ? u >> 1 : u;
-                        ok = mbar_wait(smem_u32(&sm.q_full[u & 1]), (u >> 1) & 1, abort_flag, p.status, 22) &&
-                             mbar_wait(smem_u32(&sm.acc_empty[buf]), (use & 1) ^ 1, abort_flag, p.status, 23);
+        // The whole warp walks the loop and one elected lane issues: descriptors then stay in uniform registers.  From
+        // inside a one-lane branch each instruction cost 67 clocks of moves (0.5 us per tile, whatever N is).
+        bool ok = true;
+        uint32_t u = 0, it = 0, st = 0;
+        const uint32_t idesc = umma_idesc_bf16(128, kRows);
+        const uint64_t ring_desc = umma_desc_sw128(smem_u32(s_ring)), q_desc = umma_desc_sw128(smem_u32(s_q));
+        for (int item = cid; ok && item < plan.items; item += n_clusters) {
+            for (int gi = 0; ok && gi < plan.groups_per_item; ++gi) {
+                for (bool last = false; ok && !last; ++u) {
+                    const uint32_t buf = plan.bufs == 2 ? u & 1 : 0, use = plan.bufs == 2 ? u >> 1 : u;
+                    ok = mbar_wait(smem_u32(&sm.q_full[u & 1]), (u >> 1) & 1, abort_flag, p.status, 22) &&
+                         mbar_wait(smem_u32(&sm.acc_empty[buf]), (use & 1) ^ 1, abort_flag, p.status, 23);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    last = sm.meta[u & 1].y != 0;
+                    tc_fence_after();
+                    for (int t = 0; t < T; ++t, ++it) {
+                        ok = mbar_wait(smem_u32(&sm.full[st]), (it / S) & 1, abort_flag, p.status, 24);
+                        ok = __all_sync(0xffffffffu, ok);
                         if (!ok) break;
-                        last = sm.meta[u & 1].y != 0;
-                        tc_fence_after();
-                        for (int t = 0; t < T; ++t, ++it) {
-                            const uint32_t st = it % S, slot = buf * plan.slots_per_unit + t;
-                            ok = mbar_wait(smem_u32(&sm.full[st]), (it / S) & 1, abort_flag, p.status, 24);
-                            if (!ok) break;
-                            const uint32_t a = smem_u32(s_ring + st * C::TILE_BYTES), bq = smem_u32(s_q);
+                        const uint32_t slot = buf * plan.slots_per_unit + t;
+                        const uint64_t a = ring_desc + (uint64_t)(st * (C::TILE_BYTES >> 4));
+                        if (elect_one()) {
 #pragma unroll
                             for (int kk = 0; kk < D / 16; ++kk)
-                                umma_bf16(tmem + slot * kRows, umma_desc_sw128(a + (kk >> 2) * kKeySubBytes + (kk & 3) * 32),
-                                          umma_desc_sw128(bq + (kk >> 2) * C::Q_SUB + (kk & 3) * 32), idesc, kk > 0 ? 1u : 0u);
+                                umma_bf16(tmem + slot * kRows, a + (((kk >> 2) * kKeySubBytes + (kk & 3) * 32) >> 4),
+                                          q_desc + (((kk >> 2) * C::Q_SUB + (kk & 3) * 32) >> 4), idesc, kk > 0 ? 1u : 0u);
                             umma_commit(smem_u32(&sm.empty[st]));
                             umma_commit(smem_u32(&sm.acc_full[slot]));
                         }
-                        umma_commit(smem_u32(&sm.q_free));
+                        __syncwarp();
+                        if (++st == (uint32_t)S) st = 0;
                     }
+                    if (ok && elect_one()) umma_commit(smem_u32(&sm.q_free));
+                    __syncwarp();
                 }
             }
         }
@@ -209,54 +231,168 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
         // ================================ elite rows ================================
         const int et = tid - kEliteWarp0 * 32, ew = warp - kEliteWarp0;
         const int words = (p.W + 31) >> 5;
+        const int n_vec = (p.W + p.G) * (D / 8);   // 16-byte vectors of the candidate keys and the last queries
         bool ok = true;
         uint32_t u = 0;
+        // four vectors per thread from `base` on: loaded, then stored with the norm of every row
+        auto load_rows = [&](int grp, int base, uint4 (&v)[4]) {
+            const int g = grp % p.Hkv, lb = grp / p.Hkv, l = lb / p.B, b = lb - l * p.B;
+            const uint16_t *k_cand = p.k + (int64_t)l * p.s_layer + (int64_t)b * p.s_batch + (int64_t)g * p.s_head +
+                                     (int64_t)(p.Nv + p.Nt - p.W) * p.s_token;
+            const uint16_t *q_last = p.qw + (((int64_t)lb * p.W + p.W - 1) * p.Hq + g * p.G) * D;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int idx = base + i * kEliteThreads, row = idx / (D / 8), c = idx % (D / 8);
+                v[i] = make_uint4(0u, 0u, 0u, 0u);
+                if (idx < n_vec)
+                    v[i] = __ldg(reinterpret_cast<const uint4 *>(row < p.W ? k_cand + (int64_t)row * p.s_token
+                                                                           : q_last + (int64_t)(row - p.W) * D) + c);
+            }
+        };
+        auto store_rows = [&](int base, const uint4 (&v)[4]) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int idx = base + i * kEliteThreads, row = idx / (D / 8), c = idx % (D / 8);
+                const uint32_t w4[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+                float sq = 0.f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sq = fmaf(bf16lo(w4[e]), bf16lo(w4[e]), fmaf(bf16hi(w4[e]), bf16hi(w4[e]), sq));
+#pragma unroll
+                for (int sh = 1; sh < D / 8; sh <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, sh);
+                if (idx < n_vec) {
+                    *reinterpret_cast<uint4 *>(s_k + row * C::KS + c * 8) = v[i];
+                    if (c == 0) s_norm[row] = sqrtf(sq + 1e-30f);   // (squares below fp32's range: still a bound)
+                }
+            }
+        };
+        // Eq. 4, last row only: the logit of candidate w for head hl.  The decision of Eq. 5 is defined on fp64 dot
+        // products in element order, rounded to fp32.  fp32 dot products settle it wherever the difference to the
+        // threshold exceeds what the two can differ by; a head with a candidate closer than that is done again in fp64
+        // (about one group in 200).  The fp64 chain alone took 2-4 us of a one-layer call's 19.
+        auto logit_fp32 = [&](int hl, int w) {
+            const uint4 *q = reinterpret_cast<const uint4 *>(s_k + (p.W + hl) * C::KS);
+            const uint4 *kk = reinterpret_cast<const uint4 *>(s_k + w * C::KS);
+            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 8
+            for (int c = 0; c < D / 8; ++c) {
+                const uint4 a = q[c], bb = kk[c];
+                a0 = fmaf(bf16lo(a.x), bf16lo(bb.x), a0); a1 = fmaf(bf16hi(a.x), bf16hi(bb.x), a1);
+                a2 = fmaf(bf16lo(a.y), bf16lo(bb.y), a2); a3 = fmaf(bf16hi(a.y), bf16hi(bb.y), a3);
+                a0 = fmaf(bf16lo(a.z), bf16lo(bb.z), a0); a1 = fmaf(bf16hi(a.z), bf16hi(bb.z), a1);
+                a2 = fmaf(bf16lo(a.w), bf16lo(bb.w), a2); a3 = fmaf(bf16hi(a.w), bf16hi(bb.w), a3);
+            }
+            return ((a0 + a1) + (a2 + a3)) * p.scale;
+        };
+        auto logit_fp64 = [&](int hl, int w) {
+            const uint4 *q = reinterpret_cast<const uint4 *>(s_k + (p.W + hl) * C::KS);
+            const uint4 *kk = reinterpret_cast<const uint4 *>(s_k + w * C::KS);
+            double acc = 0.0;
+#pragma unroll 1
+            for (int c = 0; c < D / 8; ++c) {
+                const uint4 a = q[c], bb = kk[c];
+                const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    // a product of two bf16 values is exact in fp64, so the fused form rounds exactly where the
+                    // separate multiply and add do
+                    acc = __fma_rn((double)bf16lo(av[e]), (double)bf16lo(bv[e]), acc);
+                    acc = __fma_rn((double)bf16hi(av[e]), (double)bf16hi(bv[e]), acc);
+                }
+            }
+            return __fmul_rn((float)acc, p.scale);
+        };
+        // How far (logit - best) can be off in fp32: per logit 34 roundings of the sum and 2 each for the scaled products,
+        // relative to |q| |k| scale (Cauchy-Schwarz), for two logits, plus the norms' own: 2 * 40 / 2^24 and a margin.
+        constexpr float kSlack = 5.5e-6f;
+
+        uint4 ahead[4];   // the first vectors of the next group, on their way while this one is worked on
+        load_rows(first_grp + cid * plan.groups_per_item, et, ahead);
+        // First unit of the block: all of the window's queries of the group come into the last ring stage at once, since
+        // which of them are elite is known two steps later only.
+        const bool preload = p.W * p.G <= kPreloadRows;
+        if (preload && et == 0) {
+            const int grp = first_grp + cid * plan.groups_per_item, g = grp % p.Hkv, lb = grp / p.Hkv;
+            mbar_expect_tx(smem_u32(&sm.q_all), p.W * p.G * D * 2);
+            for (int w = 0; w < p.W; ++w)
+                bulk_load(smem_u32(s_ring + (S - 1) * C::TILE_BYTES + w * p.G * D * 2),
+                          p.qw + (((int64_t)lb * p.W + w) * p.Hq + g * p.G) * D, p.G * D * 2, smem_u32(&sm.q_all));
+        }
+
         for (int item = cid; ok && item < plan.items; item += n_clusters) {
             for (int gi = 0; ok && gi < plan.groups_per_item; ++gi) {
                 const int grp = first_grp + item * plan.groups_per_item + gi;
-                const int g = grp % p.Hkv, lb = grp / p.Hkv, l = lb / p.B, b = lb - l * p.B;
-                const uint16_t *k_cand = p.k + (int64_t)l * p.s_layer + (int64_t)b * p.s_batch + (int64_t)g * p.s_head +
-                                         (int64_t)(p.Nv + p.Nt - p.W) * p.s_token;
+                const int g = grp % p.Hkv, lb = grp / p.Hkv;
                 const uint16_t *q_lb = p.qw + (int64_t)lb * p.W * p.Hq * D;
                 named_bar(2, kEliteThreads);   // the previous group's keys and masks have been used
-                for (int idx = et; idx < (p.W + p.G) * (D / 8); idx += kEliteThreads) {
-                    const int row = idx / (D / 8), c = idx % (D / 8);
-                    const uint16_t *src = row < p.W ? k_cand + (int64_t)row * p.s_token
-                                                    : q_lb + ((int64_t)(p.W - 1) * p.Hq + g * p.G + (row - p.W)) * D;
-                    *reinterpret_cast<uint4 *>(s_k + row * C::KS + c * 8) = __ldg(reinterpret_cast<const uint4 *>(src) + c);
+                store_rows(et, ahead);
+                if (u == 0) asm volatile("bar.arrive 3, %0;" ::"n"(kEliteThreads + 32) : "memory");
+                for (int base = et + 4 * kEliteThreads; base - et < n_vec; base += 4 * kEliteThreads) {
+                    load_rows(grp, base, ahead);
+                    store_rows(base, ahead);
+                }
+                {   // the next group of this block, if there is one
+                    const int next = gi + 1 < plan.groups_per_item ? grp + 1 : first_grp + (item + n_clusters) * plan.groups_per_item;
+                    if (gi + 1 < plan.groups_per_item || item + n_clusters < plan.items) load_rows(next, et, ahead);
                 }
                 named_bar(2, kEliteThreads);
-                // Eq. 4, last row only: logit of candidate w for head hl, fp64 dot product in element order
-                for (int idx = et; idx < p.G * p.W; idx += kEliteThreads) {
-                    const int hl = idx / p.W, w = idx - hl * p.W;
-                    const uint4 *q = reinterpret_cast<const uint4 *>(s_k + (p.W + hl) * C::KS);
-                    const uint4 *kk = reinterpret_cast<const uint4 *>(s_k + w * C::KS);
-                    double acc = 0.0;
-#pragma unroll 4
-                    for (int c = 0; c < D / 8; ++c) {
-                        const uint4 a = q[c], bb = kk[c];
-                        const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            // a product of two bf16 values is exact in fp64, so the fused form rounds exactly where
-                            // the separate multiply and add do
-                            acc = __fma_rn((double)bf16lo(av[e]), (double)bf16lo(bv[e]), acc);
-                            acc = __fma_rn((double)bf16hi(av[e]), (double)bf16hi(bv[e]), acc);
+                // Eq. 5: candidates within a factor alpha of the best one (log domain, fp32)
+                if (p.W <= 32 && !p.keep_all) {
+                    // a half-warp (or a warp) per head, a lane per candidate: no shared memory, no barrier
+                    const int seg = p.W <= 16 ? 16 : 32, per_pass = kEliteThreads / seg;
+                    const int w = lane & (seg - 1);
+                    for (int h0 = 0; h0 < p.G; h0 += per_pass) {
+                        const int hl = h0 + et / seg;
+                        const bool in = hl < p.G && w < p.W;
+                        float t = in ? logit_fp32(hl, w) : -INFINITY;
+                        float kn = in ? s_norm[w] : 0.f;
+                        float top = t;
+                        for (int sh = 1; sh < seg; sh <<= 1) {
+                            top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, sh));
+                            kn = fmaxf(kn, __shfl_xor_sync(0xffffffffu, kn, sh));
                         }
+                        float diff = __fsub_rn(t, top);
+                        const bool near = in && !(fabsf(diff - p.ln_alpha) > kSlack * p.scale * s_norm[p.W + hl] * kn);
+                        if (__any_sync(0xffffffffu, near)) {
+                            t = in ? logit_fp64(hl, w) : -INFINITY;
+                            top = t;
+                            for (int sh = 1; sh < seg; sh <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, sh));
+                            diff = __fsub_rn(t, top);
+                        }
+                        const uint32_t bits = __ballot_sync(0xffffffffu, in && diff >= p.ln_alpha);
+                        if (hl < p.G && w < 4) sm.mask[hl][w] = w > 0 ? 0u : (seg == 32 ? bits : (bits >> (lane & 16)) & 0xffffu);
                     }
-                    s_logit[idx] = __fmul_rn((float)acc, p.scale);
-                }
-                named_bar(2, kEliteThreads);
-                // Eq. 5: candidates within a factor alpha of the best one (log domain, fp32); a warp per head
-                for (int hl = ew; hl < p.G; hl += 4) {
-                    float top = -INFINITY;
-                    for (int w = lane; w < p.W; w += 32) top = fmaxf(top, s_logit[hl * p.W + w]);
-                    top = warp_max(top);
-                    for (int j = 0; j < 4; ++j) {
-                        const int w = j * 32 + lane;
-                        const bool elite = w < p.W && (p.keep_all || __fsub_rn(s_logit[hl * p.W + w], top) >= p.ln_alpha);
-                        const uint32_t bits = __ballot_sync(0xffffffffu, elite);
-                        if (lane == 0) sm.mask[hl][j] = bits;
+                } else if (p.keep_all) {
+                    for (int i = et; i < p.G * 4; i += kEliteThreads) {
+                        const int left = p.W - (i & 3) * 32;
+                        sm.mask[i >> 2][i & 3] = left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1 : 0u);
+                    }
+                } else {
+                    for (int idx = et; idx < p.G * p.W; idx += kEliteThreads) s_logit[idx] = logit_fp32(idx / p.W, idx % p.W);
+                    named_bar(2, kEliteThreads);
+                    // a warp per head; a warp that has to look closer does its head again by itself
+                    float kn = 0.f;
+                    for (int w = lane; w < p.W; w += 32) kn = fmaxf(kn, s_norm[w]);
+                    kn = warp_max(kn);
+                    for (int hl = ew; hl < p.G; hl += 4) {
+                        const float slack = kSlack * p.scale * s_norm[p.W + hl] * kn;
+                        for (bool again = true, exact = false; again; exact = true) {
+                            float top = -INFINITY;
+                            for (int w = lane; w < p.W; w += 32) top = fmaxf(top, s_logit[hl * p.W + w]);
+                            top = warp_max(top);
+                            bool near = false;
+                            for (int j = 0; j < 4; ++j) {
+                                const int w = j * 32 + lane;
+                                const float diff = w < p.W ? __fsub_rn(s_logit[hl * p.W + w], top) : -INFINITY;
+                                near = near || (w < p.W && !(fabsf(diff - p.ln_alpha) > slack));
+                                const uint32_t bits = __ballot_sync(0xffffffffu, w < p.W && diff >= p.ln_alpha);
+                                if (lane == 0) sm.mask[hl][j] = bits;
+                            }
+                            again = !exact && __any_sync(0xffffffffu, near);
+                            if (again) {
+                                for (int w = lane; w < p.W; w += 32) s_logit[hl * p.W + w] = logit_fp64(hl, w);
+                                __syncwarp();
+                            }
+                        }
                     }
                 }
                 named_bar(2, kEliteThreads);
@@ -279,7 +415,11 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                 const float head_coef = lane < p.G && count > 0 ? 1.0f / ((float)count * (float)(p.per_head ? p.G : p.Hq)) : 0.f;
                 // 8 threads per row of the unit
                 const int rr = et >> 3, sub = et & 7, quad = lane >> 3;
-                for (int row0 = 0; ok && (row0 == 0 || row0 < n_rows); row0 += kRows, ++u) {
+                if (preload && u == 0) {
+                    ok = mbar_wait(smem_u32(&sm.q_all), 0, abort_flag, p.status, 30);
+                    __syncwarp();
+                }
+                for (int row0 = 0; row0 == 0 || (ok && row0 < n_rows); row0 += kRows, ++u) {
                     int hl = 0;
 #pragma unroll
                     for (int q4 = 0; q4 < 4; ++q4) {
@@ -304,8 +444,14 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         for (; kth > 0; --kth) m &= m - 1;
                         w = j * 32 + __ffs(m) - 1;
                         const uint4 *src = reinterpret_cast<const uint4 *>(q_lb + ((int64_t)w * p.Hq + g * p.G + hl) * D);
+                        if (preload && u == 0) {
+                            const uint4 *kept = reinterpret_cast<const uint4 *>(s_ring + (S - 1) * C::TILE_BYTES) + (w * p.G + hl) * (D / 8);
 #pragma unroll
-                        for (int i = 0; i < D / 64; ++i) qv[i] = __ldg(src + i * 8 + sub);
+                            for (int i = 0; i < D / 64; ++i) qv[i] = kept[i * 8 + sub];
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < D / 64; ++i) qv[i] = __ldg(src + i * 8 + sub);
+                        }
                     }
                     // Eq. 6-7, text columns: row w sees the elite text keys w' <= w
                     float mm = kNegBig, zz = 0.f;
@@ -337,7 +483,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     __syncwarp();
                     // the query block is free when the previous unit's MMAs have completed, the small tables when
                     // the unit before that has been read
-                    ok = (u < 1 || mbar_wait(smem_u32(&sm.q_free), (u - 1) & 1, abort_flag, p.status, 25)) &&
+                    ok = ok && (u < 1 || mbar_wait(smem_u32(&sm.q_free), (u - 1) & 1, abort_flag, p.status, 25)) &&
                          (u < 2 || mbar_wait(smem_u32(&sm.meta_empty[u & 1]), ((u >> 1) & 1) ^ 1, abort_flag, p.status, 26));
                     if (ok) {
 #pragma unroll
@@ -351,7 +497,10 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // read by the tensor core
                     }
                     ok = named_bar_and(2, kEliteThreads, ok);
-                    if (et == 0 && ok) mbar_arrive(smem_u32(&sm.q_full[u & 1]));
+                    if (et == 0 && ok) {
+                        mbar_arrive(smem_u32(&sm.q_full[u & 1]));
+                        if (u == 0) mbar_arrive(smem_u32(&sm.q_taken));
+                    }
                 }
             }
         }
@@ -482,11 +631,13 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     if (leave) break;
                     if ((et >> 4) < plan.cluster) {
                         const int r = et & 15, peer = et >> 4;
-                        float2 a = sm.warp_stats[par][0][r];
+                        float2 a = make_float2(kNegBig, 0.f);
 #pragma unroll
-                        for (int w2 = 1; w2 < 4; ++w2) {
+                        for (int w2 = 0; w2 < 4; ++w2) a.x = fmaxf(a.x, sm.warp_stats[par][w2][r].x);
+#pragma unroll
+                        for (int w2 = 0; w2 < 4; ++w2) {
                             const float2 o = sm.warp_stats[par][w2][r];
-                            merge_stats(a.x, a.y, o.x, o.y);
+                            a.y = fmaf(o.y, fast_exp2(o.x - a.x), a.y);
                         }
                         st_async_f32x2(peer_smem(smem_u32(&sm.stats[par][rank][r]), peer), a.x, a.y,
                                        peer_smem(smem_u32(&sm.exchange[par]), peer));
@@ -494,12 +645,17 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     ok = mbar_wait_cluster(smem_u32(&sm.exchange[par]), (u >> 1) & 1, abort_flag, p.status, 29);
                     __syncwarp();
                     if (lane < kRows) {
-                        float2 a = sm.text[par][lane];
+                        // the largest first, so that the blocks' exponentials do not wait for one another
+                        const float2 tx = sm.text[par][lane];
+                        float mx = tx.x;
+                        for (int c = 0; c < plan.cluster; ++c) mx = fmaxf(mx, sm.stats[par][c][lane].x);
+                        float sum = tx.y * fast_exp2(tx.x - mx);
+#pragma unroll 4
                         for (int c = 0; c < plan.cluster; ++c) {
                             const float2 o = sm.stats[par][c][lane];
-                            merge_stats(a.x, a.y, o.x, o.y);
+                            sum = fmaf(o.y, fast_exp2(o.x - mx), sum);
                         }
-                        sm.fin[ew][lane] = make_float2(a.x, sm.coef[par][lane] / a.y);
+                        sm.fin[ew][lane] = make_float2(mx, sm.coef[par][lane] / sum);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&sm.meta_empty[par]));
@@ -515,7 +671,6 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         float x[kRows];
                         tmem_ld16_issue(base + t * kRows, x);
                         const int key = key0 + t * 128 + own;
-                        const float old = add && key < p.Nv ? out[key] : 0.f;
                         tmem_ld_wait(x);
                         float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -525,7 +680,13 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                                 for (int j = 0; j < 4; ++j) acc[j] = fmaf(x[4 * q + j], m[4 * q + j], acc[j]);
                             }
                         }
-                        if (key < p.Nv) out[key] = old + ((acc[0] + acc[1]) + (acc[2] + acc[3]));
+                        if (key < p.Nv) {
+                            // (added where it lies: one thread owns the key, so the order of the sum is the program's,
+                            // and nobody waits for the old value)
+                            const float v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                            if (add) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(out + key), "f"(v) : "memory");
+                            else out[key] = v;
+                        }
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -597,19 +758,26 @@ int launch_score_cluster_d(ScoreParams &p, const aircache_shape_t *s, const airc
     CUtensorMap tm;
     if (make_key_map(&tm, p, s, f) != AIRCACHE_OK) return AIRCACHE_OK;
 
+    // Cluster size and groups per item by estimated time (ns).  Measured on a B200: HBM delivers a tile of 128 keys by
+    // 128 channels in 5.3 ns over all SMs; a unit takes a block 0.6 us per tile plus the exchange (4 us where the tensor
+    // memory holds one unit only, else hidden), and never less than the elite rows of the next group, 9 us.  A sum over
+    // groups in a kernel of its own adds 2.5 us and 3 % of the traffic.
     int best = -1, best_gpi = 1;
-    int64_t best_cost = 0;
+    double best_cost = 0;
     for (int i = 0; i < 4; ++i) {
         const int c = 1 << i;
         const int per = (tiles + c - 1) / c;
         if (c > tiles || per > kSlots || at_once[i] < 1) continue;
-        for (int gpi = p.Hkv; ; gpi = 1) {
-            if (!(p.per_head && gpi > 1)) {
-                const int64_t items = (int64_t)p.n_lb * p.Hkv / gpi;
-                const int64_t rounds = (items + at_once[i] - 1) / at_once[i];
-                const int64_t cost = rounds * gpi * (10 * per + 20) + (gpi < p.Hkv && !p.per_head ? 20 : 0);
-                if (best < 0 || cost < best_cost) { best = i; best_gpi = gpi; best_cost = cost; }
-            }
+        for (int gpi = p.per_head ? 1 : p.Hkv; ; gpi = 1) {
+            const int64_t items = (int64_t)p.n_lb * p.Hkv / gpi;
+            const int64_t rounds = (items + at_once[i] - 1) / at_once[i];
+            const double hbm = 5.3 * D / 128 * tiles * p.n_lb * p.Hkv;
+            const double stream = 600.0 * per + (per > kSlots / 2 ? 4000.0 : 1000.0);
+            const double unit = (stream > 9000.0 ? stream : 9000.0) + 100.0 * per;
+            const double busy = unit * rounds * gpi;
+            double cost = (hbm > busy ? hbm : busy) + unit;
+            if (gpi < p.Hkv && !p.per_head) cost += 2500.0 + 0.03 * hbm;
+            if (best < 0 || cost < best_cost) { best = i; best_gpi = gpi; best_cost = cost; }
             if (gpi == 1) break;
         }
     }
@@ -623,7 +791,9 @@ int launch_score_cluster_d(ScoreParams &p, const aircache_shape_t *s, const airc
     plan.slots_per_unit = plan.bufs == 2 ? kSlots / 2 : kSlots;
     plan.stages = stages;
     plan.part = best_gpi < p.Hkv && !p.per_head;
-    const int clusters = plan.items < at_once[best] ? plan.items : at_once[best];
+    // as many rounds as the clusters at once need, and no more clusters than fill them evenly
+    const int rounds = (plan.items + at_once[best] - 1) / at_once[best];
+    const int clusters = (plan.items + rounds - 1) / rounds;
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * plan.cluster));

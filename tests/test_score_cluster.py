@@ -4,6 +4,7 @@ of a row has to move.  Against the CPU oracle, element by element, within the su
 log2 domain, summed in fp32 over 128 exact products, is off by some 1e-4 at most)."""
 import numpy as np
 import pytest
+import torch
 
 from harness import GpuPath, gen_inputs, logical, oracle_dims, rel_elem_err, u16
 from workloads import Workload
@@ -34,3 +35,24 @@ def test_scores_at_the_edges(oracle_mod, n_visual, d, window, alpha, sharp, per_
         err = rel_elem_err(gp.scores.cpu().numpy(), ref["scores"])
         assert err <= 2e-3, err
 
+
+
+@pytest.mark.parametrize("window", [4, 16, 31, 33, 64])
+def test_ties_at_the_threshold(oracle_mod, window):
+    """Candidates whose logits are equal in exact arithmetic (the query's channels are all alike and the keys are
+    permutations of one another) and alpha = 1: all are elite, however an fp32 sum of their products would come out."""
+    wl = Workload("ties", 1, 14, 2, 128, batch=2, n_visual=300, n_text=70, ratio=0.1, steps=1, window=window, alpha=1.0)
+    k, v, qw = gen_inputs(wl, "cpu")
+    gen = torch.Generator().manual_seed(1)
+    row = k[0, 0, 0, 0].clone()
+    for w in range(window):
+        k[:, :, -1 - w] = row[torch.randperm(128, generator=gen)]
+    qw[:, :, -1] = 0.37
+    ref = oracle_mod.score(oracle_dims(oracle_mod, wl), u16(logical(k)), u16(qw), 0.1, 1.0)
+    assert (ref["elite_mask"] == (1 << window) - 1).all()
+    gp = GpuPath(wl, device=DEV)
+    gp.sh.scale = 0.1
+    gp.set_full(logical(k.to(DEV)), logical(v.to(DEV)))
+    gp.score(qw.to(DEV), alpha=1.0)
+    assert gp.status() == 0
+    assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
