@@ -9,7 +9,7 @@ import sys
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libaircache.so")
-SOURCES = ["api.cu", "score.cu", "score_cluster.cu", "budget.cu", "compact.cu", "decode.cu"]
+SOURCES = ["api.cu", "score.cu", "score_cluster.cu", "score_dense.cu", "budget.cu", "compact.cu", "decode.cu"]
 HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "ptx.cuh"), os.path.join(CSRC, "score.cuh"), os.path.join(os.path.dirname(PKG), "include", "aircache.h")]
 
 

@@ -3,6 +3,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <atomic>
 #include <vector>
 
 #include "common.cuh"
@@ -13,6 +14,15 @@ namespace aircache {
 static thread_local int g_last_cuda_error = 0;
 
 void set_last_cuda_error(cudaError_t e) { g_last_cuda_error = (int)e; }
+
+int current_device(int *dev, int *sms) {
+    static std::atomic<int> known[kMaxDevices];
+    AIRCACHE_CUDA_TRY(cudaGetDevice(dev));
+    if (*dev >= 0 && *dev < kMaxDevices && (*sms = known[*dev].load(std::memory_order_relaxed)) > 0) return AIRCACHE_OK;
+    AIRCACHE_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev));
+    if (*dev >= 0 && *dev < kMaxDevices) known[*dev].store(*sms, std::memory_order_relaxed);
+    return AIRCACHE_OK;
+}
 
 int check_shape(const aircache_shape_t *s) {
     if (!s) return AIRCACHE_ERR_INVALID_ARG;

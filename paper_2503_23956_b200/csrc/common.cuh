@@ -55,6 +55,8 @@ void set_last_cuda_error(cudaError_t e);
 // ---------------------------------------------------------------------------------------------
 // shape helpers and the workspace carve-up (host arithmetic)
 // ---------------------------------------------------------------------------------------------
+// The current device and its number of SMs, asked once per device (the answer never changes).
+int current_device(int *dev, int *sms);
 int check_shape(const aircache_shape_t *s);
 int check_full(const aircache_shape_t *s, const aircache_full_t *f);
 int64_t kept_per_sequence(const aircache_shape_t *s, double ratio);

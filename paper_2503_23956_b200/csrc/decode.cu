@@ -1152,16 +1152,6 @@ int make_map(CUtensorMap *tm, const void *base, int D, int Hkv, int64_t rows, in
     return AIRCACHE_OK;
 }
 
-// The current device and its number of SMs, asked once per device (the answer never changes).
-int current_device(int *dev, int *sms) {
-    static std::atomic<int> known[kMaxDevices];
-    AIRCACHE_CUDA_TRY(cudaGetDevice(dev));
-    if (*dev >= 0 && *dev < kMaxDevices && (*sms = known[*dev].load(std::memory_order_relaxed)) > 0) return AIRCACHE_OK;
-    AIRCACHE_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev));
-    if (*dev >= 0 && *dev < kMaxDevices) known[*dev].store(*sms, std::memory_order_relaxed);
-    return AIRCACHE_OK;
-}
-
 template <int D, int HKV, bool G_HI, bool HS>
 int launch_decode_t(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, cudaStream_t st) {
     using C = DecodeCfg<D, HKV, G_HI, HS>;

@@ -18,7 +18,6 @@
 //                      into one (max, weight / normaliser) pair per row.  Pass two recomputes the same
 //                      tiles, turns logits into probabilities and sums the rows of all heads per key with
 //                      weight 1 / (|E_h| Hq), KV heads in ascending order by one thread per key.
-//   dense_*_kernel     alpha = 0 (every window query elite): both passes on tcgen05, see there.
 //
 // The mma.sync kernels read the keys straight from global memory into MMA fragments: every key byte is used
 // once per CTA, so staging it in shared memory would only add a round trip.
@@ -745,414 +744,6 @@ int launch_onepass(const ScoreParams &p, cudaStream_t st) {
     return p.per_head ? AIRCACHE_OK : launch_group_sum(p, st);
 }
 
-// ---------------------------------------------------------------------------------------------
-// Dense window (alpha = 0: every one of the G*W window queries is an elite row, Eq. 7 is a dense
-// [G*W x N_v] contraction per KV head).  Same two passes on the 5th-generation tensor cores:
-//   * key tiles of 128 tokens come in by TMA (5-D tensor map over the caller's strided cache, 128-byte
-//     swizzle), query blocks of 128 rows are written into the same K-major swizzled layout by the threads;
-//   * one thread issues tcgen05.mma (M = 128, N = 128, K = 16 per instruction), the accumulator lives in
-//     tensor memory and is read back with tcgen05.ld, one accumulator row per thread;
-//   * pass one puts the query rows on M, so a thread owns one softmax row and keeps its running (max, sum)
-//     in two registers; pass two swaps the operands (the same two shared-memory tiles), so a thread owns one
-//     key and sums the weighted probabilities of all rows - neither pass needs a cross-lane reduction.
-// Every mbarrier wait is bounded (status word + CTA-wide abort flag, as in the decode kernel).
-// ---------------------------------------------------------------------------------------------
-template <int D>
-struct DenseCfg {
-    static constexpr int KSUB = D / 64;             // 64-channel sub-tiles: rows of 128 bytes
-    static constexpr int SUB_BYTES = 128 * 128;     // 128 rows
-    static constexpr int TILE_BYTES = KSUB * SUB_BYTES;
-    static constexpr int NST = 2;                   // key tiles in flight (two CTAs share an SM)
-    static constexpr int SMEM_STATS = 1024 + (NST + 1) * TILE_BYTES + 256;
-    static constexpr int SMEM_IMP = 1024 + (NST + 1) * TILE_BYTES + 128 * 8 + 256;
-};
-
-// 128 query rows (row0 .. row0+127 of the group's table, zero beyond) into the swizzled K-major layout.
-// 128 threads: thread t copies 16-byte chunk t % (D/8) of rows t / (D/8) + k * (1024 / D); all table entries are
-// fetched first, then all query chunks, so the copy costs two memory round trips.
-template <int D>
-__device__ __forceinline__ void stage_queries_sw128(uint8_t *s_q, const ScoreParams &p, int grp, int lb, int g,
-                                                    int row0, int n_rows) {
-    constexpr int SUB = DenseCfg<D>::SUB_BYTES;
-    constexpr int CPR = D / 8;            // 16-byte chunks per row
-    constexpr int RPI = 128 / CPR;        // rows covered by the CTA per step
-    constexpr int STEPS = 128 / RPI;
-    const int32_t *info = p.row_info + (int64_t)grp * p.cap;
-    const uint16_t *q_lb = p.qw + (int64_t)lb * p.W * p.Hq * D;
-    const int c16 = threadIdx.x % CPR, r0 = threadIdx.x / CPR;
-    int in[STEPS];
-#pragma unroll
-    for (int k = 0; k < STEPS; ++k) {
-        const int r = row0 + r0 + k * RPI;
-        in[k] = r < n_rows ? __ldg(info + r) : -1;
-    }
-    uint4 v[STEPS];
-#pragma unroll
-    for (int k = 0; k < STEPS; ++k) {
-        v[k] = make_uint4(0, 0, 0, 0);
-        if (in[k] >= 0) {
-            const int hl = in[k] >> 8, w = in[k] & 255;
-            v[k] = __ldg(reinterpret_cast<const uint4 *>(q_lb + ((int64_t)w * p.Hq + g * p.G + hl) * D) + c16);
-        }
-    }
-    const int sub = c16 >> 3, cc = c16 & 7;
-#pragma unroll
-    for (int k = 0; k < STEPS; ++k) {
-        const int r = r0 + k * RPI;
-        *reinterpret_cast<uint4 *>(s_q + sub * SUB + r * 128 + ((cc ^ (r & 7)) << 4)) = v[k];
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes, read by the tensor core
-}
-
-// acc[128 x 128] = A[128 x D] * B[128 x D]^T, both tiles K-major swizzled at a_base / b_base.
-template <int D>
-__device__ __forceinline__ void issue_tile_mma(uint32_t tmem_d, uint32_t a_base, uint32_t b_base) {
-    constexpr int SUB = DenseCfg<D>::SUB_BYTES;
-    const uint32_t idesc = umma_idesc_bf16(128, 128);
-#pragma unroll
-    for (int kk = 0; kk < D / 16; ++kk) {
-        const uint32_t off = (kk >> 2) * SUB + (kk & 3) * 32;
-        umma_bf16(tmem_d, umma_desc_sw128(a_base + off), umma_desc_sw128(b_base + off), idesc, kk > 0 ? 1u : 0u);
-    }
-}
-
-// Both dense kernels are warp-specialised: two sets of four epilogue warps (warps 0-3 and 4-7; a thread owns one
-// accumulator row, a tensor-memory lane) run the exponent arithmetic, one thread of warp 8 drives the copies
-// and the tensor core.  Key tiles cycle through NST shared-memory stages (full: TMA landed; empty: the MMAs
-// that read the stage have completed, by tcgen05.commit), accumulators through two halves of 256 tensor-memory
-// columns (acc_full by tcgen05.commit, acc_empty by one arrival per warp of the set that read it).  Each set
-// takes the tiles of one accumulator, so two tiles' logits are read back and exponentiated at a time while the
-// MMAs of the next run.  Parities follow from running tile counts.  Every wait is bounded.
-constexpr int kDenseThreads = 288;
-constexpr int kDenseDriverWarp = 8;
-
-template <int D>
-struct DensePipe {
-    using C = DenseCfg<D>;
-    uint32_t full[C::NST], empty[C::NST], acc_full[2], acc_empty[2];   // shared-memory addresses of the mbarriers
-    __device__ void init(uint64_t *s_bar) {
-        for (int i = 0; i < C::NST; ++i) { full[i] = smem_u32(&s_bar[i]); empty[i] = smem_u32(&s_bar[C::NST + i]); }
-        for (int a = 0; a < 2; ++a) { acc_full[a] = smem_u32(&s_bar[2 * C::NST + a]); acc_empty[a] = smem_u32(&s_bar[2 * C::NST + 2 + a]); }
-    }
-    __device__ void init_barriers() const {
-        for (int i = 0; i < C::NST; ++i) { mbar_init(full[i], 1); mbar_init(empty[i], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(acc_full[a], 1); mbar_init(acc_empty[a], 4); }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-};
-
-// The driver thread's part for n_tiles key tiles starting at key0: `base` tiles went through the pipe before.
-// a_is_query: the query block is the MMA's A operand (rows on M, pass one), else the key tile is (keys on M).
-// The first key tiles of a block of work, issued by the driver thread while the other warps stage the query
-// block: returns how many loads are under way (the stages are free: the previous block's MMAs have completed).
-template <int D>
-__device__ __forceinline__ int dense_first_loads(const DensePipe<D> &pp, const CUtensorMap *tm, const ScoreParams &p,
-                                                 uint8_t *s_k, uint32_t base, int n_tiles, int key0, int g, int b, int l,
-                                                 volatile int *s_abort, uint32_t code) {
-    using C = DenseCfg<D>;
-    int loaded = 0;
-    while (loaded < n_tiles && loaded < C::NST) {
-        const uint32_t il = base + loaded, ls = il % C::NST;
-        if (!mbar_wait(pp.empty[ls], ((il / C::NST) & 1) ^ 1, s_abort, p.status, code)) break;
-        load_key_tile<D>(smem_u32(s_k + ls * C::TILE_BYTES), tm, p, key0 + loaded * 128, g, b, l, pp.full[ls]);
-        ++loaded;
-    }
-    return loaded;
-}
-
-template <int D, bool A_IS_QUERY>
-__device__ __forceinline__ bool dense_drive(const DensePipe<D> &pp, const CUtensorMap *tm, const ScoreParams &p,
-                                            uint32_t tmem, uint8_t *s_k, uint8_t *s_q, uint32_t base, int n_tiles,
-                                            int loaded, int key0, int g, int b, int l, volatile int *s_abort,
-                                            uint32_t code) {
-    using C = DenseCfg<D>;
-    bool ok = true;
-    for (int t = 0; t < n_tiles && ok; ++t) {
-        while (ok && loaded < n_tiles && loaded < t + C::NST) {
-            const uint32_t il = base + loaded, ls = il % C::NST;
-            ok = mbar_wait(pp.empty[ls], ((il / C::NST) & 1) ^ 1, s_abort, p.status, code);
-            if (ok) {
-                load_key_tile<D>(smem_u32(s_k + ls * C::TILE_BYTES), tm, p, key0 + loaded * 128, g, b, l, pp.full[ls]);
-                ++loaded;
-            }
-        }
-        if (!ok) break;
-        const uint32_t it = base + t, st = it % C::NST, a = it & 1;
-        ok = mbar_wait(pp.full[st], (it / C::NST) & 1, s_abort, p.status, code) &&
-             mbar_wait(pp.acc_empty[a], ((it >> 1) & 1) ^ 1, s_abort, p.status, code + 1);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t k_tile = smem_u32(s_k + st * C::TILE_BYTES), q_blk = smem_u32(s_q);
-        issue_tile_mma<D>(tmem + a * 128, A_IS_QUERY ? q_blk : k_tile, A_IS_QUERY ? k_tile : q_blk);
-        umma_commit(pp.empty[st]);      // the stage may be refilled
-        umma_commit(pp.acc_full[a]);    // the accumulator may be read
-    }
-    return ok;
-}
-
-// Pass one, dense.  grid = (chunks, L*B*Hkv), 160 threads.
-template <int D>
-__global__ void __launch_bounds__(kDenseThreads, 2) dense_stats_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p) {
-    using C = DenseCfg<D>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t *s_k = smem;                             // NST key tiles
-    uint8_t *s_q = smem + C::NST * C::TILE_BYTES;    // one query block
-    uint64_t *s_bar = reinterpret_cast<uint64_t *>(smem + (C::NST + 1) * C::TILE_BYTES);
-    __shared__ uint32_t s_tmem;
-    __shared__ int s_abort, s_is_last;
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int set = warp >> 2, row = (warp & 3) * 32 + lane;   // epilogue set and accumulator row (warps 0-7)
-    __shared__ float2 s_mz[128];                               // the second set's (max, sum) of every row
-    const int grp = p.lb0 * p.Hkv + blockIdx.y;
-    const int g = grp % p.Hkv, lb = grp / p.Hkv;
-    const int l = lb / p.B, b = lb % p.B;
-    const int chunk = blockIdx.x;
-    const int key0 = chunk * p.chunk_keys, key1 = min(p.Nv, key0 + p.chunk_keys);
-    const int n_tiles = key1 > key0 ? (key1 - key0 + 127) / 128 : 0;
-    const int n_rows = p.row_count[grp];
-    float2 *out = p.chunk_stats + ((int64_t)(grp - p.lb0 * p.Hkv) * p.chunks + chunk) * p.cap;
-
-    DensePipe<D> pp;
-    pp.init(s_bar);
-    if (tid == 0) {
-        pp.init_barriers();
-        s_abort = 0;
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_k)) : "memory");
-    }
-    if (warp == kDenseDriverWarp) tmem_alloc(smem_u32(&s_tmem), 256);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = s_tmem;
-    uint32_t base = 0;   // tiles that went through the pipe in earlier row blocks
-
-    for (int row0 = 0; row0 < n_rows; row0 += 128) {
-        __syncthreads();   // the previous block's MMAs have completed (their logits were read): the query block is free
-        if (s_abort) break;
-        int loaded = 0;
-        if (tid < 128) stage_queries_sw128<D>(s_q, p, grp, lb, g, row0, n_rows);
-        else if (tid == kDenseDriverWarp * 32) loaded = dense_first_loads<D>(pp, &tm_k, p, s_k, base, n_tiles, key0, g, b, l, &s_abort, 4);
-        __syncthreads();
-        float m_mine = kNegBig, z_mine = 0.f;
-        bool ok_mine = true;
-        if (warp == kDenseDriverWarp) {
-            if (lane == 0)
-                dense_drive<D, true>(pp, &tm_k, p, tmem, s_k, s_q, base, n_tiles, loaded, key0, g, b, l, &s_abort, 4);
-        } else {
-            float m = kNegBig, z = 0.f;
-            bool ok = true;
-            // one chunk of 32 logits of the thread's row: running (max, sum of exp2)
-            auto chunk32 = [&](const uint32_t (&r)[32], int kbase) {
-                float mn, sum = 0.f;
-                if (kbase + 32 <= key1) {
-                    // all 32 keys are real: the scale is positive, so the largest raw logit gives the largest
-                    // scaled one, and the exponent's argument is one fused multiply-add.  Four interleaved
-                    // partial maxima and sums keep the dependent chains short (two warps share a scheduler).
-                    float mx[4], sm[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) mx[j] = __uint_as_float(r[j]);
-#pragma unroll
-                    for (int j = 4; j < 32; ++j) mx[j & 3] = fmaxf(mx[j & 3], __uint_as_float(r[j]));
-                    mn = fmaxf(m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * p.sl2);
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) sm[j & 3] += fast_exp2(fmaf(__uint_as_float(r[j]), p.sl2, -mn));
-                    sum = (sm[0] + sm[1]) + (sm[2] + sm[3]);
-                } else {
-                    float mx = kNegBig;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (kbase + j < key1) mx = fmaxf(mx, __uint_as_float(r[j]) * p.sl2);
-                    mn = fmaxf(m, mx);
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        sum += kbase + j < key1 ? fast_exp2(fmaf(__uint_as_float(r[j]), p.sl2, -mn)) : 0.f;
-                }
-                z = z * fast_exp2(m - mn) + sum;
-                m = mn;
-            };
-            // this set's tiles: those whose accumulator (running tile count, low bit) is the set's
-            for (int t = (set - (int)base) & 1; t < n_tiles; t += 2) {
-                const uint32_t it = base + t, a = it & 1;
-                ok = mbar_wait(pp.acc_full[a], (it >> 1) & 1, &s_abort, p.status, 6);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + a * 128;
-                const int kbase = key0 + t * 128;
-                uint32_t r0[32], r1[32];
-                tmem_ld32_issue(taddr, r0);
-                tmem_ld_wait(r0);
-                tmem_ld32_issue(taddr + 32, r1);
-                chunk32(r0, kbase);
-                tmem_ld_wait(r1);
-                tmem_ld32_issue(taddr + 64, r0);
-                chunk32(r1, kbase + 32);
-                tmem_ld_wait(r0);
-                tmem_ld32_issue(taddr + 96, r1);
-                chunk32(r0, kbase + 64);
-                tmem_ld_wait(r1);
-                // the whole accumulator is in registers: hand it back before the last chunk's arithmetic
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(pp.acc_empty[a]);
-                chunk32(r1, kbase + 96);
-            }
-            if (set == 1) s_mz[row] = make_float2(m, z);
-            m_mine = m; z_mine = z; ok_mine = ok;
-        }
-        __syncthreads();   // the second set's half of every row's statistics is in shared memory
-        if (warp < 4 && ok_mine) {
-            merge_stats(m_mine, z_mine, s_mz[row].x, s_mz[row].y);
-            if (row0 + row < n_rows) __stcg(out + row0 + row, make_float2(m_mine, z_mine));
-        }
-        base += n_tiles;
-    }
-    __syncthreads();
-    const bool ok = !s_abort;
-    if (warp == kDenseDriverWarp) {
-        tc_fence_after();
-        tmem_dealloc(tmem, 256);
-    }
-    if (!ok) return;
-
-    // last CTA of the group: merge text and chunk statistics (same scheme as stats_kernel)
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        s_is_last = atomicAdd(p.group_ticket + grp, 1u) == (unsigned)p.chunks - 1;
-        if (s_is_last) __threadfence();
-    }
-    __syncthreads();
-    if (!s_is_last || warp >= 4) return;   // four warps merge
-    for (int r = warp; r < n_rows; r += 4) {
-        float mm = kNegBig, zz = 0.f;
-        if (lane == 0) {
-            const float2 tx = p.row_text[(int64_t)grp * p.cap + r];
-            mm = tx.x; zz = tx.y;
-        }
-        for (int c = lane; c < p.chunks; c += 32) {
-            const float2 cs = __ldcg(p.chunk_stats + ((int64_t)(grp - p.lb0 * p.Hkv) * p.chunks + c) * p.cap + r);
-            merge_stats(mm, zz, cs.x, cs.y);
-        }
-#pragma unroll
-        for (int sh = 1; sh < 32; sh <<= 1) {
-            const float m2 = __shfl_xor_sync(0xffffffffu, mm, sh);
-            const float z2 = __shfl_xor_sync(0xffffffffu, zz, sh);
-            merge_stats(mm, zz, m2, z2);
-        }
-        if (lane == 0) p.row_final[(int64_t)grp * p.cap + r] = make_float2(mm, p.row_coef[(int64_t)grp * p.cap + r] / zz);
-    }
-}
-
-// Pass two, dense.  grid = (chunks, L*B*Hkv) like pass one, 160 threads; an epilogue thread owns one key per tile
-// and adds the weighted probabilities of the group's rows.  The group's sums go to its row of the per-group
-// buffer (group_sum_kernel adds the groups), or straight to the scores in per-KV-head mode.
-template <int D>
-__global__ void __launch_bounds__(kDenseThreads, 2) dense_importance_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p) {
-    using C = DenseCfg<D>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t *s_k = smem;                             // NST key tiles
-    uint8_t *s_q = smem + C::NST * C::TILE_BYTES;    // one query block
-    float2 *s_stat = reinterpret_cast<float2 *>(smem + (C::NST + 1) * C::TILE_BYTES);   // (max, weight / normaliser)
-    uint64_t *s_bar = reinterpret_cast<uint64_t *>(smem + (C::NST + 1) * C::TILE_BYTES + 128 * 8);
-    __shared__ uint32_t s_tmem;
-    __shared__ int s_abort;
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int set = warp >> 2, row = (warp & 3) * 32 + lane;   // epilogue set and accumulator row (warps 0-7)
-    const int grp = p.lb0 * p.Hkv + blockIdx.y;
-    const int g = grp % p.Hkv, lb = grp / p.Hkv;
-    const int l = lb / p.B, b = lb % p.B;
-    const int key0 = blockIdx.x * p.chunk_keys, key1 = min(p.Nv, key0 + p.chunk_keys);
-    const int n_tiles = key1 > key0 ? (key1 - key0 + 127) / 128 : 0;
-    const int n_rows = p.row_count[grp];
-    float *out = (p.per_head ? p.scores : p.imp_part) + (int64_t)grp * p.Nv;
-
-    DensePipe<D> pp;
-    pp.init(s_bar);
-    if (tid == 0) {
-        pp.init_barriers();
-        s_abort = 0;
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_k)) : "memory");
-    }
-    if (warp == kDenseDriverWarp) tmem_alloc(smem_u32(&s_tmem), 256);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = s_tmem;
-    uint32_t base = 0;
-
-    for (int row0 = 0; row0 < n_rows; row0 += 128) {
-        __syncthreads();   // the previous block's MMAs have completed: query block and statistics are free
-        if (s_abort) break;
-        int loaded = 0;
-        if (tid < 128) {
-            stage_queries_sw128<D>(s_q, p, grp, lb, g, row0, n_rows);
-            s_stat[tid] = row0 + tid < n_rows ? p.row_final[(int64_t)grp * p.cap + row0 + tid] : make_float2(0.f, 0.f);
-        } else if (tid == kDenseDriverWarp * 32) {
-            loaded = dense_first_loads<D>(pp, &tm_k, p, s_k, base, n_tiles, key0, g, b, l, &s_abort, 10);
-        }
-        __syncthreads();
-        if (warp == kDenseDriverWarp) {
-            if (lane == 0)
-                dense_drive<D, false>(pp, &tm_k, p, tmem, s_k, s_q, base, n_tiles, loaded, key0, g, b, l, &s_abort, 10);
-        } else {
-            const int nch = (min(128, n_rows - row0) + 31) >> 5;   // chunks of 32 rows with a real row in them
-            // 32 rows of the thread's key: probabilities weighted and summed
-            auto chunk32 = [&](const uint32_t (&r)[32], int c0) {
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};   // interleaved partial sums: short dependent chains
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float2 sj = s_stat[c0 + j];
-                    acc[j & 3] = fmaf(fast_exp2(fmaf(__uint_as_float(r[j]), p.sl2, -sj.x)), sj.y, acc[j & 3]);
-                }
-                return (acc[0] + acc[1]) + (acc[2] + acc[3]);
-            };
-            // this set's tiles: those whose accumulator (running tile count, low bit) is the set's
-            for (int t = (set - (int)base) & 1; t < n_tiles; t += 2) {
-                const uint32_t it = base + t, a = it & 1;
-                if (!mbar_wait(pp.acc_full[a], (it >> 1) & 1, &s_abort, p.status, 12)) break;
-                tc_fence_after();
-                const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + a * 128;
-                uint32_t r0[32], r1[32];
-                float acc = 0.f;
-                tmem_ld32_issue(taddr, r0);
-                tmem_ld_wait(r0);
-                if (nch > 1) tmem_ld32_issue(taddr + 32, r1);
-                acc += chunk32(r0, 0);
-                if (nch > 1) {
-                    tmem_ld_wait(r1);
-                    if (nch > 2) tmem_ld32_issue(taddr + 64, r0);
-                    acc += chunk32(r1, 32);
-                    if (nch > 2) {
-                        tmem_ld_wait(r0);
-                        if (nch > 3) tmem_ld32_issue(taddr + 96, r1);
-                        acc += chunk32(r0, 64);
-                        if (nch > 3) {
-                            tmem_ld_wait(r1);
-                            acc += chunk32(r1, 96);
-                        }
-                    }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(pp.acc_empty[a]);
-                // the thread's key of this tile: first row block writes, later ones add (same thread every time)
-                const int key = key0 + t * 128 + row;
-                if (key < key1) out[key] = row0 == 0 ? acc : out[key] + acc;
-            }
-        }
-        base += n_tiles;
-    }
-    __syncthreads();
-    if (warp == kDenseDriverWarp) {
-        tc_fence_after();
-        tmem_dealloc(tmem, 256);
-    }
-}
-
 template <int D, int NT>
 int launch_stats(ScoreParams p, int rows_lo, int rows_hi, cudaStream_t st) {
     p.rows_lo = rows_lo; p.rows_hi = rows_hi;
@@ -1189,19 +780,6 @@ int launch_passes_d(const ScoreParams &p, cudaStream_t st) {
         if (rc) return rc;
     }
     return nt_max <= 4 ? launch_importance<D, 4>(p, st) : launch_importance<D, 8>(p, st);
-}
-
-template <int D>
-int launch_dense(ScoreParams &p, const CUtensorMap &tm, cudaStream_t st) {
-    using C = DenseCfg<D>;
-    AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(dense_stats_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_STATS));
-    AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(dense_importance_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           C::SMEM_IMP));
-    dense_stats_kernel<D><<<dim3(p.chunks, (unsigned)((int64_t)p.n_lb * p.Hkv)), kDenseThreads, C::SMEM_STATS, st>>>(tm, p);
-    AIRCACHE_LAUNCH_CHECK();
-    dense_importance_kernel<D><<<dim3(p.chunks, (unsigned)((int64_t)p.n_lb * p.Hkv)), kDenseThreads, C::SMEM_IMP, st>>>(tm, p);
-    AIRCACHE_LAUNCH_CHECK();
-    return p.per_head ? AIRCACHE_OK : launch_group_sum(p, st);
 }
 
 }  // namespace
@@ -1269,11 +847,10 @@ int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void
     p.pos_token = p.pos_head = p.pos_batch = p.pos_layer = 0;
     p.status = ws_ptr<uint32_t>(ws, w.status);
 
-    if (!(p.keep_all && p.G * p.W >= 32)) {
-        int taken = 0;
-        const int rc = launch_score_cluster(p, s, f, st, &taken);
-        if (rc || taken) return rc;
-    }
+    // alpha = 0 with more than a cluster's two query blocks keeps the tensor cores and the exponentials busy by itself
+    int taken = 0;
+    const int rc = p.keep_all && p.G * p.W >= 32 ? launch_score_dense(p, s, f, st, &taken) : launch_score_cluster(p, s, f, st, &taken);
+    if (rc || taken) return rc;
     const int64_t groups = (int64_t)p.n_lb * p.Hkv;
     const size_t elite_smem = (size_t)(p.W + p.G) * (p.d + 8) * 2;
     if (p.keep_all) {
@@ -1284,15 +861,6 @@ int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void
         else elite_kernel<128, false><<<(unsigned)groups, 128, elite_smem, st>>>(p);
     }
     AIRCACHE_LAUNCH_CHECK();
-    // alpha = 0 keeps all G*W window queries: the dense contraction goes to tcgen05 (if a tensor map over the
-    // caller's strides can be made; otherwise the mma.sync passes handle it as well)
-#ifndef AIRCACHE_NO_DENSE
-    if (p.keep_all && p.G * p.W >= 32) {
-        CUtensorMap tm;
-        if (make_key_map(&tm, p, s, f) == AIRCACHE_OK)
-            return s->head_dim == 64 ? launch_dense<64>(p, tm, st) : launch_dense<128>(p, tm, st);
-    }
-#endif
     // one pass over the keys, if a group's blocks are sure to be resident together
     const int resident = s->head_dim == 64 ? onepass_resident_blocks<64>() : onepass_resident_blocks<128>();
     if ((int64_t)p.op_chunks * 2 <= resident && (int64_t)p.n_lb * p.Hkv * p.op_chunks < ((int64_t)1 << 31))

@@ -103,6 +103,8 @@ __device__ __forceinline__ void prefetch_key_tile(const CUtensorMap *tm, const S
 
 // score_cluster.cu: the scoring kernel for sequences that a cluster of up to eight blocks holds (*taken = 1 if it ran).
 int launch_score_cluster(ScoreParams &p, const aircache_shape_t *s, const aircache_full_t *f, cudaStream_t st, int *taken);
+// score_dense.cu: the two passes for alpha = 0 (*taken = 1 if they ran).
+int launch_score_dense(ScoreParams &p, const aircache_shape_t *s, const aircache_full_t *f, cudaStream_t st, int *taken);
 // score.cu: Eq. 8 over the KV groups, behind a kernel that wrote the groups' parts.
 int launch_group_sum(const ScoreParams &p, cudaStream_t st);
 

@@ -56,3 +56,28 @@ def test_ties_at_the_threshold(oracle_mod, window):
     gp.score(qw.to(DEV), alpha=1.0)
     assert gp.status() == 0
     assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
+
+
+@pytest.mark.parametrize("n_visual,heads,d,window,sharp,per_head", [
+    (3, (8, 2), 128, 8, 1.0, 0), (127, (14, 2), 64, 5, 1.0, 1), (128, (32, 2), 128, 64, 1.0, 0),
+    (1000, (14, 2), 128, 64, 6.0, 0), (4097, (28, 4), 128, 16, 6.0, 1), (2500, (4, 4), 64, 128, 1.0, 0),
+    (20000, (16, 1), 64, 9, 1.0, 0)])
+def test_whole_window_at_the_edges(oracle_mod, n_visual, heads, d, window, sharp, per_head):
+    """alpha = 0: one tile and fewer, query blocks that fill 128 rows and that do not, several of them, references that
+    have to move, and a sequence cut into many pieces."""
+    wl = Workload("edge0", 2, heads[0], heads[1], d, batch=2, n_visual=n_visual, n_text=130, ratio=0.1, steps=1,
+                  window=window, alpha=0.0)
+    scale = sharp / d ** 0.5
+    k, v, qw = gen_inputs(wl, "cpu")
+    score = oracle_mod.score_groups if per_head else oracle_mod.score
+    ref = score(oracle_dims(oracle_mod, wl), u16(logical(k)), u16(qw), scale, 0.0)
+    gp = GpuPath(wl, device=DEV, per_kv_head=per_head)
+    gp.sh.scale = scale
+    gp.set_full(logical(k.to(DEV)), logical(v.to(DEV)))
+    for _ in range(2):
+        gp.scores.fill_(float("nan"))
+        gp.score(qw.to(DEV), alpha=0.0)
+        assert gp.status() == 0
+        assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
+        err = rel_elem_err(gp.scores.cpu().numpy(), ref["scores"])
+        assert err <= 2e-3, err
