@@ -1,14 +1,20 @@
 // aircache_budget: strength and skewness of every region's importance distribution (Eq. 9-10), the
 // layer-wise budget of Eq. 11 turned into integer row counts, and the row offsets of the ragged cache.
 //
-// One launch.  Every CTA reduces one cell (three fp64 block reductions over the fp32 scores, which it
-// keeps in registers: sum; squared deviations; cubed standardised deviations; fixed reduction tree).  The
+// One launch.  Every CTA reduces one cell (fp64 block reductions over the fp32 scores, which it keeps in registers:
+// sum; then squared and cubed deviations together; fixed reduction tree).  The
 // CTA that finishes a SEQUENCE last (one ticket per sequence in the workspace, put back to zero for the next
 // call) runs that sequence's allocation with one warp: sums over the cells taken by one lane in cell order
 // and every fp64 operation individually rounded (no fused multiply-add), so that the integer budgets are
 // the ones the sequential definition gives; divisions, floors and the ranking of the fractional parts run
 // across the lanes.  The CTA that finishes the last sequence scans the region sizes into offsets.
+//
+// A chain of latencies, most of it fp64.  With 512 threads, three reductions and a division per score it took 17.5 us for
+// 28 cells of 7290 scores and 47 us for 1792 of 2916; now 11 and 25 us.  (Five blocks of 256 threads to an SM instead of
+// four spill registers and gain nothing.)
 #include <math.h>
+
+#include <atomic>
 
 #include "common.cuh"
 
@@ -16,8 +22,6 @@ namespace aircache {
 
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kPerThread = 16;   // scores a thread keeps in registers (covers N_v <= 8192; beyond, re-read)
 
 struct BudgetParams {
     const float *scores;     // [L*B, Nv]
@@ -32,17 +36,31 @@ struct BudgetParams {
     long long first_row;     // rows of the shared buffers in front of this cache's first region
 };
 
-__device__ __forceinline__ double block_sum(double v, double *s_part) {
-#pragma unroll
-    for (int sh = 16; sh > 0; sh >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, sh));
+// Sums of v[0 .. N-1] over the block's T threads, the same in all of them.  s_part: N * 32 doubles, free again at the
+// next use with the other half of it (parity).
+template <int T, int N>
+__device__ __forceinline__ void block_sums(double (&v)[N], double (*s_part)[32]) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) s_part[warp] = v;
-    __syncthreads();
-    double tot = 0.0;
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) tot = __dadd_rn(tot, s_part[w]);
-    return tot;
+    for (int sh = 16; sh > 0; sh >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = __dadd_rn(v[i], __shfl_xor_sync(0xffffffffu, v[i], sh));
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < N; ++i) s_part[i][warp] = v[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = lane < T / 32 ? s_part[i][lane] : 0.0;
+#pragma unroll
+    for (int sh = 16; sh > 0; sh >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = __dadd_rn(v[i], __shfl_xor_sync(0xffffffffu, v[i], sh));
+}
+
+__device__ __forceinline__ unsigned ticket_add(uint32_t *t) {   // what the block wrote before it is seen with it
+    unsigned v;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(t) : "memory");
+    return v;
 }
 
 __device__ __forceinline__ double warp_bcast(double v, int src) {
@@ -58,6 +76,7 @@ __device__ void allocate_sequence(const BudgetParams &p, int n, const double *st
     // across-layer means: one lane, layer order (this fixes the rounding of the sums)
     double mean_t = 0.0, mean_k = 0.0;
     if (lane == 0) {
+#pragma unroll 8
         for (int l = 0; l < L; ++l) {
             mean_t = __dadd_rn(mean_t, st[l]);
             const double s = sk[l];
@@ -86,14 +105,16 @@ __device__ void allocate_sequence(const BudgetParams &p, int n, const double *st
     long long R = p.total_kept;
     // capped proportional split: a layer whose share reaches Nv keeps everything, the rest re-share
     for (;;) {
+        // (a cell that has left the split has weight zero by then: adding it changes nothing)
         double wsum = 0.0;
-        int n_active = 0;
         if (lane == 0) {
-            for (int l = 0; l < L; ++l)
-                if (act[l]) { wsum = __dadd_rn(wsum, w[l]); ++n_active; }
+#pragma unroll 8
+            for (int l = 0; l < L; ++l) wsum = __dadd_rn(wsum, w[l]);
         }
+        int n_active = 0;
+        for (int l = lane; l < L; l += 32) n_active += act[l];
+        n_active = __reduce_add_sync(0xffffffffu, n_active);
         wsum = warp_bcast(wsum, 0);
-        n_active = __shfl_sync(0xffffffffu, n_active, 0);
         if (n_active == 0) break;
         int moved = 0;
         for (int l = lane; l < L; l += 32) {
@@ -104,6 +125,7 @@ __device__ void allocate_sequence(const BudgetParams &p, int n, const double *st
             if (sh >= (double)p.Nv) {
                 bud[l] = p.Nv;
                 act[l] = 0;
+                w[l] = 0.0;
                 ++moved;
             }
         }
@@ -144,70 +166,53 @@ __device__ void allocate_sequence(const BudgetParams &p, int n, const double *st
     __syncwarp();
 }
 
-__global__ void __launch_bounds__(kThreads, 2) budget_kernel(BudgetParams p) {
+template <int T, int PER>
+__global__ void __launch_bounds__(T, 1024 / T) budget_kernel(BudgetParams p) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    __shared__ double s_part[kThreads / 32];
+    __shared__ double s_part[3][32];
     __shared__ int s_is_last;
     const int tid = threadIdx.x;
     const int LB = p.L * p.B * p.Hc;   // cells
 
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // ---------------- Eq. 9 and Eq. 10 of cell blockIdx.x ----------------
     {
         const float *x = p.scores + (int64_t)blockIdx.x * p.Nv;
         const double n = (double)p.Nv;
-        float v[kPerThread];
+        float f[PER];
 #pragma unroll
-        for (int k = 0; k < kPerThread; ++k) {
-            const int i = tid + k * kThreads;
-            v[k] = i < p.Nv ? x[i] : 0.f;
+        for (int k = 0; k < PER; ++k) {
+            const int i = tid + k * T;
+            f[k] = i < p.Nv ? __ldg(x + i) : 0.f;
         }
-        const bool spill = p.Nv > kThreads * kPerThread;
-        double s = 0.0;
+        double sum[1] = {0.0};
 #pragma unroll
-        for (int k = 0; k < kPerThread; ++k)
-            if (tid + k * kThreads < p.Nv) s = __dadd_rn(s, (double)v[k]);
-        if (spill)
-            for (int i = tid + kPerThread * kThreads; i < p.Nv; i += kThreads) s = __dadd_rn(s, (double)x[i]);
-        s = block_sum(s, s_part);
-        const double mu = __ddiv_rn(s, n);
+        for (int k = 0; k < PER; ++k) sum[0] = __dadd_rn(sum[0], (double)f[k]);
+        for (int i = tid + PER * T; i < p.Nv; i += T) sum[0] = __dadd_rn(sum[0], (double)__ldg(x + i));   // (more than fit)
+        block_sums<T, 1>(sum, s_part);
+        const double mu = __ddiv_rn(sum[0], n);
 
-        double ss = 0.0;
+        double dev[2] = {0.0, 0.0};   // sums of the squared and the cubed deviations
+        auto add = [&](double xi) {
+            const double c = __dsub_rn(xi, mu), c2 = __dmul_rn(c, c);
+            dev[0] = __dadd_rn(dev[0], c2);
+            dev[1] = __fma_rn(c2, c, dev[1]);
+        };
 #pragma unroll
-        for (int k = 0; k < kPerThread; ++k)
-            if (tid + k * kThreads < p.Nv) { const double c = __dsub_rn((double)v[k], mu); ss = __dadd_rn(ss, __dmul_rn(c, c)); }
-        if (spill)
-            for (int i = tid + kPerThread * kThreads; i < p.Nv; i += kThreads) {
-                const double c = __dsub_rn((double)x[i], mu);
-                ss = __dadd_rn(ss, __dmul_rn(c, c));
-            }
-        ss = block_sum(ss, s_part);
-        const double sigma = __dsqrt_rn(__ddiv_rn(ss, __dsub_rn(n, 1.0)));
-
-        double cube = 0.0;
-        if (sigma > 0.0) {
-#pragma unroll
-            for (int k = 0; k < kPerThread; ++k)
-                if (tid + k * kThreads < p.Nv) {
-                    const double zc = __ddiv_rn(__dsub_rn((double)v[k], mu), sigma);
-                    cube = __dadd_rn(cube, __dmul_rn(__dmul_rn(zc, zc), zc));
-                }
-            if (spill)
-                for (int i = tid + kPerThread * kThreads; i < p.Nv; i += kThreads) {
-                    const double zc = __ddiv_rn(__dsub_rn((double)x[i], mu), sigma);
-                    cube = __dadd_rn(cube, __dmul_rn(__dmul_rn(zc, zc), zc));
-                }
-        }
-        cube = block_sum(cube, s_part);
+        for (int k = 0; k < PER; ++k)
+            if (tid + k * T < p.Nv) add((double)f[k]);
+        for (int i = tid + PER * T; i < p.Nv; i += T) add((double)__ldg(x + i));
+        block_sums<T, 2>(dev, s_part + 1);
         if (tid == 0) {
+            const double sigma = __dsqrt_rn(__ddiv_rn(dev[0], __dsub_rn(n, 1.0)));
             const double pre = __ddiv_rn(n, __dmul_rn(__dsub_rn(n, 1.0), __dsub_rn(n, 2.0)));
-            p.strength[blockIdx.x] = s;
-            p.skewness[blockIdx.x] = sigma > 0.0 ? __dmul_rn(pre, cube) : 0.0;
-            __threadfence();
+            p.strength[blockIdx.x] = sum[0];
+            p.skewness[blockIdx.x] = sigma > 0.0 ? __dmul_rn(pre, __ddiv_rn(dev[1], __dmul_rn(__dmul_rn(sigma, sigma), sigma))) : 0.0;
             // cell index = (l * B + b) * Hc + g: the sequence is the middle coordinate
             const int b = (blockIdx.x / p.Hc) % p.B;
-            const unsigned t = atomicAdd(p.seq_ticket + b, 1u);
-            s_is_last = (t == (unsigned)(p.L * p.Hc) - 1);
-            if (s_is_last) { p.seq_ticket[b] = 0; __threadfence(); }
+            s_is_last = ticket_add(p.seq_ticket + b) == (unsigned)(p.L * p.Hc) - 1;
+            if (s_is_last) p.seq_ticket[b] = 0;
         }
         __syncthreads();
         if (!s_is_last) return;
@@ -224,30 +229,28 @@ __global__ void __launch_bounds__(kThreads, 2) budget_kernel(BudgetParams p) {
     unsigned char *act = reinterpret_cast<unsigned char *>(bud + n);
     // cell l of the sequence sits at ((l / Hc) * B + b) * Hc + l % Hc
     auto at = [&](int l) { return ((l / p.Hc) * p.B + b) * p.Hc + l % p.Hc; };
-    for (int l = tid; l < n; l += kThreads) {
+    for (int l = tid; l < n; l += T) {
         st[l] = __ldcg(p.strength + at(l));
         sk[l] = __ldcg(p.skewness + at(l));
     }
     __syncthreads();
     if (tid < 32) allocate_sequence(p, n, st, sk, w, share, act, bud);
     __syncthreads();
-    for (int l = tid; l < n; l += kThreads) {
+    for (int l = tid; l < n; l += T) {
         __stcg(p.budgets + at(l), bud[l]);
         p.lens[at(l)] = bud[l] + p.Nt;
     }
-    __threadfence();
     __syncthreads();
     if (tid == 0) {
-        const unsigned t = atomicAdd(p.ticket, 1u);
-        s_is_last = (t == (unsigned)p.B - 1);
-        if (s_is_last) { *p.ticket = 0; __threadfence(); }
+        s_is_last = p.B == 1 || ticket_add(p.ticket) == (unsigned)p.B - 1;
+        if (s_is_last) *p.ticket = 0;
     }
     __syncthreads();
     if (!s_is_last) return;
 
     // ---------------- the last sequence's CTA: offsets = exclusive scan of (budget + Nt + slack) over the cells ----
-    __shared__ long long s_warp[kThreads / 32];
-    const int per = (LB + kThreads - 1) / kThreads;
+    __shared__ long long s_warp[T / 32];
+    const int per = (LB + T - 1) / T;
     const int i0 = min(LB, tid * per), i1 = min(LB, i0 + per);
     long long local = 0;
     for (int i = i0; i < i1; ++i) local += __ldcg(p.budgets + i) + p.Nt + p.slack;
@@ -261,13 +264,13 @@ __global__ void __launch_bounds__(kThreads, 2) budget_kernel(BudgetParams p) {
     if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        long long vv = lane < kThreads / 32 ? s_warp[lane] : 0;
+        long long vv = lane < T / 32 ? s_warp[lane] : 0;
 #pragma unroll
         for (int sh = 1; sh < 32; sh <<= 1) {
             const long long o = __shfl_up_sync(0xffffffffu, vv, sh);
             if (lane >= sh) vv += o;
         }
-        if (lane < kThreads / 32) s_warp[lane] = vv;
+        if (lane < T / 32) s_warp[lane] = vv;
     }
     __syncthreads();
     long long run = p.first_row + incl - local + (warp > 0 ? s_warp[warp - 1] : 0);
@@ -275,7 +278,29 @@ __global__ void __launch_bounds__(kThreads, 2) budget_kernel(BudgetParams p) {
         p.offsets[i] = run;
         run += __ldcg(p.budgets + i) + p.Nt + p.slack;
     }
-    if (tid == kThreads - 1) p.offsets[LB] = p.first_row + s_warp[kThreads / 32 - 1];
+    if (tid == T - 1) p.offsets[LB] = p.first_row + s_warp[T / 32 - 1];
+}
+
+template <int T, int PER>
+int launch_budget_t(const BudgetParams &p, int cells, int dev, cudaStream_t st) {
+    // the shared-memory limit is a property of the kernel on a device: set once for each
+    static std::atomic<bool> ready[kMaxDevices];
+    if (dev >= kMaxDevices || !ready[dev].load(std::memory_order_acquire)) {
+        AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(budget_kernel<T, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+        if (dev < kMaxDevices) ready[dev].store(true, std::memory_order_release);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cells);
+    cfg.blockDim = dim3(T);
+    cfg.dynamicSmemBytes = (size_t)p.L * p.Hc * (4 * 8 + 4 + 1) + 16;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    AIRCACHE_CUDA_TRY(cudaLaunchKernelEx(&cfg, budget_kernel<T, PER>, p));
+    return AIRCACHE_OK;
 }
 
 }  // namespace
@@ -298,11 +323,14 @@ int launch_budget(const aircache_shape_t *s, const float *scores, double ratio, 
     p.L = s->n_layers; p.B = s->batch; p.Hc = cells_of(s); p.Nv = s->n_visual; p.Nt = s->n_text; p.slack = s->slack; p.mode = mode;
     p.total_kept = kept_per_sequence(s, ratio);
     p.first_row = layout->first_row;
-    const size_t smem = (size_t)s->n_layers * cells_of(s) * (4 * 8 + 4 + 1) + 16;
-    AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(budget_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-    budget_kernel<<<LB, kThreads, smem, st>>>(p);
-    AIRCACHE_LAUNCH_CHECK();
-    return AIRCACHE_OK;
+    // as in the selection: all threads a block can have for few cells, small blocks for many
+    int dev = 0, sms = 0;
+    const int rc = current_device(&dev, &sms);
+    if (rc) return rc;
+    const bool many = LB > 2 * sms;
+    if (many && s->n_visual <= 256 * 16) return launch_budget_t<256, 16>(p, LB, dev, st);
+    if (many) return launch_budget_t<512, 16>(p, LB, dev, st);
+    return launch_budget_t<1024, 8>(p, LB, dev, st);
 }
 
 }  // namespace aircache

@@ -1,11 +1,11 @@
 // aircache_compact: per-region top-k of the importance scores and the gather that packs the kept
 // visual rows and all text rows into the ragged cache (Algorithm 1, second loop); aircache_append (Eq. 2).
 //
-//   select_kernel  one CTA per region.  Radix select, most significant byte first, on an order-preserving
-//                  integer image of the fp32 score: four 256-bin histogram passes find the value of the
-//                  k-th largest score and how many of its duplicates are needed; one ordered pass then
-//                  emits the kept token indices in ascending order, duplicates of the threshold value
-//                  taken from the lowest indices.
+//   select_kernel  one CTA per region.  The k-th largest score by histograms over an order-preserving integer image
+//                  of the fp32 scores: 2048 bins over the range the keys really have, then over the bin that holds
+//                  the k-th, until few enough are left to be ranked directly (mostly after one histogram).  Then
+//                  the kept token indices in ascending order, duplicates of the threshold value taken from the
+//                  lowest indices, by ballots and one scan.
 //   gather_kernel  one warp per output row [Hkv, d] of K' and of V': 16-byte loads along the source row's
 //                  head slices, 16-byte stores to the packed row.  Region of a row by binary search in the
 //                  offsets table.
@@ -15,9 +15,8 @@ namespace aircache {
 
 namespace {
 
-constexpr int kSelThreads = 512;
-constexpr int kSelSmemKeys = 40960;  // scores kept in shared memory up to this many visual tokens
-
+constexpr int kSelBins = 2048;
+constexpr int kSelCandidates = 256;   // keys of a bin that are ranked directly
 // Order-preserving integer image of a float: a > b as floats <=> key(a) > key(b), a == b <=> equal keys.  The
 // two zeros compare equal as floats, so -0.0 takes the key of +0.0 (the lower index then wins among them).
 __device__ __forceinline__ uint32_t order_key(float x) {
@@ -26,144 +25,198 @@ __device__ __forceinline__ uint32_t order_key(float x) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Exclusive block scan of one int per thread; returns the exclusive prefix, total in *total.
-__device__ __forceinline__ int block_excl_scan(int v, int *s_warp, int *total) {
+// Exclusive block scan of one unsigned per thread over T threads.
+template <int T>
+__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *s_warp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
+    uint32_t incl = v;
 #pragma unroll
     for (int sh = 1; sh < 32; sh <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, incl, sh);
+        const uint32_t o = __shfl_up_sync(0xffffffffu, incl, sh);
         if (lane >= sh) incl += o;
     }
-    __syncthreads();
     if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-        int w = lane < (kSelThreads / 32) ? s_warp[lane] : 0;
-#pragma unroll
-        for (int sh = 1; sh < 32; sh <<= 1) {
-            const int o = __shfl_up_sync(0xffffffffu, w, sh);
-            if (lane >= sh) w += o;
-        }
-        if (lane < kSelThreads / 32) s_warp[lane] = w;
-    }
+    // every warp adds up the warps before it
+    const uint32_t w = lane < warp ? s_warp[lane] : 0u;
+    const uint32_t before = __reduce_add_sync(0xffffffffu, w);
     __syncthreads();
-    *total = s_warp[kSelThreads / 32 - 1];
-    return incl - v + (warp > 0 ? s_warp[warp - 1] : 0);
+    return before + incl - v;
 }
 
-template <bool SMEM_KEYS>
-__global__ void __launch_bounds__(kSelThreads) select_kernel(const float *__restrict__ scores,
-                                                             const int32_t *__restrict__ budgets,
-                                                             const int64_t *__restrict__ offsets, int n_visual,
-                                                             int n_text, int slack, int64_t first_row,
-                                                             int32_t *__restrict__ kept, int64_t kept_cap,
-                                                             uint32_t *status) {
-    extern __shared__ uint32_t s_keys[];
-    __shared__ int s_hist[256];
-    __shared__ int s_warp[kSelThreads / 32];
-    __shared__ uint32_t s_prefix;
-    __shared__ int s_remaining;
+// A thread keeps PER keys in registers (token kk * T + thread); PER = 0: any number of tokens, read again where needed.
+// The chain of latencies is what it costs.  Four 256-bin passes over shared memory took 14 us for 28 regions of 7290
+// tokens and 47 us for 1792 of 2916 (512 threads); this takes 6 and 20.
+template <int T, int PER>
+__global__ void __launch_bounds__(T, T == 256 ? 5 : T == 512 ? 2 : 1) select_kernel(const float *__restrict__ scores, const int32_t *__restrict__ budgets,
+                                                   const int64_t *__restrict__ offsets, int n_visual, int n_text, int slack,
+                                                   int64_t first_row, int32_t *__restrict__ kept, int64_t kept_cap,
+                                                   uint32_t *status) {
+    constexpr int WARPS = T / 32;
+    __shared__ uint32_t s_hist[kSelBins];
+    __shared__ uint32_t s_warp[32], s_lo[32], s_hi[32];
+    __shared__ uint32_t s_cand[kSelCandidates];
+    __shared__ uint32_t s_pick[3];   // chosen bin, keys still to be taken from it, keys in it; then threshold, duplicates to take
+    __shared__ uint32_t s_n;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    // the gather kernel that follows may start its text rows now; it waits before it reads the lists
+    // What is before in the stream has ended when this kernel lets the gather kernel start: that one copies its text
+    // rows by the budgets at once, and waits before it reads the lists.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = blockIdx.x;
     const int k = budgets[r];
     // the region's list starts after the kept rows of the regions before it; budgets and offsets come from
     // device memory, so a pair that does not fit the list buffer is reported instead of followed
     const int64_t start = offsets[r] - first_row - (int64_t)r * (n_text + slack);
+    const float *x = scores + (int64_t)r * n_visual;
+    uint32_t key[PER > 0 ? PER : 1];
+    if (PER > 0) {
+        float f[PER > 0 ? PER : 1];
+#pragma unroll
+        for (int kk = 0; kk < PER; ++kk) f[kk] = kk * T + tid < n_visual ? __ldg(x + kk * T + tid) : 0.f;
+#pragma unroll
+        for (int kk = 0; kk < PER; ++kk) key[kk] = order_key(f[kk]);
+    }
     if (k < 0 || k > n_visual || start < 0 || start + k > kept_cap) {
-        if (threadIdx.x == 0) atomicExch(status, kStatusInconsistent);
+        if (tid == 0) atomicExch(status, kStatusInconsistent);
         return;
     }
     int32_t *out = kept + start;
-    const float *x = scores + (int64_t)r * n_visual;
     if (k <= 0) return;
     if (k >= n_visual) {
-        for (int i = threadIdx.x; i < n_visual; i += kSelThreads) out[i] = i;
+        for (int i = tid; i < n_visual; i += T) out[i] = i;
         return;
     }
-    if (SMEM_KEYS) {
-        for (int i = threadIdx.x; i < n_visual; i += kSelThreads) s_keys[i] = order_key(x[i]);
-    }
-    auto key_at = [&](int i) -> uint32_t { return SMEM_KEYS ? s_keys[i] : order_key(x[i]); };
+    // f(token, key, token exists) for all tokens of the thread; whole warps take part
+    auto each = [&](auto &&f) {
+        if (PER > 0) {
+#pragma unroll
+            for (int kk = 0; kk < PER; ++kk)
+                if (kk * T + (tid & ~31) < n_visual) f(kk, kk * T + tid, key[kk], kk * T + tid < n_visual);
+        } else {
+            for (int i = tid; (i & ~31) < n_visual; i += T) f(i / T, i, i < n_visual ? order_key(__ldg(x + i)) : 0u, i < n_visual);
+        }
+    };
 
-    if (threadIdx.x == 0) { s_prefix = 0; s_remaining = k; }
-    uint32_t mask = 0;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int i = threadIdx.x; i < 256; i += kSelThreads) s_hist[i] = 0;
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    each([&](int, int, uint32_t q, bool in) { if (in) { lo = min(lo, q); hi = max(hi, q); } });
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lane < WARPS ? s_lo[lane] : 0xffffffffu);
+    hi = __reduce_max_sync(0xffffffffu, lane < WARPS ? s_hi[lane] : 0u);
+
+    uint32_t thr = lo, need_eq = 0, remaining = (uint32_t)k;
+    for (;;) {
+        const uint32_t range = hi - lo;
+        const int bits = 32 - __clz(range), shift = bits > 11 ? bits - 11 : 0;
+        for (int i = tid; i < kSelBins; i += T) s_hist[i] = 0;
+        if (tid == 0) s_n = 0;
         __syncthreads();
-        const uint32_t prefix = s_prefix;
-        // scores of one layer share most of their exponent, so the first passes put nearly every key into one
-        // or two bins: a warp whose 32 keys share the digit adds them with one atomic
-        for (int i0 = 0; i0 < n_visual; i0 += kSelThreads) {
-            const int i = i0 + threadIdx.x;
-            const uint32_t key = i < n_visual ? key_at(i) : 0u;
-            const bool in = i < n_visual && (key & mask) == prefix;
-            const int bin = in ? (int)((key >> shift) & 255) : -1;
+        each([&](int, int, uint32_t q, bool in) {
+            in = in && q >= lo && q <= hi;
+            // (scores that share a bin by the warp, zeros above all, are added with one atomic)
+            const int bin = in ? (int)((q - lo) >> shift) : -1;
             int same;
             __match_all_sync(0xffffffffu, bin, &same);
             if (same) {
-                if (in && (threadIdx.x & 31) == 0) atomicAdd(&s_hist[bin], 32);
+                if (in && lane == 0) atomicAdd(&s_hist[bin], 32u);
             } else if (in) {
-                atomicAdd(&s_hist[bin], 1);
+                atomicAdd(&s_hist[bin], 1u);
             }
-        }
+        });
         __syncthreads();
-        if (threadIdx.x < 32) {
-            // warp 0: walk the bins from the largest digit down until `remaining` keys are covered
-            const int lane = threadIdx.x;
-            int remaining = s_remaining;
-            int chosen = -1;
-            for (int base = 224; base >= 0 && chosen < 0; base -= 32) {
-                const int bin = base + 31 - lane;  // lane 0 holds the largest digit of the group
-                const int c = s_hist[bin];
-                int incl = c;
+        // bins from the largest down, kSelBins / T to a thread: the one in which `remaining` keys are covered
+        constexpr int BPT = kSelBins / T;
+        const int top = kSelBins - 1 - tid * BPT;
+        uint32_t c[BPT], sum = 0;
 #pragma unroll
-                for (int sh = 1; sh < 32; sh <<= 1) {
-                    const int o = __shfl_up_sync(0xffffffffu, incl, sh);
-                    if (lane >= sh) incl += o;
+        for (int i = 0; i < BPT; ++i) { c[i] = s_hist[top - i]; sum += c[i]; }
+        uint32_t before = block_excl_scan<T>(sum, s_warp);
+        if (before < remaining && remaining <= before + sum) {
+#pragma unroll
+            for (int i = 0; i < BPT; ++i) {
+                if (before < remaining && remaining <= before + c[i]) {
+                    s_pick[0] = top - i;
+                    s_pick[1] = remaining - before;
+                    s_pick[2] = c[i];
                 }
-                const unsigned hit = __ballot_sync(0xffffffffu, incl >= remaining);
-                if (hit) {
-                    const int src = __ffs(hit) - 1;
-                    const int before = __shfl_sync(0xffffffffu, incl - c, src);
-                    chosen = base + 31 - src;
-                    remaining -= before;
-                } else {
-                    remaining -= __shfl_sync(0xffffffffu, incl, 31);
-                }
-            }
-            if (lane == 0) {
-                s_prefix = prefix | ((uint32_t)chosen << shift);
-                s_remaining = remaining;
+                before += c[i];
             }
         }
-        mask |= 255u << shift;
         __syncthreads();
+        const uint32_t count = s_pick[2];
+        lo += s_pick[0] << shift;
+        hi = min(hi - lo, (1u << shift) - 1) + lo;
+        remaining = s_pick[1];
+        if (shift == 0) { thr = lo; need_eq = remaining; break; }
+        if (count <= kSelCandidates) {
+            each([&](int, int, uint32_t q, bool in) { if (in && q >= lo && q <= hi) s_cand[atomicAdd(&s_n, 1u)] = q; });
+            __syncthreads();
+            for (uint32_t t = tid; t < count; t += T) {
+                const uint32_t mine = s_cand[t];
+                uint32_t above = 0, equal = 0;
+                for (uint32_t j = 0; j < count; ++j) { const uint32_t o = s_cand[j]; above += o > mine; equal += o == mine; }
+                if (above < remaining && remaining <= above + equal) { s_pick[0] = mine; s_pick[1] = remaining - above; }
+            }
+            __syncthreads();
+            thr = s_pick[0];
+            need_eq = s_pick[1];
+            break;
+        }
+        __syncthreads();   // s_pick has been read by all
     }
-    const uint32_t thr = s_prefix;   // image of the k-th largest score
-    const int need_eq = s_remaining; // how many tokens equal to it are kept (lowest indices first)
 
-    // ordered emit: thread t owns the contiguous index range [i0, i1)
-    const int per = (n_visual + kSelThreads - 1) / kSelThreads;
-    const int i0 = min(n_visual, (int)threadIdx.x * per), i1 = min(n_visual, i0 + per);
-    int n_eq = 0, n_gt = 0;
-    for (int i = i0; i < i1; ++i) {
-        const uint32_t key = key_at(i);
-        n_eq += key == thr;
-        n_gt += key > thr;
-    }
-    int tot;
-    const int eq_before = block_excl_scan(n_eq, s_warp, &tot);
-    int take_eq = min(max(need_eq - eq_before, 0), n_eq);
-    const int pos0 = block_excl_scan(n_gt + take_eq, s_warp, &tot);
-    int pos = pos0;
-    for (int i = i0; i < i1; ++i) {
-        const uint32_t key = key_at(i);
-        bool keep = key > thr;
-        if (key == thr && take_eq > 0) { keep = true; --take_eq; }
-        if (keep) out[pos++] = i;
+    // ---- the kept tokens in ascending order: `need_eq` of those equal to thr (lowest indices first), all above it ----
+    const uint32_t lower = (1u << lane) - 1;
+    if (PER > 0) {
+        // (above, equal) per warp and step, in token order, both in one word: fewer than 65536 tokens
+        __syncthreads();
+        for (int i = tid; i < PER * WARPS; i += T) s_hist[i] = 0;
+        __syncthreads();
+        each([&](int kk, int, uint32_t q, bool in) {
+            const uint32_t gt = __ballot_sync(0xffffffffu, in && q > thr), eq = __ballot_sync(0xffffffffu, in && q == thr);
+            if (lane == 0) s_hist[kk * WARPS + warp] = __popc(gt) | (__popc(eq) << 16);
+        });
+        __syncthreads();
+        uint32_t mine[(PER * WARPS + T - 1) / T > 0 ? (PER * WARPS + T - 1) / T : 1], sum = 0;
+        constexpr int EPT = (PER * WARPS + T - 1) / T > 0 ? (PER * WARPS + T - 1) / T : 1;
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) { mine[i] = tid * EPT + i < PER * WARPS ? s_hist[tid * EPT + i] : 0u; sum += mine[i]; }
+        uint32_t before = block_excl_scan<T>(sum, s_warp);
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) {
+            if (tid * EPT + i < PER * WARPS) s_hist[tid * EPT + i] = before;
+            before += mine[i];
+        }
+        __syncthreads();
+        each([&](int kk, int i, uint32_t q, bool in) {
+            const uint32_t gt = __ballot_sync(0xffffffffu, in && q > thr), eq = __ballot_sync(0xffffffffu, in && q == thr);
+            const uint32_t b = s_hist[kk * WARPS + warp];
+            const uint32_t eq_before = (b >> 16) + __popc(eq & lower);
+            if (in && (q > thr || (q == thr && eq_before < need_eq)))
+                out[(b & 0xffffu) + __popc(gt & lower) + min(eq_before, need_eq)] = i;
+        });
+    } else {
+        uint32_t gt_base = 0, eq_base = 0;
+        for (int i0 = 0; i0 < n_visual; i0 += T) {
+            const int i = i0 + tid;
+            const bool in = i < n_visual;
+            const uint32_t q = in ? order_key(__ldg(x + i)) : 0u;
+            const uint32_t gt = __ballot_sync(0xffffffffu, in && q > thr), eq = __ballot_sync(0xffffffffu, in && q == thr);
+            __syncthreads();
+            if (lane == 0) s_warp[warp] = __popc(gt) | (__popc(eq) << 16);
+            __syncthreads();
+            const uint32_t o = lane < WARPS ? s_warp[lane] : 0u;
+            const uint32_t b = __reduce_add_sync(0xffffffffu, lane < warp ? o : 0u), all = __reduce_add_sync(0xffffffffu, o);
+            const uint32_t eq_before = eq_base + (b >> 16) + __popc(eq & lower);
+            if (in && (q > thr || (q == thr && eq_before < need_eq)))
+                out[gt_base + (b & 0xffffu) + __popc(gt & lower) + min(eq_before, need_eq)] = i;
+            gt_base += all & 0xffffu;
+            eq_base += all >> 16;
+        }
     }
 }
 
@@ -248,42 +301,61 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams 
         copy_rows(src_off, dst_row);
     }
 
-    // ---- kept visual rows, once the selection has written its lists ----
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // ---- kept visual rows: where they go follows from the offsets, what goes there from the selection's lists ----
     const int64_t per = p.Nt + p.slack;   // offsets[r] - first_row - r * per = kept rows of the regions before r
-    int64_t n_kept = p.offsets[n_regions] - p.first_row - (int64_t)n_regions * per;
+    auto kept_before = [&](int r) { return p.offsets[r] - p.first_row - (int64_t)r * per; };
+    int64_t n_kept = kept_before(n_regions);
     if (n_kept < 0 || n_kept > p.kept_cap) {
         if (threadIdx.x == 0) atomicExch(p.status, kStatusInconsistent);
         n_kept = 0;
     }
+    bool waited = false;
     for (int64_t first = warp0 * kGatherRowsPerWarp; first < n_kept; first += row_step) {
+        // Largest r with (kept rows before r) <= first (regions without kept rows are passed over), 32 probes at a
+        // time; the further rows are found by walking on.  (A binary search per row and behind the wait
+        // took 2 to 6 us of a warp's time.)
+        int lo = 0, n = n_regions;
+        while (n > 1) {
+            const int step = (n + 31) >> 5, at = lo + lane * step;
+            const bool below = lane * step < n && kept_before(at) <= first;
+            const int hits = __popc(__ballot_sync(0xffffffffu, below));   // offsets ascend: the first `hits` probes
+            const int next = hits > 0 ? lo + (hits - 1) * step : lo;
+            n = min(step, lo + n - next);
+            lo = next;
+        }
+        int region[kGatherRowsPerWarp];
         int64_t src_off[kGatherRowsPerWarp], dst_row[kGatherRowsPerWarp];
+        int r = lo;
+        int64_t begin = kept_before(r), end = kept_before(r + 1);
 #pragma unroll
         for (int i = 0; i < kGatherRowsPerWarp; ++i) {
             const int64_t idx = first + i;
             dst_row[i] = -1;
             src_off[i] = 0;
+            region[i] = 0;
             if (idx >= n_kept) continue;
-            // largest r with (kept rows before r) <= idx: regions without kept rows are passed over
-            int lo = 0, hi = n_regions - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (p.offsets[mid] - p.first_row - (int64_t)mid * per <= idx) lo = mid; else hi = mid - 1;
-            }
-            const int r = lo;
-            const int64_t base = p.offsets[r];
-            const int j = (int)(idx - (base - p.first_row - (int64_t)r * per));
-            const int tok = p.kept[idx];
-            const int64_t dst = base + j;
-            if (tok < 0 || tok >= p.Nv || dst < 0 || dst >= p.total_rows) {
+            while (r < n_regions - 1 && idx >= end) { ++r; begin = end; end = kept_before(r + 1); }
+            region[i] = r;
+            dst_row[i] = begin + p.first_row + r * per + (idx - begin);
+        }
+        if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+        waited = true;
+        int tok[kGatherRowsPerWarp];
+#pragma unroll
+        for (int i = 0; i < kGatherRowsPerWarp; ++i) tok[i] = first + i < n_kept ? p.kept[first + i] : 0;
+#pragma unroll
+        for (int i = 0; i < kGatherRowsPerWarp; ++i) {
+            if (first + i >= n_kept) continue;
+            if (tok[i] < 0 || tok[i] >= p.Nv || dst_row[i] < 0 || dst_row[i] >= p.total_rows) {
                 atomicExch(p.status, kStatusInconsistent);   // not copied
+                dst_row[i] = -1;
             } else {
-                src_off[i] = src_of(r, tok);
-                dst_row[i] = dst;
+                src_off[i] = src_of(region[i], tok[i]);
             }
         }
         copy_rows(src_off, dst_row);
     }
+    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 __global__ void append_kernel(uint16_t *k_out, uint16_t *v_out, const int64_t *offsets, int32_t *lens,
@@ -299,6 +371,32 @@ __global__ void append_kernel(uint16_t *k_out, uint16_t *v_out, const int64_t *o
     if (threadIdx.x == 0) lens[r] += 1;
 }
 
+struct SelectArgs {
+    const float *scores;
+    const int32_t *budgets;
+    const int64_t *offsets;
+    int n_visual, n_text, slack;
+    int64_t first_row;
+    int32_t *kept;
+    int64_t kept_cap;
+    uint32_t *status;
+};
+
+template <int T, int PER>
+cudaError_t launch_select(const SelectArgs &a, int regions, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)regions);
+    cfg.blockDim = dim3(T);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, select_kernel<T, PER>, a.scores, a.budgets, a.offsets, a.n_visual, a.n_text, a.slack,
+                              a.first_row, a.kept, a.kept_cap, a.status);
+}
+
 }  // namespace
 
 int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const float *scores,
@@ -309,17 +407,20 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
     int32_t *kept = kept_idx ? kept_idx : ws_ptr<int32_t>(ws, w.kept);
     uint32_t *status = ws_ptr<uint32_t>(ws, w.status);
     const int64_t kept_cap = (int64_t)s->batch * kept_per_sequence(s, ratio);
-    if (s->n_visual <= kSelSmemKeys) {
-        const size_t smem = (size_t)s->n_visual * 4;
-        AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               kSelSmemKeys * 4));
-        select_kernel<true><<<LB, kSelThreads, smem, st>>>(scores, budgets, out->offsets, s->n_visual, s->n_text,
-                                                           s->slack, out->first_row, kept, kept_cap, status);
-    } else {
-        select_kernel<false><<<LB, kSelThreads, 0, st>>>(scores, budgets, out->offsets, s->n_visual, s->n_text,
-                                                         s->slack, out->first_row, kept, kept_cap, status);
-    }
-    AIRCACHE_LAUNCH_CHECK();
+    // Few regions: as many threads as a block has, since the chain of a region is all there is.  Many: small blocks, of
+    // which an SM holds eight (256 threads) or four.
+    int dev = 0, sms = 0;
+    const int rc = current_device(&dev, &sms);
+    if (rc) return rc;
+    const SelectArgs a = {scores, budgets, out->offsets, s->n_visual, s->n_text, s->slack, out->first_row, kept, kept_cap, status};
+    const bool many = LB > 2 * sms;
+    cudaError_t e;
+    if (many && s->n_visual <= 256 * 16) e = launch_select<256, 16>(a, LB, st);
+    else if (many && s->n_visual <= 512 * 16) e = launch_select<512, 16>(a, LB, st);
+    else if (s->n_visual <= 1024 * 8) e = launch_select<1024, 8>(a, LB, st);
+    else if (s->n_visual <= 1024 * 16) e = launch_select<1024, 16>(a, LB, st);
+    else e = launch_select<1024, 0>(a, LB, st);
+    AIRCACHE_CUDA_TRY(e);
 
     GatherParams p;
     p.k = (const uint16_t *)f->k; p.v = (const uint16_t *)f->v;
