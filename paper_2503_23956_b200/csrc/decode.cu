@@ -8,7 +8,7 @@
 // than the grid has, the pieces are aligned to regions instead (one query load and one flush per CTA).
 // When even (region, KV head) pairs do not outnumber the CTAs, the launcher cuts by such pairs
 // ("head-split": the one-KV-head instantiation, the head taken from the item index).  With many regions
-// every CTA builds the unit prefix in shared memory (block-wide scan); with few, every warp derives the
+// every CTA builds the unit prefix in shared memory (block-wide scan), ahead of the dependency wait; with few, every warp derives the
 // handful of numbers it needs in registers (plan_few_regions), rehearsed before the dependency wait and
 // kept in the workspace between calls.  Consecutive units of one region accumulate in registers; a region
 // that lies wholly inside one CTA's range is finished and written by that CTA, otherwise the CTA writes
@@ -54,6 +54,7 @@ struct DecodeParams {
     float *partials;         // [2 * CTAs][Hq * (D + 2)]
     uint32_t *status;
     int n_regions, Hq, G;
+    int total_rows;          // of the cache
     const uint16_t *k_new, *v_new;   // Eq. 2: [L*B, Hkv, D] K and V of the token appended by this call, or NULL
     uint16_t *k_cache, *v_cache;     // the ragged cache, for the appended rows
     int32_t *lens_rw;                // lens, bumped by the last CTA when a token is appended
@@ -176,7 +177,7 @@ __device__ __forceinline__ int find_region(const int *P, int n, int u) {
 //   words 0..4: n, hs, n_ctas, ch_log2, outcome (1 or 2);  8..13: item, first unit, end unit, units, first CTA of the
 //   item, pieces;  14: region;  16..: unit count of every region
 template <int RPL, bool BALANCED>
-__device__ __forceinline__ int plan_few_regions(const int32_t *lens, const int64_t *offsets, int n, int hs, int n_ctas,
+__device__ __forceinline__ int plan_few_regions(const int32_t *lens, int appended, const int64_t *offsets, int n, int hs, int n_ctas,
                                                 int ch_log2, int c, bool store, bool force_balanced, int32_t *memo,
                                                 int *s_P, int *s_off, int *s_Q, int4 *plan) {
     const int lane = threadIdx.x & 31;
@@ -192,7 +193,7 @@ __device__ __forceinline__ int plan_few_regions(const int32_t *lens, const int64
         un[j] = ln[j] = of[j] = kept_un[j] = 0;
         const int reg = lane * rpl + j;
         if (j < rpl && reg < nr) {
-            ln[j] = max(lens[reg], 0);
+            ln[j] = max(lens[reg], 0) + appended;
             of[j] = (int)offsets[reg];
             if (memo) kept_un[j] = memo[16 + reg];
         }
@@ -374,7 +375,9 @@ __device__ __forceinline__ int plan_few_regions(const int32_t *lens, const int64
     return 1;
 }
 
-template <int D, int HKV, bool G_HI, bool HS>
+// APPEND: the call appends a token to every region (Eq. 2).  An instantiation of its own: the few instructions it takes in
+// the loop over the units cost the plain call 1 to 2 % where it streams (four requests of 1100 rows a layer: 49.1 -> 49.7 us).
+template <int D, int HKV, bool G_HI, bool HS, bool APPEND>
 __global__ void __launch_bounds__(DecodeCfg<D, HKV, G_HI, HS>::THREADS, 1)
 decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, DecodeParams p) {
     using C = DecodeCfg<D, HKV, G_HI, HS>;
@@ -398,6 +401,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     const int n = p.n_regions;   // items: regions, or (region, KV head) pairs in head-split mode
     const int hs = HS ? p.hs : 1;
     const int n_ctas = (int)gridDim.x;
+    constexpr int appended = APPEND ? 1 : 0;   // every region is one row longer than lens says
     // Programmatic dependent launch: the next kernel in the stream may be scheduled as soon as SMs free up,
     // and this one does everything that reads no global memory before it waits for its predecessor.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -425,7 +429,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     int32_t *rehearsal_memo = reinterpret_cast<int32_t *>(s_part + 3 * kPlanRegions);
     static_assert((3 * kPlanRegions + kPlanMemoInts) * 4 <= C::SCRATCH_BYTES, "rehearsal inputs fit the scratch area");
     for (int i = tid; i < kPlanRegions; i += C::THREADS) {
-        rehearsal_lens[i] = CH;
+        rehearsal_lens[i] = CH - appended;
         rehearsal_offsets[i] = 0;
         rehearsal_memo[16 + i] = i < n / hs ? 1 : 0;
         if (i < 16) {
@@ -460,7 +464,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     int r_own = -1, len_own = 0;   // the one item of this CTA and its rows, when the register plan found them
     // Eq. 2 bookkeeping: the CTA that finishes last adds the appended token to every region's length
     auto finish = [&](bool all_threads) {
-        if (p.k_new == nullptr) return;
+        if (!APPEND) return;
         if (tid == 0) {
             __threadfence();
             s_last = atomicAdd(p.done_ticket, 1) == n_ctas - 1;
@@ -471,50 +475,15 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             for (int i = tid; i < n / hs; i += (all_threads ? C::THREADS : NCW * 32)) p.lens_rw[i] += 1;
     };
 
-    // ---- few regions: every warp plans for itself, in registers; otherwise the tables below decide ----
-    bool planned = false;
-    {
-        // The plan runs twice through the same instructions: first on the made-up lengths in shared memory (with a
-        // kept plan that matches them, the usual case of a head-split launch; the by-region kernels rehearse the
-        // balanced schedule), while the kernel may not read global memory yet, then on the real ones.  A kernel's
-        // first pass through a stretch of code waits for its instructions line by line, which for this serial
-        // stretch costs more than its arithmetic; the rehearsal moves that wait in front of the dependency wait,
-        // where the CTA idles.
-        int4 plan;
-        int rc = 0;
-        const bool few = n <= n_ctas && n / hs <= kPlanRegions;   // else only the wait remains of the loop below
-#pragma unroll 1
-        for (int pass = few ? 0 : 1; pass < 2; ++pass) {
-            if (pass) {
-                asm volatile("griddepcontrol.wait;" ::: "memory");
-                if (!few) break;
-            }
-            rc = plan_few_regions<kPlanRpl, !HS>(
-                pass ? p.lens : rehearsal_lens, pass ? p.offsets : rehearsal_offsets, n, hs, n_ctas, C::CH_LOG2,
-                (int)blockIdx.x, pass != 0, pass == 0,
-                !p.plan_memo ? nullptr
-                             : (pass ? p.plan_memo + (size_t)blockIdx.x * kPlanMemoInts : (HS ? rehearsal_memo : nullptr)),
-                s_P, s_off, s_Q, &plan);
-        }
-        if (rc == 2) { finish(true); return; }
-        if (rc == 1) {
-            planned = aligned = true;
-            r_own = plan.x; len_own = plan.y; u0 = plan.z; u1 = plan.w;
-        } else if (rc == 3) {
-            planned = true;
-            total = plan.y; u0 = plan.z; u1 = plan.w;
-            upc = max(1, small_div(total + n_ctas - 1, n_ctas));
-        }
-    }
-    if (!planned) {
-        // ---- unit prefix and first row of all regions (every CTA computes the same tables) ----
+    // ---- the tables: unit prefix and first row of all regions (every CTA computes the same), and the schedule ----
+    auto build_tables = [&]() {
         {
             const int per = (n + C::THREADS - 1) / C::THREADS;
             const int i0 = min(n, tid * per), i1 = min(n, i0 + per);
             int local = 0;
             for (int i = i0; i < i1; ++i) {
-                local += (max(p.lens[i / hs], 0) + CH - 1) / CH;
-                s_off[i] = (int)p.offsets[i / hs];
+                local += (max(__ldcg(p.lens + i / hs), 0) + appended + CH - 1) / CH;
+                s_off[i] = (int)__ldcg(p.offsets + i / hs);
             }
             s_part[tid] = local;
             __syncthreads();
@@ -527,7 +496,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                     if (idx < C::THREADS) sum += s_part[idx];
                 }
                 int incl = sum;
-    #pragma unroll
+#pragma unroll
                 for (int sh = 1; sh < 32; sh <<= 1) {
                     const int o = __shfl_up_sync(0xffffffffu, incl, sh);
                     if (lane >= sh) incl += o;
@@ -542,7 +511,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             int run = s_part[tid];
             for (int i = i0; i < i1; ++i) {
                 s_P[i] = run;
-                run += (max(p.lens[i / hs], 0) + CH - 1) / CH;
+                run += (max(__ldcg(p.lens + i / hs), 0) + appended + CH - 1) / CH;
             }
             if (i1 == n && i0 < n) s_P[n] = run;
             if (n == 0 && tid == 0) s_P[0] = 0;
@@ -565,14 +534,14 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             const bool few = n <= n_ctas && total > 0 && !(2 * n > n_ctas && upc > 4);
             const int nr = n / hs;
             int sum0 = 0, sum1 = 0, sum2 = 0;
-    #pragma unroll 1
+#pragma unroll 1
             for (int r = lane; few && r < nr; r += 32) {
                 const int u = s_P[r * hs + 1] - s_P[r * hs];
                 sum0 += small_div(u + upc - 1, upc);
                 sum1 += small_div(u + upc, upc + 1);
                 sum2 += small_div(u + upc + 1, upc + 2);
             }
-    #pragma unroll
+#pragma unroll
             for (int sh = 16; sh > 0; sh >>= 1) {
                 sum0 += __shfl_xor_sync(0xffffffffu, sum0, sh);
                 sum1 += __shfl_xor_sync(0xffffffffu, sum1, sh);
@@ -582,18 +551,18 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             const bool found = few && (sum0 <= lim || sum1 <= lim || sum2 <= lim);
             const int upc_a = sum0 <= lim ? upc : (sum1 <= lim ? upc + 1 : upc + 2);
             int carry = 0;
-    #pragma unroll 1
+#pragma unroll 1
             for (int base = 0; found && base <= nr; base += 32) {
                 const int r = base + lane;
                 const int v = r < nr ? small_div(s_P[r * hs + 1] - s_P[r * hs] + upc_a - 1, upc_a) : 0;
                 int incl = v;
-    #pragma unroll
+#pragma unroll
                 for (int sh = 1; sh < 32; sh <<= 1) {
                     const int o = __shfl_up_sync(0xffffffffu, incl, sh);
                     if (lane >= sh) incl += o;
                 }
                 if (r < nr) {
-    #pragma unroll 1
+#pragma unroll 1
                     for (int h = 0; h < hs; ++h) s_Q[r * hs + h] = (carry + incl - v) * hs + h * v;
                 } else if (r == nr) {
                     s_Q[n] = (carry + incl - v) * hs;
@@ -605,38 +574,87 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         __syncthreads();
         aligned = s_aligned != 0;
 
-        // an item without rows yields zeros - or, when a token is appended, that token's value (softmax over one key)
-        for (int r = blockIdx.x; r < n; r += n_ctas) {
-            if (s_P[r + 1] != s_P[r]) continue;
-            const int reg = r / hs;
-            for (int i = tid; i < p.Hq * D; i += C::THREADS) {
-                float v = 0.f;
-                if (p.k_new) {
-                    const int kvh = HS ? r % hs : (i / D) / p.G;
-                    v = bf16_to_f32(p.v_new[((int64_t)reg * p.kv_heads + kvh) * D + i % D]);
-                }
-                p.out[(int64_t)r * p.Hq * D + i] = v;
-            }
-            if (p.k_new) {
-                const int heads = HS ? 1 : p.kv_heads, h0 = HS ? r % hs : 0;
-                for (int i = tid; i < heads * D; i += C::THREADS) {
-                    const int64_t src = ((int64_t)reg * p.kv_heads + h0) * D + i;
-                    const int64_t dst = ((int64_t)s_off[r] * p.kv_heads + h0) * D + i;
-                    p.k_cache[dst] = p.k_new[src];
-                    p.v_cache[dst] = p.v_new[src];
-                }
-            }
-        }
         if (aligned) {
             const int c = (int)blockIdx.x;
-            if (c >= s_Q[n]) { finish(true); return; }
-            const int r = find_region(s_Q, n, c);      // largest r with s_Q[r] <= c: the region this CTA cuts
-            const int pieces = s_Q[r + 1] - s_Q[r], j = c - s_Q[r], units = s_P[r + 1] - s_P[r];
-            u0 = s_P[r] + small_div(units * j, pieces);          // units * pieces < 2^24: both are at most a few thousand
-            u1 = s_P[r] + small_div(units * (j + 1), pieces);
+            if (c < s_Q[n]) {
+                const int r = find_region(s_Q, n, c);      // largest r with s_Q[r] <= c: the region this CTA cuts
+                const int pieces = s_Q[r + 1] - s_Q[r], j = c - s_Q[r], units = s_P[r + 1] - s_P[r];
+                u0 = s_P[r] + small_div(units * j, pieces);          // units * pieces < 2^24: both are at most a few thousand
+                u1 = s_P[r] + small_div(units * (j + 1), pieces);
+            } else {
+                u0 = u1 = 0;
+            }
         } else {
             u0 = min(total, (int)blockIdx.x * upc);
             u1 = min(total, u0 + upc);
+        }
+    };
+    // ---- few regions: every warp plans for itself, in registers; otherwise the tables below decide ----
+    bool planned = false;
+    const bool few = n <= n_ctas && n / hs <= kPlanRegions;
+    if (few) {
+        // The plan runs twice through the same instructions: first on the made-up lengths in shared memory (with a
+        // kept plan that matches them, the usual case of a head-split launch; the by-region kernels rehearse the
+        // balanced schedule), while the kernel may not read global memory yet, then on the real ones.  A kernel's
+        // first pass through a stretch of code waits for its instructions line by line, which for this serial
+        // stretch costs more than its arithmetic; the rehearsal moves that wait in front of the dependency wait,
+        // where the CTA idles.
+        int4 plan;
+        int rc = 0;
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            if (pass) asm volatile("griddepcontrol.wait;" ::: "memory");
+            rc = plan_few_regions<kPlanRpl, !HS>(
+                pass ? p.lens : rehearsal_lens, appended, pass ? p.offsets : rehearsal_offsets, n, hs, n_ctas, C::CH_LOG2,
+                (int)blockIdx.x, pass != 0, pass == 0,
+                !p.plan_memo ? nullptr
+                             : (pass ? p.plan_memo + (size_t)blockIdx.x * kPlanMemoInts : (HS ? rehearsal_memo : nullptr)),
+                s_P, s_off, s_Q, &plan);
+        }
+        if (rc == 2) { finish(true); return; }
+        if (rc == 1) {
+            planned = aligned = true;
+            r_own = plan.x; len_own = plan.y; u0 = plan.z; u1 = plan.w;
+        } else if (rc == 3) {
+            planned = true;
+            total = plan.y; u0 = plan.z; u1 = plan.w;
+            upc = max(1, small_div(total + n_ctas - 1, n_ctas));
+        }
+    }
+    // Many regions: the tables are built before the dependency wait, from whatever lengths and first rows are there -
+    // usually the right ones - and checked against what is read behind it.  With them the CTA asks for its first units'
+    // lines to be brought into L2: a hint that consumes no value, kept inside the cache whatever was read.  (What is
+    // read early goes around L1.)  Four requests of 1100 rows in 28 layers: 49.0 us a call with the tables built behind the
+    // wait, 47.8 with them built before it, 46.3 with the hint as well.
+    const bool tables = !planned;
+#pragma unroll 1
+    for (int pass = few ? 1 : 0; pass < 2 && !planned; ++pass) {
+        build_tables();
+        if (pass) break;
+        if (wid == NCW && lane == 0 && u0 < u1) {
+            int r = find_region(s_P, n, u0);
+            for (int u = u0; u < u1 && u < u0 + kStages; ++u) {
+                while (u >= s_P[r + 1] && r + 1 < n) ++r;
+                const int row0 = s_off[r] + (u - s_P[r]) * CH;
+                for (int x = 0; x < HKV * C::HALVES && row0 >= 0 && row0 < p.total_rows; ++x) {
+                    const int head = HS ? r % hs : x / C::HALVES;
+                    tma_prefetch_3d(&tm_k, x % C::HALVES * 64, head, row0);
+                    tma_prefetch_3d(&tm_v, x % C::HALVES * 64, head, row0);
+                }
+            }
+        }
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        bool same = true;
+        for (int i = tid; i < n; i += C::THREADS)
+            same = same && (max(__ldcg(p.lens + i / hs), 0) + appended + CH - 1) / CH == s_P[i + 1] - s_P[i] &&
+                   (int)__ldcg(p.offsets + i / hs) == s_off[i];
+        planned = __syncthreads_and(same);
+    }
+    if (tables) {
+        // an item without rows yields zeros
+        for (int r = blockIdx.x; r < n; r += n_ctas) {
+            if (s_P[r + 1] != s_P[r]) continue;
+            for (int i = tid; i < p.Hq * D; i += C::THREADS) p.out[(int64_t)r * p.Hq * D + i] = 0.f;
         }
     }
     if (u0 >= u1) { finish(true); return; }
@@ -686,7 +704,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                 }
             }
         }
-        if (p.k_new != nullptr && r_own >= 0) {
+        if (APPEND && r_own >= 0) {
             // Eq. 2 bookkeeping off the critical path: a CTA planned in registers needs lens no more (its row
             // count sits in registers), so its idle producer draws the ticket now instead of the consumers at
             // the end; lens is bumped by whoever draws the last ticket, when no CTA will read it again.
@@ -707,7 +725,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     const int gid = lane >> 2, t = lane & 3;
     const int G = p.G;
 
-    int len = 0;      // rows of the item being processed
+    int len = 0;      // rows of the item being processed, an appended token among them
     // The block's products are taken transposed - S^T = K Q^T and O^T = V^T P^T - so that the 16 rows of the tensor
     // core tile are keys (respectively channels) and its 8 columns the query heads of the KV group: a group of up
     // to 8 heads fills one column tile, where heads as rows would leave half of a 16-row tile empty.
@@ -736,8 +754,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     };
 
     // One block of 16 keys at rows blk_row0.. of a (K, V) tile in shared memory; the block's first key is row j0
-    // of the region, which has len rows.  sub_stride is the distance between the two 64-channel halves.
-    auto process_block = [&](uint32_t k_base, uint32_t v_base, uint32_t sub_stride, int blk_row0, int j0, int len) {
+    // of the region, which has len rows.
+    auto process_block = [&](uint32_t k_base, uint32_t v_base, int blk_row0, int j0, int len) {
         const int mi = lane >> 3, rr = lane & 7;
 
         // ---- S^T = K Q^T for 16 keys; two accumulators per tile halve the chain of dependent MMAs ----
@@ -752,7 +770,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             for (int kk = 0; kk < D / 16; ++kk) {
                 const int hf = kk >> 2, chunk = ((kk & 3) << 1) + (mi >> 1);
                 uint32_t a[4];   // keys 0-7 / 8-15 of channels kk*16.., then of channels kk*16 + 8..
-                ldmatrix_x4(a, k_base + hf * sub_stride + row * 128 + ((chunk ^ (row & 7)) << 4));
+                ldmatrix_x4(a, k_base + hf * C::SUBTILE + row * 128 + ((chunk ^ (row & 7)) << 4));
 #pragma unroll
                 for (int nt = 0; nt < NROW; ++nt)
                     mma_bf16_16816(sacc[nt][kk & 1], a[0], a[1], a[2], a[3], qb[nt][kk][0], qb[nt][kk][1]);
@@ -821,7 +839,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                 const int cg = mt * 2 + (mi & 1);
                 const int hf = cg >> 3, chunk = cg & 7;
                 uint32_t a[4];   // channels mt*16.. / +8 of keys 2t, 2t+1, then of keys 2t+8, 2t+9
-                ldmatrix_x4_trans(a, v_base + hf * sub_stride + row * 128 + ((chunk ^ (row & 7)) << 4));
+                ldmatrix_x4_trans(a, v_base + hf * C::SUBTILE + row * 128 + ((chunk ^ (row & 7)) << 4));
                 if (tail) { a[0] &= vmask0; a[1] &= vmask0; a[2] &= vmask1; a[3] &= vmask1; }
 #pragma unroll
                 for (int nt = 0; nt < NROW; ++nt) {
@@ -832,40 +850,32 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         }
     };
 
-    // Writes the region's result (whole region inside this CTA) or an unnormalised partial.
-    uint4 tok = make_uint4(0u, 0u, 0u, 0u);
-    bool tok_ready = false;
-    // 16 bytes of the appended token's row of item r: lanes 0-15 chunk c of K, lanes 16-31 chunk c of V
-    auto load_token = [&](int r) {
-        const int reg = r / hs, head = HS ? r % hs : g;
-        const int64_t src = ((int64_t)reg * p.kv_heads + head) * D;
-        const int c = lane & 15;
-        const uint16_t *from = lane < 16 ? p.k_new : p.v_new;
-        return c < D / 8 ? __ldg(reinterpret_cast<const uint4 *>(from + src) + c) : make_uint4(0u, 0u, 0u, 0u);
+    // Eq. 2: the appended token is the last row of its item, which the cache does not hold yet.  The warp whose block has
+    // that row (in the CTA that holds the item's last unit) asks for it when it starts on the item, and lays it over
+    // what the tile's load found there.  (As a block of its own at the end it took 0.9 us of a call's 11.8, at the
+    // beginning, while the first keys are on their way, as much.)
+    uint4 tok = make_uint4(0u, 0u, 0u, 0u);   // 16 bytes: lanes 0-15 chunk c of K, lanes 16-31 chunk c of V
+    bool tok_mine = false;
+    auto ask_token = [&](int r) {
+        tok_mine = APPEND && u1 >= s_P[r + 1] && ks == ((len - 1) & (CH - 1)) >> 4;
+        const int reg = r / hs, head = HS ? r % hs : g, c = lane & 15;
+        if (tok_mine && c < D / 8)
+            tok = __ldg(reinterpret_cast<const uint4 *>((lane < 16 ? p.k_new : p.v_new) + ((int64_t)reg * p.kv_heads + head) * D) + c);
     };
-    auto flush = [&](int r, int ustart, int uend) {
-        if (p.k_new != nullptr && uend == s_P[r + 1]) {
-            // Eq. 2: this CTA holds the item's last unit, so the appended token joins here.  Warp ks = 0 of every
-            // head copies the token's K and V rows into a one-row tile in the scratch area (rows 1..15 of that
-            // tile are whatever lies behind it: masked like any row past the end), stores them into the cache
-            // and runs the block routine on it.
-            if (ks == 0) {
-                const int head = HS ? r % hs : g;
-                uint8_t *area = reinterpret_cast<uint8_t *>(s_merge) + g * (4 * 128);
-                const int64_t dst = (((int64_t)s_off[r] + len) * p.kv_heads + head) * D;
-                const int c = lane & 15;
-                const uint4 v = tok_ready ? tok : load_token(r);
-                tok_ready = false;
-                if (c < D / 8) {
-                    uint16_t *to = lane < 16 ? p.k_cache : p.v_cache;
-                    *reinterpret_cast<uint4 *>(area + (lane < 16 ? 0 : 2 * 128) + (c >> 3) * 128 + (c & 7) * 16) = v;
-                    reinterpret_cast<uint4 *>(to + dst)[c] = v;
-                }
-                __syncwarp();
-                process_block(smem_u32(area), smem_u32(area + 2 * 128), 128, 0, len, len + 1);
-            }
-            consumer_bar(NCW * 32);   // the scratch area becomes the merge buffer below
+    auto place_token = [&](int r, uint32_t k_base) {
+        const int head = HS ? r % hs : g, c = lane & 15, row = (len - 1) & (CH - 1);
+        if (c < D / 8) {
+            const uint32_t at = k_base + (lane < 16 ? 0 : C::KV_BYTES) + (c >> 3) * C::SUBTILE + row * 128 + (((c & 7) ^ (row & 7)) << 4);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(tok.x), "r"(tok.y), "r"(tok.z), "r"(tok.w) : "memory");
+            uint16_t *to = (lane < 16 ? p.k_cache : p.v_cache) + (((int64_t)s_off[r] + len - 1) * p.kv_heads + head) * D;
+            reinterpret_cast<uint4 *>(to)[c] = tok;
         }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the next load into the stage comes after it
+        __syncwarp();
+    };
+
+    // Writes the region's result (whole region inside this CTA) or an unnormalised partial.
+    auto flush = [&](int r, int ustart, int uend) {
 #pragma unroll
         for (int nt = 0; nt < NROW; ++nt)
 #pragma unroll
@@ -874,11 +884,13 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                 l_run[nt][1] += __shfl_xor_sync(0xffffffffu, l_run[nt][1], sh);
             }
         // the KSPLIT warps of a KV head merge their states pairwise: in every round the upper half of the
-        // remaining warps hands its (max, sum, accumulator) to the lower half through shared memory
+        // remaining warps hands its (max, sum, accumulator) to the lower half through shared memory.  Slots: ks - half in
+        // the first round, later the slot that the warp itself has read then, so one barrier a round is enough.
 #pragma unroll
         for (int half = KSPLIT / 2; half >= 1; half >>= 1) {
             if (ks >= half && ks < 2 * half) {
-                float *dst = s_merge + (size_t)(g * C::MERGE_SLOTS + ks - half) * C::MERGE_FLOATS_PER_WARP + lane;
+                const int slot = half == KSPLIT / 2 ? ks - half : ks;
+                float *dst = s_merge + (size_t)(g * C::MERGE_SLOTS + slot) * C::MERGE_FLOATS_PER_WARP + lane;
                 int c = 0;
 #pragma unroll
                 for (int nt = 0; nt < NROW; ++nt) {
@@ -894,7 +906,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             }
             consumer_bar(NCW * 32);
             if (ks < half) {
-                const float *src = s_merge + (size_t)(g * C::MERGE_SLOTS + ks) * C::MERGE_FLOATS_PER_WARP + lane;
+                const int slot = half == KSPLIT / 2 ? ks : ks + half;
+                const float *src = s_merge + (size_t)(g * C::MERGE_SLOTS + slot) * C::MERGE_FLOATS_PER_WARP + lane;
                 int c = 0;
 #pragma unroll
                 for (int nt = 0; nt < NROW; ++nt) {
@@ -916,9 +929,10 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                         for (int i = 0; i < 4; ++i)
                             oacc[nt][mt][i] = oacc[nt][mt][i] * a[i & 1] + src[32 * c++] * b[i & 1];
                 }
+                __syncwarp();
             }
-            consumer_bar(NCW * 32);
         }
+        if (KSPLIT > 1 && uend != u1) consumer_bar(NCW * 32);   // the slots are free for the next item's merge
         const bool whole = (ustart == s_P[r]) && (uend == s_P[r + 1]);
         if (ks == 0) {
             // this thread's values: heads nt*8 + 2t + e, channels mt*16 + gid and + 8 (the eight gid lanes of a
@@ -957,14 +971,14 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         if (!whole) {
             // split-K combine without a second launch: publish the partial, draw a ticket; the CTA that draws
             // the region's last ticket merges all partials in CTA order
-            __threadfence();
             consumer_bar(NCW * 32);
             int c0, c1;
             span_of(r, c0, c1);
             if (tid == 0) {
-                const int tk = atomicAdd(p.tickets + r, 1);
+                // (releases what the barrier has gathered; cheaper than a fence by every thread)
+                int tk;
+                asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(tk) : "l"(p.tickets + r) : "memory");
                 s_last = (tk == c1 - c0);
-                if (s_last) __threadfence();
             }
             consumer_bar(NCW * 32);
             if (s_last) {
@@ -1101,14 +1115,9 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
 
     int r = r_own >= 0 ? r_own : find_region(s_P, n, u0);
     int seg_start = u0;
-    len = r_own >= 0 ? len_own : p.lens[r / hs];
+    len = r_own >= 0 ? len_own : max(p.lens[r / hs], 0) + appended;
     load_q(r);
-    // Eq. 2: when this CTA will flush the item's last unit, the appended token's K (lanes 0-15) and V (lanes 16-31)
-    // are requested now, so that the flush does not wait for them
-    if (p.k_new != nullptr && ks == 0 && r_own >= 0 && u1 == s_P[r + 1]) {
-        tok = load_token(r);
-        tok_ready = true;
-    }
+    ask_token(r);
     int it = 0;
     bool ok = true;
     for (int u = u0; u < u1; ++u, ++it) {
@@ -1116,8 +1125,9 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             flush(r, seg_start, u);
             while (u >= s_P[r + 1]) ++r;
             seg_start = u;
-            len = p.lens[r / hs];
+            len = max(p.lens[r / hs], 0) + appended;
             load_q(r);
+            ask_token(r);
         }
         const int s = it % kStages;
         ok = mbar_wait(smem_u32(&s_bar[s]), (it / kStages) & 1, &s_abort, p.status, 2);
@@ -1125,7 +1135,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         const int j0 = (u - s_P[r]) * CH + ks * 16;  // first row of this warp's block inside the region
         if (j0 < len) {
             const uint32_t k_base = smem_u32(s_stage + s * C::STAGE_BYTES) + g * C::HALVES * C::SUBTILE;
-            process_block(k_base, k_base + C::KV_BYTES, C::SUBTILE, ks * 16, j0, len);
+            if (APPEND && tok_mine && u + 1 == s_P[r + 1]) place_token(r, k_base);
+            process_block(k_base, k_base + C::KV_BYTES, ks * 16, j0, len);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&s_bar[kStages + s]));
@@ -1152,8 +1163,8 @@ int make_map(CUtensorMap *tm, const void *base, int D, int Hkv, int64_t rows, in
     return AIRCACHE_OK;
 }
 
-template <int D, int HKV, bool G_HI, bool HS>
-int launch_decode_t(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, cudaStream_t st) {
+template <int D, int HKV, bool G_HI, bool HS, bool APPEND>
+int launch_decode_a(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, cudaStream_t st) {
     using C = DecodeCfg<D, HKV, G_HI, HS>;
     CUtensorMap tm_k, tm_v;
     int rc = make_map(&tm_k, c->k, D, kv_heads, c->total_rows, C::CH);
@@ -1165,7 +1176,7 @@ int launch_decode_t(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, c
     // the shared-memory limit is a property of the kernel on a device: set once for each
     static std::atomic<bool> ready[kMaxDevices];
     if (dev >= kMaxDevices || !ready[dev].load(std::memory_order_acquire)) {
-        AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, HKV, G_HI, HS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, HKV, G_HI, HS, APPEND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                C::SMEM_BYTES));
         if (dev < kMaxDevices) ready[dev].store(true, std::memory_order_release);
     }
@@ -1179,8 +1190,14 @@ int launch_decode_t(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    AIRCACHE_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_kernel<D, HKV, G_HI, HS>, tm_k, tm_v, p));
+    AIRCACHE_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_kernel<D, HKV, G_HI, HS, APPEND>, tm_k, tm_v, p));
     return AIRCACHE_OK;
+}
+
+template <int D, int HKV, bool G_HI, bool HS>
+int launch_decode_t(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, cudaStream_t st) {
+    return p.k_new ? launch_decode_a<D, HKV, G_HI, HS, true>(c, p, kv_heads, st)
+                   : launch_decode_a<D, HKV, G_HI, HS, false>(c, p, kv_heads, st);
 }
 
 template <int D, int HKV>
@@ -1259,6 +1276,7 @@ int launch_decode(const aircache_shape_t *s, const aircache_ragged_t *c, const v
     p.Hq = s->n_q_heads;
     p.G = s->n_q_heads / s->n_kv_heads;
     p.sl2 = s->scale * kLog2e;
+    p.total_rows = (int)c->total_rows;
     p.hs = 1;
     aircache_shape_t view;
     s = decode_view(s, p, &view);
@@ -1318,6 +1336,7 @@ int launch_decode_static(const aircache_shape_t *s, const aircache_ragged_t *c, 
     p.Hq = s->n_q_heads;
     p.G = s->n_q_heads / s->n_kv_heads;
     p.sl2 = s->scale * kLog2e;
+    p.total_rows = (int)c->total_rows;
     p.hs = 1;
     aircache_shape_t view;
     s = decode_view(s, p, &view);
