@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libaircache.so, the sm_100a CUDA library of the AirCache hot path.
+"""Thin binding of libaircache.so, the sm_100a CUDA library of the AirCache hot path (ctypes; csrc/binding.c for the calls
+that a decoder makes for every token).
 
 Argument marshalling only: every function below forwards to the C entry point of the same name
 (include/aircache.h) with raw device pointers taken from torch tensors.  All arithmetic of the
@@ -105,6 +106,22 @@ def lib() -> C.CDLL:
 
 def exported_symbols() -> list[str]:
     return list(_SIGNATURES)
+
+
+_native = None   # (module, addresses of aircache_decode_attn and aircache_decode_step) once CUDA is up
+
+
+def _per_token_calls():
+    """The native marshalling of the per-token entry points (csrc/binding.c); None while CUDA is not initialised (there
+    is no current stream to ask for then)."""
+    global _native
+    if _native is None and torch.cuda.is_initialized():
+        from . import _binding
+        _binding.setup(Shape, Ragged, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        handle = lib()
+        _native = (_binding, C.cast(handle.aircache_decode_attn, C.c_void_p).value,
+                   C.cast(handle.aircache_decode_step, C.c_void_p).value)
+    return _native
 
 
 # ------------------------------------------------------------------------------------------------
@@ -215,16 +232,24 @@ def aircache_compact(sh, full, scores, budgets, ratio, out, kept_idx, workspace,
 
 
 def aircache_decode_attn(sh, cache, q, out, workspace, stream=None, check=True) -> int:
-    rc = lib().aircache_decode_attn(C.byref(sh), C.byref(cache), _ptr(q), _ptr(out), _ptr(workspace),
-                                    _nbytes(workspace), _stream(stream))
+    native = _native or _per_token_calls()
+    if native:
+        rc = native[0].decode_attn(native[1], sh, cache, q, out, workspace, stream)
+    else:
+        rc = lib().aircache_decode_attn(C.byref(sh), C.byref(cache), _ptr(q), _ptr(out), _ptr(workspace),
+                                        _nbytes(workspace), _stream(stream))
     if check:
         _check("aircache_decode_attn", rc)
     return rc
 
 
 def aircache_decode_step(sh, cache, q, k_new, v_new, appended, out, workspace, stream=None, check=True) -> int:
-    rc = lib().aircache_decode_step(C.byref(sh), C.byref(cache), _ptr(q), _ptr(k_new), _ptr(v_new), appended,
-                                    _ptr(out), _ptr(workspace), _nbytes(workspace), _stream(stream))
+    native = _native or _per_token_calls()
+    if native:
+        rc = native[0].decode_step(native[2], sh, cache, q, k_new, v_new, appended, out, workspace, stream)
+    else:
+        rc = lib().aircache_decode_step(C.byref(sh), C.byref(cache), _ptr(q), _ptr(k_new), _ptr(v_new), appended,
+                                        _ptr(out), _ptr(workspace), _nbytes(workspace), _stream(stream))
     if check:
         _check("aircache_decode_step", rc)
     return rc

@@ -5,10 +5,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libaircache.so")
+BINDING_SOURCE = os.path.join(CSRC, "binding.c")
+BINDING = os.path.join(PKG, "_binding" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 SOURCES = ["api.cu", "score.cu", "score_cluster.cu", "score_dense.cu", "budget.cu", "compact.cu", "decode.cu"]
 HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "ptx.cuh"), os.path.join(CSRC, "score.cuh"), os.path.join(os.path.dirname(PKG), "include", "aircache.h")]
 
@@ -28,8 +31,22 @@ def stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_binding(force: bool = False) -> str:
+    """Compile the native argument marshalling of the per-token calls (csrc/binding.c) next to this file."""
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= os.path.getmtime(BINDING_SOURCE):
+        return BINDING
+    tmp = BINDING + f".tmp{os.getpid()}"
+    cc = os.environ.get("CC") or shutil.which("gcc") or shutil.which("cc")
+    if not cc:
+        raise RuntimeError("no C compiler found: the binding cannot be built")
+    subprocess.check_call([cc, "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], BINDING_SOURCE, "-o", tmp])
+    os.replace(tmp, BINDING)
+    return BINDING
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu for sm_100a into one shared library next to this file."""
+    """Compile every .cu for sm_100a into one shared library next to this file, and the native part of the binding."""
+    build_binding(force)
     if not force and not stale():
         return LIB
     tmp = LIB + f".tmp{os.getpid()}"

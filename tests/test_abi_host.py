@@ -6,6 +6,7 @@ import re
 
 import numpy as np
 import pytest
+import torch
 
 import paper_2503_23956_b200 as ac
 
@@ -161,3 +162,29 @@ def test_binding_has_no_fallback(monkeypatch, tmp_path):
     monkeypatch.setattr(ac, "LIB", str(tmp_path / "libaircache.so"))
     with pytest.raises(RuntimeError, match="no CPU or PyTorch fallback"):
         ac.aircache_version()
+
+
+def test_native_marshalling_of_the_per_token_calls(monkeypatch):
+    """csrc/binding.c hands over what the ctypes path does: the same return codes, for tensors, addresses and None, and a
+    TypeError where ctypes refuses an argument."""
+    import ctypes as C
+    from paper_2503_23956_b200 import _binding
+    _binding.setup(ac.Shape, ac.Ragged, lambda: 0, lambda dev: 0)
+    fns = [C.cast(f, C.c_void_p).value for f in (ac.lib().aircache_decode_attn, ac.lib().aircache_decode_step)]
+    sh = ac.shape(2, 1, 4, 2, 64, 16, 8, 4, slack=2)
+    P = 0x10000000   # 256-byte aligned fake address, never followed: every call fails in the host-side checks
+    cache = ac.Ragged(P, P, P, P, 100, 0)
+    small, odd = torch.zeros(16, dtype=torch.uint8), P + 4
+    calls = [("attn", (sh, cache, q, P, ws)) for q in (P, None, odd) for ws in (None, P, small)]
+    calls += [("attn", (ac.shape(0, 1, 4, 2, 64, 16, 8, 4), cache, P, P, P)), ("attn", (sh, ac.Ragged(), P, P, P))]
+    calls += [("step", (sh, cache, P, k, P, n, P, P)) for k in (P, None, odd) for n in (0, -1, 2)]
+    for kind, args in calls:
+        fn = ac.aircache_decode_attn if kind == "attn" else ac.aircache_decode_step
+        monkeypatch.setattr(ac, "_native", None)
+        monkeypatch.setattr(ac, "_per_token_calls", lambda: None)
+        want = fn(*args, stream=0, check=False)
+        monkeypatch.setattr(ac, "_native", (_binding, *fns))
+        assert want < 0 and fn(*args, stream=None, check=False) == want, (kind, want)
+    with pytest.raises(TypeError):
+        ac.aircache_decode_attn(cache, cache, P, P, P, stream=0)
+    monkeypatch.setattr(ac, "_native", None)   # (set up again, with torch's functions, at the next call)
