@@ -175,12 +175,13 @@ int64_t aircache_workspace_bytes(const aircache_shape_t *shape);
  *   scores      fp32 [L, B, Nv]        output I_v
  *   elite_mask  u64  [L, B, Hq, ceil(W/64)]  output, candidate w is elite <=> bit w % 64 of word w / 64 is
  *                                      set (one word per head up to W = 64, two beyond); may be NULL
- * The blocks of the scoring kernel that share a KV group wait for one another
- * (a bounded wait; safe because the library only lets them when at most half of
- * the blocks the GPU holds at once are involved).  If other work keeps most of
- * the GPU busy for the whole wait (a quarter of a second), the wait gives up,
- * the scores are incomplete and aircache_check_status() reports
- * AIRCACHE_ERR_TIMEOUT.
+ * The blocks that share a KV group wait for one another: the blocks of one thread-
+ * block cluster, which the hardware starts together, up to 16384 visual tokens;
+ * beyond (and for caches that no tensor map describes) blocks of one grid, which
+ * the library only lets do so when at most half of the blocks the GPU holds at
+ * once are involved.  All waits are bounded; if one gives up (other work keeps
+ * most of the GPU busy for a quarter of a second), the scores are incomplete and
+ * aircache_check_status() reports AIRCACHE_ERR_TIMEOUT.
  */
 int aircache_score(const aircache_shape_t *shape, const aircache_full_t *full, const void *q_window,
                    float alpha, float *scores, uint64_t *elite_mask, void *workspace, int64_t workspace_bytes,
