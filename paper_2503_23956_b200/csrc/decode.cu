@@ -645,9 +645,20 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         }
         asm volatile("griddepcontrol.wait;" ::: "memory");
         bool same = true;
-        for (int i = tid; i < n; i += C::THREADS)
-            same = same && (max(__ldcg(p.lens + i / hs), 0) + appended + CH - 1) / CH == s_P[i + 1] - s_P[i] &&
-                   (int)__ldcg(p.offsets + i / hs) == s_off[i];
+        for (int i0 = tid; i0 < n; i0 += 4 * C::THREADS) {   // eight loads in flight: they are what the check costs
+            int ln[4], of[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = i0 + k * C::THREADS;
+                ln[k] = i < n ? __ldcg(p.lens + i / hs) : 0;
+                of[k] = i < n ? (int)__ldcg(p.offsets + i / hs) : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = i0 + k * C::THREADS;
+                if (i < n && ((max(ln[k], 0) + appended + CH - 1) / CH != s_P[i + 1] - s_P[i] || of[k] != s_off[i])) same = false;
+            }
+        }
         planned = __syncthreads_and(same);
     }
     if (tables) {
