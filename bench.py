@@ -55,7 +55,7 @@ Q_RING, O_RING = 16, 8
 # batch 16, the largest case the capture rules allow; traffic grows in proportion to the rows, so it is scaled
 # to the launch that was timed).  Valid only for the kernel source it was taken on (sha1 of csrc/decode.cu,
 # first 12 hex); null otherwise.
-NCU_TRAFFIC = {"workload": "c3", "decode_cu_sha1": "275867bb0ec6", "bytes_per_valid_row": 2101.25}
+NCU_TRAFFIC = {"workload": "c3", "decode_cu_sha1": "0ce8e1446ce4", "bytes_per_valid_row": 2101.65}
 
 
 def parse_args():
@@ -308,7 +308,7 @@ def rooflines(ac, wl, m, rotate, n_dec, traffic=None):
     comp = roof("select_kernel + gather_kernel per aircache_compact call", compact_bytes,
                 m["stage_ms"]["compact"] * 1e3 / rotate)
     score_bytes = LB * wl.n_visual * (row_bytes + 4)
-    score = roof("elite_kernel + onepass_kernel + group_sum_kernel per aircache_score call", score_bytes,
+    score = roof("score_cluster_kernel per aircache_score call", score_bytes,
                  m["stage_ms"]["score"] * 1e3 / rotate)
     return dec, comp, score
 
