@@ -89,6 +89,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 __device__ __forceinline__ void consumer_bar(int n_threads) {
     asm volatile("bar.sync 1, %0;" ::"r"(n_threads) : "memory");
 }
+// the warps of a CTA that have planned, by consumers (arrive) and the producer (wait)
+template <bool ARRIVE>
+__device__ __forceinline__ void plan_bar(int n_threads) {
+    if (ARRIVE) asm volatile("bar.arrive 2, %0;" ::"r"(n_threads) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"r"(n_threads) : "memory");
+}
 __device__ __forceinline__ float exp2_or_zero(float m, float m_new) {
     return m == -INFINITY ? 0.f : fast_exp2(m - m_new);
 }
@@ -465,6 +471,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     // Eq. 2 bookkeeping: the CTA that finishes last adds the appended token to every region's length
     auto finish = [&](bool all_threads) {
         if (!APPEND) return;
+        // (no thread reads lens any more, for its plan or for an item's rows, when the ticket is drawn)
+        if (all_threads) __syncthreads();
         if (tid == 0) {
             __threadfence();
             s_last = atomicAdd(p.done_ticket, 1) == n_ctas - 1;
@@ -718,7 +726,10 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         if (APPEND && r_own >= 0) {
             // Eq. 2 bookkeeping off the critical path: a CTA planned in registers needs lens no more (its row
             // count sits in registers), so its idle producer draws the ticket now instead of the consumers at
-            // the end; lens is bumped by whoever draws the last ticket, when no CTA will read it again.
+            // the end; lens is bumped by whoever draws the last ticket, when no CTA will read it again.  Every warp
+            // read lens for its own plan: the consumers have arrived here when they have theirs.
+            __syncwarp();
+            plan_bar<false>(C::THREADS);
             int last = 0;
             if (lane == 0) {
                 last = atomicAdd(p.done_ticket, 1) == n_ctas - 1;
@@ -732,6 +743,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     }
 
     // ================================= consumer warps =================================
+    if (APPEND && r_own >= 0) plan_bar<true>(C::THREADS);   // (the producer waits, these do not)
     const int g = wid / KSPLIT, ks = wid % KSPLIT;
     const int gid = lane >> 2, t = lane & 3;
     const int G = p.G;
