@@ -179,7 +179,7 @@ __device__ __forceinline__ int find_region(const int *P, int n, int u) {
 // keeps the unit counts it planned for and the outcome; when the counts read now equal the kept ones, the
 // outcome is taken from there and the arithmetic (about a microsecond of dependent steps) is skipped.  A CTA
 // reads and writes only its own words, and only after the kernel's dependency wait (the rehearsal passes words
-// in shared memory, hence the plain loads).
+// in shared memory, hence the plain loads); its warps, each of which reads them, meet before one writes.
 //   words 0..4: n, hs, n_ctas, ch_log2, outcome (1 or 2);  8..13: item, first unit, end unit, units, first CTA of the
 //   item, pieces;  14: region;  16..: unit count of every region
 template <int RPL, bool BALANCED>
@@ -333,6 +333,8 @@ __device__ __forceinline__ int plan_few_regions(const int32_t *lens, int appende
         }
     }
     const unsigned ball = __ballot_sync(0xffffffffu, v_reg >= 0);
+    // All warps of the CTA have read the kept plan (and all found that it does not fit) before one of them writes it.
+    if (memo != nullptr && store) __syncthreads();
     if (record) {
 #pragma unroll
         for (int j = 0; j < RPL; ++j)

@@ -63,3 +63,13 @@ def test_steps_planned_in_registers(layers, hq, hkv, d):
     """The CTA that ends last raises the lengths, while warps of other CTAs may still be about to read them."""
     rng = np.random.default_rng(layers)
     run_steps(layers, hq, hkv, d, rng.integers(1, 200, layers).tolist(), 24, layers)
+
+
+@pytest.mark.parametrize("layers,hq,hkv,d,first,steps", [
+    (4, 14, 2, 128, 120, 150),    # units of 128 rows: the kept plan is replaced on the way to 129 rows and to 257
+    (28, 28, 4, 64, 250, 20),     # whole items and pieces change places
+    (60, 16, 8, 128, 9, 40)])     # by region, units of 16 rows
+def test_steps_over_the_ends_of_units(layers, hq, hkv, d, first, steps):
+    """Where a region's unit count changes, the plan kept in the workspace fits no more: every block makes a new one and
+    keeps that, while its warps still compare the old one."""
+    run_steps(layers, hq, hkv, d, [first + i % 11 for i in range(layers)], steps, layers)
