@@ -473,8 +473,9 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     // Eq. 2 bookkeeping: the CTA that finishes last adds the appended token to every region's length
     auto finish = [&](bool all_threads) {
         if (!APPEND) return;
-        // (no thread reads lens any more, for its plan or for an item's rows, when the ticket is drawn)
-        if (all_threads) __syncthreads();
+        // (no thread reads lens any more, for its plan or for an item's rows, when the ticket is drawn; nor what the last
+        // flush left in s_last)
+        if (all_threads) __syncthreads(); else consumer_bar(NCW * 32);
         if (tid == 0) {
             __threadfence();
             s_last = atomicAdd(p.done_ticket, 1) == n_ctas - 1;

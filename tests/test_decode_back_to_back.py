@@ -73,3 +73,48 @@ def test_steps_over_the_ends_of_units(layers, hq, hkv, d, first, steps):
     """Where a region's unit count changes, the plan kept in the workspace fits no more: every block makes a new one and
     keeps that, while its warps still compare the old one."""
     run_steps(layers, hq, hkv, d, [first + i % 11 for i in range(layers)], steps, layers)
+
+
+@pytest.mark.parametrize("layers,hq,hkv,d", [
+    (80, 28, 4, 128), (112, 8, 8, 64), (90, 64, 8, 128), (200, 3, 1, 128), (70, 32, 2, 64)])
+def test_steps_over_shared_tables(layers, hq, hkv, d):
+    """More regions than the register plan takes: the tables are built ahead of the dependency wait from lengths that the
+    step before is raising, and built again where they turn out stale (some region opens a unit at every step); the
+    consumers read a region's rows as they come to it and draw the ticket at the end.  With eight KV heads a warp has a
+    head to itself and meets no other on its way."""
+    rng = np.random.default_rng(layers)
+    run_steps(layers, hq, hkv, d, rng.integers(0, 140, layers).tolist(), 40, layers)
+
+
+@pytest.mark.parametrize("layers,batch,hq,hkv,d", [(28, 4, 28, 4, 128), (30, 3, 8, 8, 64), (40, 2, 4, 1, 128)])
+def test_new_layouts_back_to_back(layers, batch, hq, hkv, d):
+    """Scores, budgets, compaction and a decode call in a row, again and again into the same cache, without a wait: the
+    decode call's tables are read early and then belong to the layout before.  Bit for bit what the same calls give with
+    a wait behind each."""
+    gen = torch.Generator(device=DEV).manual_seed(batch)
+    normal = lambda *shape: torch.randn(shape, generator=gen, device=DEV).to(torch.bfloat16)
+    nv, nt, window, rounds = 300, 20, 8, 6
+    from paper_2503_23956_b200.session import Session
+    s = Session(ac.shape(layers, batch, hq, hkv, d, nv, nt, window), 0.2, 0.9, DEV)
+    k, v = (normal(layers, batch, hkv, nv + nt, d) for _ in range(2))
+    s.set_full(k, v)
+    qw = normal(rounds, layers, batch, window, hq, d)
+    qw *= torch.linspace(0.3, 3, layers, device=DEV).to(torch.bfloat16)[:, None, None, None, None]
+    q = normal(layers, batch, hq, d)
+    results = []
+    for wait in (True, False):
+        s.k_c.zero_(), s.v_c.zero_(), s.lens.zero_(), s.offsets.zero_()
+        out = torch.empty((rounds,) + tuple(s.out.shape), device=DEV)
+        kept = torch.empty((rounds, s.kept_n), dtype=torch.int32, device=DEV)
+        torch.cuda.synchronize()
+        for i in range(rounds):
+            for call in (lambda: s.score(qw[i]), s.budget, s.compact, lambda: s.decode(q, out[i])):
+                call()
+                if wait:
+                    torch.cuda.synchronize()
+            kept[i].copy_(s.kept)
+        assert s.status() == 0
+        results.append((out, kept, s.k_c.clone(), s.lens.clone()))
+    assert not torch.equal(results[0][1][0], results[0][1][1])   # the layouts do differ
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
