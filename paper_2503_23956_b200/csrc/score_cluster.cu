@@ -423,20 +423,20 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     int hl = 0;
 #pragma unroll
                     for (int q4 = 0; q4 < 4; ++q4) {
-                        const int row_q = row0 + ew * 4 + q4;
+                        const int row_q = min(row0 + ew * 4 + q4, n_rows - 1);
                         const int before = __popc(__ballot_sync(0xffffffffu, lane < p.G && incl <= row_q));
                         if (quad == q4) hl = before;
                     }
-                    const int row = row0 + rr;
-                    const bool real = row < n_rows;
-                    if (!real) hl = 0;
-                    int kth = row - (__shfl_sync(0xffffffffu, incl, hl) - __shfl_sync(0xffffffffu, count, hl));
+                    // (the rows that fill the last four are the last one again with weight 0: zeros make NaN of a masked key's
+                    // infinities)
+                    const bool real = row0 + rr < n_rows;
+                    int kth = min(row0 + rr, n_rows - 1) - (__shfl_sync(0xffffffffu, incl, hl) - __shfl_sync(0xffffffffu, count, hl));
                     const float coef = __shfl_sync(0xffffffffu, head_coef, hl);
                     int w = 0;
                     uint4 qv[D / 64];
 #pragma unroll
                     for (int i = 0; i < D / 64; ++i) qv[i] = make_uint4(0u, 0u, 0u, 0u);
-                    if (real) {
+                    if (n_rows > 0 && row0 + rr < ((n_rows + 3) & ~3)) {
                         // the kth elite slot of the head
                         int j = 0;
                         uint32_t m = sm.mask[hl][0];
@@ -544,34 +544,45 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         const bool valid = key0 + t * 128 + own < p.Nv;
                         if (t == 0) {
 #pragma unroll
-                            for (int r = 0; r < kRows; ++r) m[r] = valid ? x[r] * p.sl2 : kNegBig;
+                            for (int r = 0; r < kRows; ++r) m[r] = valid ? fmaxf(x[r] * p.sl2, kNegBig) : kNegBig;   // (a masked key: -inf)
                         }
+                        // What is left of a logit beside the reference made from it: the rounding of the product.  (Of a masked
+                        // key's 1e29 that would be 1e21: nothing then.)
+                        auto beside = [&](float logit, float ref) {
+                            const float d = fmaf(logit, p.sl2, -ref);
+                            return fabsf(d) > 1.f && ref > kNegBig ? 0.f : d;
+                        };
                         float top = -INFINITY;
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             if (q < quads) {
 #pragma unroll
                                 for (int r = 4 * q; r < 4 * q + 4; ++r) {
-                                    x[r] = fmaf(x[r], p.sl2, -m[r]);
+                                    x[r] = t == 0 ? beside(x[r], m[r]) : fmaf(x[r], p.sl2, -m[r]);
                                     if (tail && !valid) x[r] = -INFINITY;
                                     top = fmaxf(top, x[r]);
                                 }
                             }
                         }
                         if (__any_sync(0xffffffffu, top > kRescale)) {
-                            // move the references of the rows that outgrew them and rescale what is stored
+                            // Move the references of the rows that outgrew them and rescale what is stored.  The new one is
+                            // the logit itself, read again: reference plus difference has only the bits that are left beside
+                            // the old reference, which may be a masked key's.
                             tmem_st_wait();
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
                                 if (q < quads) {
-                                    float fac[4];
+                                    float fac[4], raw[4];
+                                    tmem_ld4(base + t * kRows + 4 * q, raw);
 #pragma unroll
                                     for (int j = 0; j < 4; ++j) {
                                         const int r = 4 * q + j;
                                         const bool move = x[r] > kRescale;
-                                        fac[j] = move ? fast_exp2(-x[r]) : 1.f;
+                                        const float mn = move ? raw[j] * p.sl2 : m[r];
+                                        fac[j] = move ? fast_exp2(m[r] - mn) : 1.f;
                                         z[r] *= fac[j];
-                                        if (move) { m[r] += x[r]; x[r] = 0.f; }
+                                        if (move) x[r] = beside(raw[j], mn);
+                                        m[r] = mn;
                                     }
 #pragma unroll 1
                                     for (int t2 = 0; t2 < t; ++t2) {

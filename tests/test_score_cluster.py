@@ -81,3 +81,49 @@ def test_whole_window_at_the_edges(oracle_mod, n_visual, heads, d, window, sharp
         assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
         err = rel_elem_err(gp.scores.cpu().numpy(), ref["scores"])
         assert err <= 2e-3, err
+
+
+def masked_case(oracle_mod, edit, n_visual, window, alpha, d=128, heads=(14, 2)):
+    """Scores of a case whose keys and window queries `edit` changes, and the oracle's.  Channel 0 of every query is positive
+    and that of every key zero before: a key gets an extra logit by its channel 0."""
+    wl = Workload("masked", 2, heads[0], heads[1], d, batch=1, n_visual=n_visual, n_text=70, ratio=0.1, steps=1,
+                  window=window, alpha=alpha)
+    k, v, qw = gen_inputs(wl, "cpu")
+    qw[..., 0] = qw[..., 0].abs() + 0.125
+    k[..., 0] = 0
+    edit(k, qw)
+    scale = 1 / d ** 0.5
+    ref = oracle_mod.score(oracle_dims(oracle_mod, wl), u16(logical(k)), u16(qw), scale, alpha)
+    gp = GpuPath(wl, device=DEV)
+    gp.sh.scale = scale
+    gp.set_full(logical(k.to(DEV)), logical(v.to(DEV)))
+    gp.score(qw.to(DEV), alpha=alpha)
+    assert gp.status() == 0
+    assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
+    return gp.scores.cpu().numpy(), ref["scores"]
+
+
+@pytest.mark.parametrize("value", [float("-inf"), -3.3e38])
+@pytest.mark.parametrize("tokens", [(0, 1), (128, 131), (5, 290)])
+@pytest.mark.parametrize("n_visual,window,alpha", [(300, 16, 0.9), (300, 2, 0.0), (3000, 16, 0.3)])
+def test_masked_keys(oracle_mod, value, tokens, n_visual, window, alpha):
+    """Keys that no query attends to (a channel of minus infinity, or so low that the logit overflows) score zero, also where
+    such a key is the first that a thread meets, and the others score what they do without them."""
+    def edit(k, qw):
+        k[:, :, tokens[0]:tokens[1], :, 0] = value
+    got, want = masked_case(oracle_mod, edit, n_visual, window, alpha)
+    assert (want[..., tokens[0]:tokens[1]] == 0).all() and (want > 0).any()
+    assert rel_elem_err(got, want) <= 2e-3
+
+
+@pytest.mark.parametrize("low", [-1e30, -1e6, -1500.0])
+@pytest.mark.parametrize("n_visual,window,alpha", [(300, 16, 0.9), (3000, 16, 0.9), (3000, 64, 0.2), (5000, 2, 0.0)])
+def test_references_far_below(oracle_mod, low, n_visual, window, alpha):
+    """The first key of every thread far below the others, so that its logit is no reference for them: the one that takes its
+    place has to be exact beside it.  Logits up to 12 in magnitude otherwise: their rounding in 32 bits and that of a sum
+    of 128 products is 2e-6 of a score; 2e-5 leaves room for the exponentials and the sums over keys."""
+    def edit(k, qw):
+        for tile in range(0, n_visual, 2048):
+            k[:, :, tile:min(tile + 128, n_visual), :, 0] = low
+    got, want = masked_case(oracle_mod, edit, n_visual, window, alpha)
+    assert rel_elem_err(got, want) <= 2e-5
