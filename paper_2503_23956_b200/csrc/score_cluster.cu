@@ -51,6 +51,7 @@ constexpr int kEliteThreads = 128, kEpiThreads = 128;
 constexpr int kEliteWarp0 = 4, kEpiWarp0 = 8;
 constexpr int kSmemPerBlock = (228 * 1024) / 2 - 1024;   // two blocks per SM, 1 KB each is the system's
 constexpr float kRescale = 24.f;
+constexpr float kScaleUp = 18446744073709551616.f;   // 2^64
 constexpr int kPreloadRows = 128;     // window queries of a group that fit a ring stage
 constexpr int kFirstAhead = 5;        // tiles asked into L2 behind the first full ring
 
@@ -672,8 +673,13 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     if (lane == 0) mbar_arrive(smem_u32(&sm.meta_empty[par]));
 #pragma unroll
                     for (int r = 0; r < kRows; ++r) {
+                        // 2^64 times the factor: where a thread's reference is 2^126 below the row's maximum, its keys may still
+                        // be 2^24 above the reference and their scores in range.  (Exact: powers of two, and the sum in the
+                        // exponent loses no bits where it is taken.)
                         const float2 f = sm.fin[ew][r];
-                        m[r] = f.y * fast_exp2(m[r] - f.x);
+                        const float below = m[r] - f.x;
+                        const bool far = below < -100.f;
+                        m[r] = f.y * (fast_exp2(far ? below + 64.f : below) * (far ? 1.f : kScaleUp));
                     }
                     __syncwarp();
 
@@ -694,7 +700,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         if (key < p.Nv) {
                             // (added where it lies: one thread owns the key, so the order of the sum is the program's,
                             // and nobody waits for the old value)
-                            const float v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                            const float v = ((acc[0] + acc[1]) + (acc[2] + acc[3])) * (1.f / kScaleUp);
                             if (add) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(out + key), "f"(v) : "memory");
                             else out[key] = v;
                         }

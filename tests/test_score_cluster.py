@@ -127,3 +127,31 @@ def test_references_far_below(oracle_mod, low, n_visual, window, alpha):
             k[:, :, tile:min(tile + 128, n_visual), :, 0] = low
     got, want = masked_case(oracle_mod, edit, n_visual, window, alpha)
     assert rel_elem_err(got, want) <= 2e-5
+
+
+@pytest.mark.parametrize("n_visual", [300, 3000, 9000])
+@pytest.mark.parametrize("window,alpha", [(16, 0.9), (2, 0.0)])
+def test_scores_near_the_smallest(oracle_mod, n_visual, window, alpha):
+    """Keys of 2^-104 of the largest weight, met by threads whose reference is 2^-127 of it: such a reference's own factor is
+    below the smallest 32-bit number, the scores are not (5e-32), and a ranking of the tokens depends on them.  The oracle
+    is compared above 1e-30 only, so the error of these scores is taken relative to themselves."""
+    unit = np.log(2) * 128 ** 0.5   # a logit of 1 in the log2 domain, in two channels for the bits
+
+    def put(k, tokens, x):
+        hi = torch.tensor(x * unit).to(torch.bfloat16)
+        k[:, :, tokens, :, 0] = hi
+        k[:, :, tokens, :, 1] = (torch.tensor(x * unit) - hi.double()).to(torch.bfloat16)
+
+    def edit(k, qw):
+        k.zero_()
+        qw.zero_()
+        qw[..., :2] = 1.0
+        put(k, slice(0, n_visual), -104.0)
+        for tile in range(0, n_visual, 384):
+            put(k, slice(tile, min(tile + 128, n_visual)), -127.0)
+        put(k, 10, 0.0)
+        put(k, slice(n_visual, None), -30.0)
+    got, want = masked_case(oracle_mod, edit, n_visual, window, alpha)
+    small = want > 2.0 ** -120
+    assert small.sum() > want.size // 2
+    assert (np.abs(got - want)[small] / want[small]).max() <= 2e-5
