@@ -2,7 +2,7 @@
 // layer-wise budget of Eq. 11 turned into integer row counts, and the row offsets of the ragged cache.
 //
 // One launch.  Every CTA reduces one cell (fp64 block reductions over the fp32 scores, which it keeps in registers:
-// sum; then squared and cubed deviations together; fixed reduction tree).  The
+// sum; then squared and cubed deviations together; one reduction tree for all block sizes).  The
 // CTA that finishes a SEQUENCE last (one ticket per sequence in the workspace, put back to zero for the next
 // call) runs that sequence's allocation with one warp: sums over the cells taken by one lane in cell order
 // and every fp64 operation individually rounded (no fused multiply-add), so that the integer budgets are
@@ -36,25 +36,38 @@ struct BudgetParams {
     long long first_row;     // rows of the shared buffers in front of this cache's first region
 };
 
-// Sums of v[0 .. N-1] over the block's T threads, the same in all of them.  s_part: N * 32 doubles, free again at the
-// next use with the other half of it (parity).
+// The sums run over kSlots slots, token i in slot i % kSlots, whatever the block size T: a thread holds kSlots / T slots
+// that lie side by side, and the tree over the slots is the same one (neighbours first), so that a sequence's sums have
+// the same bits in a call of its own and in a batch.
+constexpr int kSlots = 1024;
+
+// Sums of v[0 .. N-1] over the slots, the same in all threads.  s_part: N * 32 doubles.
 template <int T, int N>
-__device__ __forceinline__ void block_sums(double (&v)[N], double (*s_part)[32]) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__device__ __forceinline__ void block_sums(double (&v)[N][kSlots / T], double (&sum)[N], double (*s_part)[32]) {
+    constexpr int S = kSlots / T, LANES = 32 / S;   // lanes that hold 32 slots
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int sh = 16; sh > 0; sh >>= 1)
+    for (int i = 0; i < N; ++i) {
 #pragma unroll
-        for (int i = 0; i < N; ++i) v[i] = __dadd_rn(v[i], __shfl_xor_sync(0xffffffffu, v[i], sh));
-    if (lane == 0)
+        for (int n = S; n > 1; n >>= 1)
 #pragma unroll
-        for (int i = 0; i < N; ++i) s_part[i][warp] = v[i];
+            for (int j = 0; j < n / 2; ++j) v[i][j] = __dadd_rn(v[i][2 * j], v[i][2 * j + 1]);
+        sum[i] = v[i][0];
+    }
+#pragma unroll
+    for (int sh = 1; sh < LANES; sh <<= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) sum[i] = __dadd_rn(sum[i], __shfl_xor_sync(0xffffffffu, sum[i], sh));
+    if (lane % LANES == 0)
+#pragma unroll
+        for (int i = 0; i < N; ++i) s_part[i][threadIdx.x / LANES] = sum[i];
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < N; ++i) v[i] = lane < T / 32 ? s_part[i][lane] : 0.0;
+    for (int i = 0; i < N; ++i) sum[i] = s_part[i][lane];
 #pragma unroll
     for (int sh = 16; sh > 0; sh >>= 1)
 #pragma unroll
-        for (int i = 0; i < N; ++i) v[i] = __dadd_rn(v[i], __shfl_xor_sync(0xffffffffu, v[i], sh));
+        for (int i = 0; i < N; ++i) sum[i] = __dadd_rn(sum[i], __shfl_xor_sync(0xffffffffu, sum[i], sh));
 }
 
 __device__ __forceinline__ unsigned ticket_add(uint32_t *t) {   // what the block wrote before it is seen with it
@@ -180,30 +193,35 @@ __global__ void __launch_bounds__(T, 1024 / T) budget_kernel(BudgetParams p) {
     {
         const float *x = p.scores + (int64_t)blockIdx.x * p.Nv;
         const double n = (double)p.Nv;
+        constexpr int S = kSlots / T;
+        auto token = [&](int k) { return k / S * kSlots + tid * S + k % S; };   // of the thread's k-th score, in slot k % S
         float f[PER];
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int i = tid + k * T;
-            f[k] = i < p.Nv ? __ldg(x + i) : 0.f;
-        }
-        double sum[1] = {0.0};
+        for (int k = 0; k < PER; ++k) f[k] = token(k) < p.Nv ? __ldg(x + token(k)) : 0.f;
+        double slot[1][S] = {}, sum[1];
 #pragma unroll
-        for (int k = 0; k < PER; ++k) sum[0] = __dadd_rn(sum[0], (double)f[k]);
-        for (int i = tid + PER * T; i < p.Nv; i += T) sum[0] = __dadd_rn(sum[0], (double)__ldg(x + i));   // (more than fit)
-        block_sums<T, 1>(sum, s_part);
+        for (int k = 0; k < PER; ++k) slot[0][k % S] = __dadd_rn(slot[0][k % S], (double)f[k]);
+        for (int i = token(PER); i < p.Nv; i += kSlots)   // (more than fit)
+#pragma unroll
+            for (int j = 0; j < S; ++j)
+                if (i + j < p.Nv) slot[0][j] = __dadd_rn(slot[0][j], (double)__ldg(x + i + j));
+        block_sums<T, 1>(slot, sum, s_part);
         const double mu = __ddiv_rn(sum[0], n);
 
-        double dev[2] = {0.0, 0.0};   // sums of the squared and the cubed deviations
-        auto add = [&](double xi) {
+        double dslot[2][S] = {}, dev[2];   // sums of the squared and the cubed deviations
+        auto add = [&](int j, double xi) {
             const double c = __dsub_rn(xi, mu), c2 = __dmul_rn(c, c);
-            dev[0] = __dadd_rn(dev[0], c2);
-            dev[1] = __fma_rn(c2, c, dev[1]);
+            dslot[0][j] = __dadd_rn(dslot[0][j], c2);
+            dslot[1][j] = __fma_rn(c2, c, dslot[1][j]);
         };
 #pragma unroll
         for (int k = 0; k < PER; ++k)
-            if (tid + k * T < p.Nv) add((double)f[k]);
-        for (int i = tid + PER * T; i < p.Nv; i += T) add((double)__ldg(x + i));
-        block_sums<T, 2>(dev, s_part + 1);
+            if (token(k) < p.Nv) add(k % S, (double)f[k]);
+        for (int i = token(PER); i < p.Nv; i += kSlots)
+#pragma unroll
+            for (int j = 0; j < S; ++j)
+                if (i + j < p.Nv) add(j, (double)__ldg(x + i + j));
+        block_sums<T, 2>(dslot, dev, s_part + 1);
         if (tid == 0) {
             const double sigma = __dsqrt_rn(__ddiv_rn(dev[0], __dsub_rn(n, 1.0)));
             const double pre = __ddiv_rn(n, __dmul_rn(__dsub_rn(n, 1.0), __dsub_rn(n, 2.0)));

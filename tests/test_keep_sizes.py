@@ -37,3 +37,24 @@ def test_budget_and_selection(oracle_mod, layers, batch, n_visual):
     flat, k = scores.reshape(-1, n_visual), bud.reshape(-1)
     want = [np.sort(np.argsort(-flat[i], kind="stable")[:k[i]]) for i in range(len(k))]
     assert np.array_equal(gp.kept.cpu().numpy()[:int(k.sum())], np.concatenate(want))
+
+
+@pytest.mark.parametrize("n_visual", [3, 40, 2916, 4097, 8193, 16385])
+def test_a_sequence_alone_and_in_a_batch(n_visual):
+    """Strength, skewness and budgets of a sequence do not depend, to the last bit, on how many sequences share the call (the
+    kernel takes smaller blocks for many cells)."""
+    layers, batch = 19, 24
+    gen = torch.Generator(device=DEV).manual_seed(n_visual)
+    scores = torch.exp(2 * torch.randn((layers, batch, n_visual), generator=gen, device=DEV))
+    results = []
+    for seqs in (list(range(batch)), [0], [5], [7, 23]):
+        wl = Workload("alone", layers, 1, 1, 64, batch=len(seqs), n_visual=n_visual, n_text=2, ratio=0.23, steps=1, window=2)
+        gp = GpuPath(wl, device=DEV)
+        gp.budget(scores=scores[:, seqs].contiguous())
+        assert gp.status() == 0
+        got = (gp.strength.view(torch.int64), gp.skew.view(torch.int64), gp.budgets)
+        if results:
+            for a, b in zip(results, got):
+                assert torch.equal(a[:, seqs], b)
+        else:
+            results = got
