@@ -108,16 +108,29 @@ def exported_symbols() -> list[str]:
     return list(_SIGNATURES)
 
 
-_native = None   # (module, addresses of aircache_decode_attn and aircache_decode_step) once CUDA is up
+_native = None   # (module, addresses of aircache_decode_attn and aircache_decode_step) once CUDA is up; False: not to be had
+
+# torch's current device and the raw handle of its current stream: names that torch keeps to itself, hence looked up once
+# and done without where they are missing
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _per_token_calls():
-    """The native marshalling of the per-token entry points (csrc/binding.c); None while CUDA is not initialised (there
-    is no current stream to ask for then)."""
+    """The native marshalling of the per-token entry points (csrc/binding.c).  None while CUDA is not initialised (there is no
+    current stream to ask for then), False where the extension cannot be loaded (built for another Python, or not built:
+    it needs Python.h): ctypes then hands over the same arguments to the same functions, 2 us a call later."""
     global _native
     if _native is None and torch.cuda.is_initialized():
-        from . import _binding
-        _binding.setup(Shape, Ragged, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        try:
+            from . import _binding
+        except ImportError:
+            _native = False
+            return _native
+        if _raw_device is None or _raw_stream is None:
+            _native = False
+            return _native
+        _binding.setup(Shape, Ragged, _raw_device, _raw_stream)
         handle = lib()
         _native = (_binding, C.cast(handle.aircache_decode_attn, C.c_void_p).value,
                    C.cast(handle.aircache_decode_step, C.c_void_p).value)
@@ -137,10 +150,10 @@ def _ptr(t) -> int | None:
 
 def _stream(stream) -> int | None:
     if stream is None:
-        if torch.cuda.is_initialized():
+        if _raw_device is not None and _raw_stream is not None and torch.cuda.is_initialized():
             # the raw handle: torch.cuda.current_stream() builds a Stream object around it first (3.4 against 0.4 us
             # per call of an entry point whose kernel may take 5)
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
+            return _raw_stream(_raw_device()) or None
         stream = torch.cuda.current_stream()
     if isinstance(stream, int):
         return stream or None
@@ -233,9 +246,14 @@ def aircache_compact(sh, full, scores, budgets, ratio, out, kept_idx, workspace,
 
 def aircache_decode_attn(sh, cache, q, out, workspace, stream=None, check=True) -> int:
     native = _native or _per_token_calls()
+    rc = None
     if native:
-        rc = native[0].decode_attn(native[1], sh, cache, q, out, workspace, stream)
-    else:
+        try:
+            rc = native[0].decode_attn(native[1], sh, cache, q, out, workspace, stream)
+        except TypeError:   # (before the call) perhaps an argument of a kind that only ctypes takes
+            if not (isinstance(sh, Shape) and isinstance(cache, Ragged)):
+                raise
+    if rc is None:
         rc = lib().aircache_decode_attn(C.byref(sh), C.byref(cache), _ptr(q), _ptr(out), _ptr(workspace),
                                         _nbytes(workspace), _stream(stream))
     if check:
@@ -245,9 +263,14 @@ def aircache_decode_attn(sh, cache, q, out, workspace, stream=None, check=True) 
 
 def aircache_decode_step(sh, cache, q, k_new, v_new, appended, out, workspace, stream=None, check=True) -> int:
     native = _native or _per_token_calls()
+    rc = None
     if native:
-        rc = native[0].decode_step(native[2], sh, cache, q, k_new, v_new, appended, out, workspace, stream)
-    else:
+        try:
+            rc = native[0].decode_step(native[2], sh, cache, q, k_new, v_new, appended, out, workspace, stream)
+        except TypeError:
+            if not (isinstance(sh, Shape) and isinstance(cache, Ragged)):
+                raise
+    if rc is None:
         rc = lib().aircache_decode_step(C.byref(sh), C.byref(cache), _ptr(q), _ptr(k_new), _ptr(v_new), appended,
                                         _ptr(out), _ptr(workspace), _nbytes(workspace), _stream(stream))
     if check:

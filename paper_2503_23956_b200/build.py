@@ -31,15 +31,20 @@ def stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build_binding(force: bool = False) -> str:
-    """Compile the native argument marshalling of the per-token calls (csrc/binding.c) next to this file."""
+def build_binding(force: bool = False) -> str | None:
+    """Compile the native argument marshalling of the per-token calls (csrc/binding.c) next to this file.  Without it (no C
+    compiler, no Python.h) those calls go through ctypes: None then, with a word on why."""
     if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= os.path.getmtime(BINDING_SOURCE):
         return BINDING
     tmp = BINDING + f".tmp{os.getpid()}"
     cc = os.environ.get("CC") or shutil.which("gcc") or shutil.which("cc")
-    if not cc:
-        raise RuntimeError("no C compiler found: the binding cannot be built")
-    subprocess.check_call([cc, "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], BINDING_SOURCE, "-o", tmp])
+    try:
+        if not cc:
+            raise OSError("no C compiler found")
+        subprocess.check_call([cc, "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], BINDING_SOURCE, "-o", tmp])
+    except (OSError, subprocess.CalledProcessError) as e:
+        print(f"the native marshalling is not built ({e}): the per-token calls go through ctypes", file=sys.stderr)
+        return None
     os.replace(tmp, BINDING)
     return BINDING
 

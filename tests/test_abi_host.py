@@ -188,3 +188,69 @@ def test_native_marshalling_of_the_per_token_calls(monkeypatch):
     with pytest.raises(TypeError):
         ac.aircache_decode_attn(cache, cache, P, P, P, stream=0)
     monkeypatch.setattr(ac, "_native", None)   # (set up again, with torch's functions, at the next call)
+
+
+class _Tensor:
+    """What the binding asks of a tensor, with a word's worth of nothing behind it."""
+
+    def __init__(self, ptr=0x10000000, n=16):
+        self.ptr, self.n = ptr, n
+
+    def data_ptr(self):
+        return self.ptr
+
+    def numel(self):
+        return self.n
+
+    def element_size(self):
+        return 1
+
+
+def _per_token(sh, cache, **kw):
+    """Return codes of both calls with a workspace that is too small: the last of the host-side checks."""
+    t = _Tensor()
+    return (ac.aircache_decode_attn(sh, cache, t, t, t, check=False, **kw),
+            ac.aircache_decode_step(sh, cache, t, t, t, 1, t, t, check=False, **kw))
+
+
+def test_without_the_native_marshalling(monkeypatch):
+    """Where the extension was not built, or for another Python, or torch keeps its stream elsewhere, the per-token calls go
+    through ctypes; nothing is refused that was taken before there was an extension."""
+    import sys
+    from paper_2503_23956_b200 import _binding
+    sh = ac.shape(2, 1, 4, 2, 64, 16, 8, 4, slack=2)
+    P = 0x10000000
+    cache = ac.Ragged(P, P, P, P, 100, 0)
+    want = (ac.ERR_WORKSPACE_TOO_SMALL,) * 2
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(ac, "_native", None)
+    with monkeypatch.context() as m:   # the extension is missing
+        m.setitem(sys.modules, "paper_2503_23956_b200._binding", None)
+        m.delattr(ac, "_binding", raising=False)
+        assert _per_token(sh, cache, stream=0) == want
+        assert ac._native is False
+    monkeypatch.setattr(ac, "_native", None)
+    with monkeypatch.context() as m:   # torch's own names are missing: the public ones are asked
+        m.setattr(ac, "_raw_stream", None)
+        m.setattr(torch.cuda, "current_stream", lambda: type("S", (), {"cuda_stream": 0})())
+        assert _per_token(sh, cache) == want
+        assert ac._native is False
+    # with the extension: kinds of argument that ctypes alone takes
+    _binding.setup(ac.Shape, ac.Ragged, lambda: 0, lambda dev: 0)
+    monkeypatch.setattr(ac, "_native", (_binding, *(C.cast(f, C.c_void_p).value for f in (
+        ac.lib().aircache_decode_attn, ac.lib().aircache_decode_step))))
+    t = _Tensor()
+    assert ac.aircache_decode_step(sh, cache, t, t, t, C.c_int32(1), t, t, stream=0, check=False) == want[0]
+    assert _per_token(sh, cache, stream=type("S", (), {"cuda_stream": None})()) == want
+    assert ac.aircache_decode_attn(sh, cache, _Tensor(None), t, t, stream=0, check=False) == ac.ERR_INVALID_ARG
+    with pytest.raises(C.ArgumentError):
+        ac.aircache_decode_step(sh, cache, t, t, t, 1.5, t, t, stream=0)
+    monkeypatch.setattr(ac, "_native", None)
+
+
+def test_building_without_a_c_compiler(monkeypatch, tmp_path, capsys):
+    from paper_2503_23956_b200 import build
+    monkeypatch.setattr(build, "BINDING", str(tmp_path / "_binding.so"))
+    monkeypatch.setenv("CC", "/nonexistent/cc")
+    assert build.build_binding() is None
+    assert "through ctypes" in capsys.readouterr().err
