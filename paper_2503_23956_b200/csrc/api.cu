@@ -24,6 +24,29 @@ int current_device(int *dev, int *sms) {
     return AIRCACHE_OK;
 }
 
+uint64_t context_id() {
+    typedef CUresult (*GetIdFn)(CUcontext, unsigned long long *);
+    static const GetIdFn get_id = []() -> GetIdFn {
+        void *ptr = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuCtxGetId", &ptr, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            return nullptr;
+        return reinterpret_cast<GetIdFn>(ptr);
+    }();
+    unsigned long long id = 0;
+    return get_id && get_id(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+int allow_shared_memory(const void *kernel, int bytes, int dev, std::atomic<uint64_t> (&done_for)[kMaxDevices]) {
+    const bool known = dev >= 0 && dev < kMaxDevices;
+    const uint64_t id = context_id();
+    if (known && id != 0 && done_for[dev].load(std::memory_order_acquire) == id) return AIRCACHE_OK;
+    AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    if (known) done_for[dev].store(id, std::memory_order_release);
+    return AIRCACHE_OK;
+}
+
 int check_shape(const aircache_shape_t *s) {
     if (!s) return AIRCACHE_ERR_INVALID_ARG;
     if (s->n_layers < 1 || s->batch < 1 || s->n_q_heads < 1 || s->n_kv_heads < 1 || s->head_dim < 1 ||

@@ -301,12 +301,9 @@ __global__ void __launch_bounds__(T, 1024 / T) budget_kernel(BudgetParams p) {
 
 template <int T, int PER>
 int launch_budget_t(const BudgetParams &p, int cells, int dev, cudaStream_t st) {
-    // the shared-memory limit is a property of the kernel on a device: set once for each
-    static std::atomic<bool> ready[kMaxDevices];
-    if (dev >= kMaxDevices || !ready[dev].load(std::memory_order_acquire)) {
-        AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(budget_kernel<T, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-        if (dev < kMaxDevices) ready[dev].store(true, std::memory_order_release);
-    }
+    static std::atomic<uint64_t> allowed[kMaxDevices];
+    const int rc = allow_shared_memory((const void *)budget_kernel<T, PER>, 96 * 1024, dev, allowed);
+    if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cells);
     cfg.blockDim = dim3(T);

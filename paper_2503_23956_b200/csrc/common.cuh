@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/aircache.h"
 
 namespace aircache {
@@ -57,6 +59,12 @@ void set_last_cuda_error(cudaError_t e);
 // ---------------------------------------------------------------------------------------------
 // The current device and its number of SMs, asked once per device (the answer never changes).
 int current_device(int *dev, int *sms);
+// The id of the current context, which no other one of the process gets; 0 when there is none yet.  What belongs to a
+// context (a kernel's shared-memory limit, a variable's address) is kept under it, since cudaDeviceReset ends the
+// context and the program may go on with a new one.
+uint64_t context_id();
+// Lets a kernel use `bytes` of dynamic shared memory, once per context; done_for: the kernel's own, by device.
+int allow_shared_memory(const void *kernel, int bytes, int dev, std::atomic<uint64_t> (&done_for)[kMaxDevices]);
 int check_shape(const aircache_shape_t *s);
 int check_full(const aircache_shape_t *s, const aircache_full_t *f);
 int64_t kept_per_sequence(const aircache_shape_t *s, double ratio);

@@ -1199,13 +1199,8 @@ int launch_decode_a(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, c
     int dev = 0, sms = 0;
     if ((rc = current_device(&dev, &sms))) return rc;
     const int ctas = sms < kMaxDecodeCtas ? sms : kMaxDecodeCtas;
-    // the shared-memory limit is a property of the kernel on a device: set once for each
-    static std::atomic<bool> ready[kMaxDevices];
-    if (dev >= kMaxDevices || !ready[dev].load(std::memory_order_acquire)) {
-        AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, HKV, G_HI, HS, APPEND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               C::SMEM_BYTES));
-        if (dev < kMaxDevices) ready[dev].store(true, std::memory_order_release);
-    }
+    static std::atomic<uint64_t> allowed[kMaxDevices];
+    if ((rc = allow_shared_memory((const void *)decode_kernel<D, HKV, G_HI, HS, APPEND>, C::SMEM_BYTES, dev, allowed))) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(C::THREADS);
@@ -1319,6 +1314,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[AIRCACHE_STATIC_
 namespace {
 std::mutex g_static_mutex;
 unsigned char *g_static_ptr[kMaxDevices] = {};
+uint64_t g_static_context[kMaxDevices] = {};   // the context that the address belongs to
 }  // namespace
 
 int launch_decode_static(const aircache_shape_t *s, const aircache_ragged_t *c, const void *q, float *out,
@@ -1333,12 +1329,14 @@ int launch_decode_static(const aircache_shape_t *s, const aircache_ragged_t *c, 
     unsigned char *base = nullptr;
     {
         // In host code the array's name is only a handle; its device address on the current device comes
-        // from the runtime, once per device.
+        // from the runtime, once per context.
         std::lock_guard<std::mutex> lock(g_static_mutex);
-        if (!g_static_ptr[dev]) {
+        const uint64_t id = context_id();
+        if (!g_static_ptr[dev] || id == 0 || g_static_context[dev] != id) {
             void *ptr = nullptr;
             AIRCACHE_CUDA_TRY(cudaGetSymbolAddress(&ptr, g_static_scratch));
             g_static_ptr[dev] = static_cast<unsigned char *>(ptr);
+            g_static_context[dev] = context_id();
         }
         base = g_static_ptr[dev];
     }

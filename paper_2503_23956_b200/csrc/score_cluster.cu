@@ -735,10 +735,14 @@ const int *clusters_at_once(int smem) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
     const int st = smem / ClusterCfg<D>::TILE_BYTES > kMaxStages ? kMaxStages : smem / ClusterCfg<D>::TILE_BYTES;
+    static std::atomic<uint64_t> allowed[kMaxDevices];
+    if (allow_shared_memory((const void *)score_cluster_kernel<D>, kSmemPerBlock, dev, allowed)) {
+        cudaGetLastError();
+        return nullptr;
+    }
     std::lock_guard<std::mutex> guard(lock);
     if (!have[dev][st]) {
-        if (cudaFuncSetAttribute(score_cluster_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock) != cudaSuccess ||
-            cudaFuncSetAttribute(cluster_room_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock) != cudaSuccess) {
+        if (cudaFuncSetAttribute(cluster_room_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }

@@ -450,12 +450,9 @@ int choose_pieces(int64_t items, int tiles, int steps, int blocks, int most, dou
 
 template <int D, int PASS>
 int launch_pass(const CUtensorMap &tk, const CUtensorMap &tq, const ScoreParams &p, const DensePlan &plan, int dev, int64_t pieces, cudaStream_t st) {
-    // the shared-memory limit is a property of the kernel on a device: set once for each
-    static std::atomic<bool> ready[kMaxDevices];
-    if (dev >= kMaxDevices || !ready[dev].load(std::memory_order_acquire)) {
-        AIRCACHE_CUDA_TRY(cudaFuncSetAttribute(dense_kernel<D, PASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseCfg<D>::SMEM));
-        if (dev < kMaxDevices) ready[dev].store(true, std::memory_order_release);
-    }
+    static std::atomic<uint64_t> allowed[kMaxDevices];
+    const int rc = allow_shared_memory((const void *)dense_kernel<D, PASS>, DenseCfg<D>::SMEM, dev, allowed);
+    if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(pieces < plan.blocks ? pieces : plan.blocks));
     cfg.blockDim = dim3(kDenseThreads);
