@@ -801,7 +801,7 @@ int launch_group_sum(const ScoreParams &p, cudaStream_t st) {
 int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void *q_window, float alpha,
                  int layer_begin, int layer_count, float *scores, uint64_t *elite_mask, void *ws, cudaStream_t st) {
     const WsLayout w = ws_layout(s);
-    ScoreParams p;
+    ScoreParams p = {};
     p.k = (const uint16_t *)f->k;
     p.s_layer = f->stride_layer; p.s_batch = f->stride_batch; p.s_head = f->stride_head; p.s_token = f->stride_token;
     p.qw = (const uint16_t *)q_window;
@@ -817,28 +817,12 @@ int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void
     p.dispatch = ws_ptr<uint32_t>(ws, w.dispatch);
     p.imp_part = ws_ptr<float>(ws, w.imp_part);
     p.q_block = ws_ptr<uint16_t>(ws, w.q_block);
-    // A call over few KV groups (a layer at a time, a single short sequence) would leave SMs idle with 512- and
-    // 1024-key blocks: while the blocks would fill less than half of the GPU, they take half the tiles per warp,
-    // down to 256 keys per block (config 4 a layer at a time: 41 -> 33 us per layer).
-    {
-        const int resident = s->head_dim == 64 ? onepass_resident_blocks<64>() : onepass_resident_blocks<128>();
-        const int64_t groups = (int64_t)layer_count * s->batch * s->n_kv_heads;
-        auto numbers_per_group = [&](int cap) { const int k = 64 * (cap < 8 ? cap : 8); return (s->n_visual + k - 1) / k; };
-        p.op_tile_cap = 16;
-        while (p.op_tile_cap > 4 &&
-               groups * ((s->n_visual + 64 * p.op_tile_cap - 1) / (64 * p.op_tile_cap)) * 2 < (int64_t)resident &&
-               (int64_t)numbers_per_group(p.op_tile_cap / 2) * 2 <= resident)
-            p.op_tile_cap >>= 1;
-        p.op_chunks = numbers_per_group(p.op_tile_cap);
-    }
     p.L = s->n_layers; p.B = s->batch; p.Hq = s->n_q_heads; p.Hkv = s->n_kv_heads;
     p.G = s->n_q_heads / s->n_kv_heads; p.d = s->head_dim; p.Nv = s->n_visual; p.Nt = s->n_text; p.W = s->window;
     p.per_head = s->per_kv_head;
     p.lb0 = layer_begin * s->batch;
     p.n_lb = layer_count * s->batch;
     p.cap = score_row_cap(s);
-    p.chunks = score_chunks(s->n_visual, (int64_t)layer_count * s->batch * s->n_kv_heads);
-    p.chunk_keys = (int)align_up((s->n_visual + p.chunks - 1) / p.chunks, 16);
     p.scale = s->scale;
     p.sl2 = s->scale * kLog2e;
     p.keep_all = alpha <= 0.0f;
@@ -847,11 +831,26 @@ int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void
     p.pos_token = p.pos_head = p.pos_batch = p.pos_layer = 0;
     p.status = ws_ptr<uint32_t>(ws, w.status);
 
-    // alpha = 0 with more than a cluster's two query blocks keeps the tensor cores and the exponentials busy by itself
+    // alpha = 0 with at least a cluster's two query blocks keeps the tensor cores and the exponentials busy by itself
     int taken = 0;
     const int rc = p.keep_all && p.G * p.W >= 32 ? launch_score_dense(p, s, f, st, &taken) : launch_score_cluster(p, s, f, st, &taken);
     if (rc || taken) return rc;
+
+    // What the remaining kernels need.  A call over few KV groups (a layer at a time, a single sequence) would leave SMs
+    // idle with 512- and 1024-key blocks of the one-pass kernel: while the blocks would fill less than half of the GPU,
+    // they take half the tiles per warp, down to 256 keys per block (four sequences of 6272 tokens, a layer at a time, when
+    // this kernel still took them: 41 -> 33 us per layer).
+    const int resident = s->head_dim == 64 ? onepass_resident_blocks<64>() : onepass_resident_blocks<128>();
     const int64_t groups = (int64_t)p.n_lb * p.Hkv;
+    auto numbers_per_group = [&](int cap) { const int k = 64 * (cap < 8 ? cap : 8); return (s->n_visual + k - 1) / k; };
+    p.op_tile_cap = 16;
+    while (p.op_tile_cap > 4 &&
+           groups * ((s->n_visual + 64 * p.op_tile_cap - 1) / (64 * p.op_tile_cap)) * 2 < (int64_t)resident &&
+           (int64_t)numbers_per_group(p.op_tile_cap / 2) * 2 <= resident)
+        p.op_tile_cap >>= 1;
+    p.op_chunks = numbers_per_group(p.op_tile_cap);
+    p.chunks = score_chunks(s->n_visual, groups);
+    p.chunk_keys = (int)align_up((s->n_visual + p.chunks - 1) / p.chunks, 16);
     const size_t elite_smem = (size_t)(p.W + p.G) * (p.d + 8) * 2;
     if (p.keep_all) {
         if (s->head_dim == 64) elite_kernel<64, true><<<(unsigned)groups, 128, elite_smem, st>>>(p);
@@ -862,7 +861,6 @@ int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void
     }
     AIRCACHE_LAUNCH_CHECK();
     // one pass over the keys, if a group's blocks are sure to be resident together
-    const int resident = s->head_dim == 64 ? onepass_resident_blocks<64>() : onepass_resident_blocks<128>();
     if ((int64_t)p.op_chunks * 2 <= resident && (int64_t)p.n_lb * p.Hkv * p.op_chunks < ((int64_t)1 << 31))
         return s->head_dim == 64 ? launch_onepass<64>(p, st) : launch_onepass<128>(p, st);
     return s->head_dim == 64 ? launch_passes_d<64>(p, st) : launch_passes_d<128>(p, st);
