@@ -60,6 +60,7 @@ struct DecodeParams {
     int32_t *lens_rw;                // lens, bumped by the last CTA when a token is appended
     int32_t *done_ticket;            // CTAs finished (append only); zero between calls
     int kv_heads;                    // KV heads of the cache
+    int early;               // many regions: the tables are built ahead of the dependency wait
     int hs;                  // head-split mode: KV heads per region (items are (region, head) pairs); else 1
     float sl2;               // scale * log2(e)
 };
@@ -487,14 +488,16 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     };
 
     // ---- the tables: unit prefix and first row of all regions (every CTA computes the same), and the schedule ----
-    auto build_tables = [&]() {
+    auto build_tables = [&](bool late) {
+        // (ahead of the wait around L1, which would keep what is read then)
+        auto rows_of = [&](int i) { return max(late ? p.lens[i / hs] : __ldcg(p.lens + i / hs), 0) + appended; };
         {
             const int per = (n + C::THREADS - 1) / C::THREADS;
             const int i0 = min(n, tid * per), i1 = min(n, i0 + per);
             int local = 0;
             for (int i = i0; i < i1; ++i) {
-                local += (max(__ldcg(p.lens + i / hs), 0) + appended + CH - 1) / CH;
-                s_off[i] = (int)__ldcg(p.offsets + i / hs);
+                local += (rows_of(i) + CH - 1) / CH;
+                s_off[i] = (int)(late ? p.offsets[i / hs] : __ldcg(p.offsets + i / hs));
             }
             s_part[tid] = local;
             __syncthreads();
@@ -522,7 +525,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             int run = s_part[tid];
             for (int i = i0; i < i1; ++i) {
                 s_P[i] = run;
-                run += (max(__ldcg(p.lens + i / hs), 0) + appended + CH - 1) / CH;
+                run += (rows_of(i) + CH - 1) / CH;
             }
             if (i1 == n && i0 < n) s_P[n] = run;
             if (n == 0 && tid == 0) s_P[0] = 0;
@@ -636,11 +639,13 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     // usually the right ones - and checked against what is read behind it.  With them the CTA asks for its first units'
     // lines to be brought into L2: a hint that consumes no value, kept inside the cache whatever was read.  (What is
     // read early goes around L1.)  Four requests of 1100 rows in 28 layers: 49.0 us a call with the tables built behind the
-    // wait, 47.8 with them built before it, 46.3 with the hint as well.
+    // wait, 47.8 with them built before it, 46.3 with the hint as well.  (p.early: worth it unless the call is little
+    // else, see the launcher.)
     const bool tables = !planned;
+    if (!few && !p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll 1
-    for (int pass = few ? 1 : 0; pass < 2 && !planned; ++pass) {
-        build_tables();
+    for (int pass = few || !p.early ? 1 : 0; pass < 2 && !planned; ++pass) {
+        build_tables(pass != 0);
         if (pass) break;
         if (wid == NCW && lane == 0 && u0 < u1) {
             int r = find_region(s_P, n, u0);
@@ -1199,6 +1204,14 @@ int launch_decode_a(const aircache_ragged_t *c, DecodeParams &p, int kv_heads, c
     int dev = 0, sms = 0;
     if ((rc = current_device(&dev, &sms))) return rc;
     const int ctas = sms < kMaxDecodeCtas ? sms : kMaxDecodeCtas;
+    // Many regions of hardly a unit and one CTA per SM: the CTAs of the call before end together, so the early tables cover
+    // nothing, and their check is one more look at every length.  640 cells of 8 heads of 128 (units of 64 rows): 13.6 us a
+    // call of 20 rows a cell with the tables built once, 14.8 early; of 45 rows 16.1 and 15.1.  1792 cells of 7 heads: 28.7
+    // and 32.1, 31.8 and 32.6 at 45 rows, 45.4 and 43.8 at 90.  1792 regions of 4 KV heads (32 rows): 34.5 and 37.1 at 10
+    // rows, 40.4 and 39.8 at 20, 50.7 and 47.3 at 30.  300 cells of 20 rows: 13.1 and 9.7; 1792 cells of 64 channels, of
+    // which an SM holds two CTAs: 24.6 and 22.8.  (The rows are those of the buffers: the lengths are on the device.)
+    p.early = 2 * C::SMEM_BYTES <= 227 * 1024 || p.n_regions <= 3 * ctas ||
+              8 * (int64_t)p.total_rows >= 5 * C::CH * (int64_t)p.n_regions;
     static std::atomic<uint64_t> allowed[kMaxDevices];
     if ((rc = allow_shared_memory((const void *)decode_kernel<D, HKV, G_HI, HS, APPEND>, C::SMEM_BYTES, dev, allowed))) return rc;
     cudaLaunchConfig_t cfg = {};

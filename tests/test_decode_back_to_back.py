@@ -86,6 +86,15 @@ def test_steps_over_shared_tables(layers, hq, hkv, d):
     run_steps(layers, hq, hkv, d, rng.integers(0, 140, layers).tolist(), 40, layers)
 
 
+@pytest.mark.parametrize("most", [25, 45])
+@pytest.mark.parametrize("layers,hq,hkv,d", [(460, 7, 1, 128), (450, 8, 2, 64), (460, 4, 1, 64), (440, 7, 1, 128)])
+def test_steps_over_many_short_regions(layers, hq, hkv, d, most):
+    """More than three regions to a block, of few rows: there the tables are built behind the dependency wait only, unless
+    two blocks share an SM or the buffers hold five eighths of a unit (40 rows here) a region: both sides of each line."""
+    rng = np.random.default_rng(layers)
+    run_steps(layers, hq, hkv, d, rng.integers(most - 12, most + 12, layers).tolist(), 7, layers)
+
+
 @pytest.mark.parametrize("layers,batch,hq,hkv,d", [(28, 4, 28, 4, 128), (30, 3, 8, 8, 64), (40, 2, 4, 1, 128)])
 def test_new_layouts_back_to_back(layers, batch, hq, hkv, d):
     """Scores, budgets, compaction and a decode call in a row, again and again into the same cache, without a wait: the
