@@ -407,13 +407,13 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
     int32_t *kept = kept_idx ? kept_idx : ws_ptr<int32_t>(ws, w.kept);
     uint32_t *status = ws_ptr<uint32_t>(ws, w.status);
     const int64_t kept_cap = (int64_t)s->batch * kept_per_sequence(s, ratio);
-    // Few regions: as many threads as a block has, since the chain of a region is all there is.  Many: small blocks, of
-    // which an SM holds eight (256 threads) or four.
+    // At most one region per SM: as many threads as a block has, since the chain of a region is all there is.  More: small
+    // blocks, of which an SM holds five (256 threads) or two.
     int dev = 0, sms = 0;
     const int rc = current_device(&dev, &sms);
     if (rc) return rc;
     const SelectArgs a = {scores, budgets, out->offsets, s->n_visual, s->n_text, s->slack, out->first_row, kept, kept_cap, status};
-    const bool many = LB > 2 * sms;
+    const bool many = LB > sms;
     cudaError_t e;
     if (many && s->n_visual <= 256 * 16) e = launch_select<256, 16>(a, LB, st);
     else if (many && s->n_visual <= 512 * 16) e = launch_select<512, 16>(a, LB, st);
