@@ -1,8 +1,10 @@
 // aircache_score: importance of every visual token seen from the elite observation window
 // (Section 3.3, Eq. 4-8), all layers and sequences per launch.
 //
-// Sequences of up to 16384 visual tokens are scored by the cluster kernel of score_cluster.cu.  Here is the rest:
-// longer ones, caches that no tensor map describes, and alpha = 0 with 32 window rows or more.  Kernels on one stream:
+// Sequences of up to 16384 visual tokens are scored by the cluster kernel of score_cluster.cu, alpha = 0 with 32 window
+// rows or more by the passes of score_dense.cu.  Here is the rest: longer sequences, windows too wide for the cluster
+// kernel's shared memory (128 channels, 128 window queries and 8 heads to a group), many groups of hardly a tile, and
+// caches that no tensor map describes.  Kernels on one stream:
 //   elite_kernel       one CTA per (layer, sequence, KV head): the W candidate keys and the last text query
 //                      are staged in shared memory; Eq. 4 logits as fp64 dot products in element order (so
 //                      the Eq. 5 decision does not depend on a summation order), the elite set of each
@@ -798,6 +800,21 @@ int launch_group_sum(const ScoreParams &p, cudaStream_t st) {
     return AIRCACHE_OK;
 }
 
+// Many KV groups of hardly a tile of keys: a cluster then spends its time on a group's elite rows, one unit of 16 after the
+// other, with two blocks to an SM; elite_kernel and the one-pass kernel hold six and five.  What there is of it grows with
+// the elite rows, of which a low alpha leaves many, and large groups fill the cluster kernel's units better.  Measured
+// (older kernels, cluster kernel; us a call):
+//   14336 groups of 4 heads, 64 channels, 16 window queries: alpha 0.9, 3 tokens 210, 270; 32 tokens 242, 277; 96 tokens 306,
+//   278.  alpha 0.1, 3 tokens 508, 944; 64 tokens 700, 939; 128 tokens 954, 961.  alpha 0.3, 16 tokens 346, 596.
+//   3584 groups of 2 heads: alpha 0.9, 32 tokens 64, 79; 128 tokens 92, 90 (alpha 0.5).  14336 groups of 1 head of 128 channels:
+//   alpha 0.9, 3 tokens 230, 292; 64 tokens 303, 287.  7168 groups of 7 heads: alpha 0.9, 64 tokens 219, 171.
+//   224 groups of 4 heads, alpha 0.1, 3 tokens: 36, 25.
+static bool hardly_a_tile(const ScoreParams &p, float alpha, int sms) {
+    if ((int64_t)p.n_lb * p.Hkv < 6 * (int64_t)sms || p.keep_all) return false;
+    if (alpha < 0.75f) return (int64_t)p.Nv * p.Nv * p.G <= 136 * 136;
+    return p.G <= 4 && p.W <= 64 && p.Nv <= 32;
+}
+
 int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void *q_window, float alpha,
                  int layer_begin, int layer_count, float *scores, uint64_t *elite_mask, void *ws, cudaStream_t st) {
     const WsLayout w = ws_layout(s);
@@ -832,8 +849,11 @@ int launch_score(const aircache_shape_t *s, const aircache_full_t *f, const void
     p.status = ws_ptr<uint32_t>(ws, w.status);
 
     // alpha = 0 with at least a cluster's two query blocks keeps the tensor cores and the exponentials busy by itself
-    int taken = 0;
-    const int rc = p.keep_all && p.G * p.W >= 32 ? launch_score_dense(p, s, f, st, &taken) : launch_score_cluster(p, s, f, st, &taken);
+    int taken = 0, dev = 0, sms = 0;
+    int rc = current_device(&dev, &sms);
+    if (rc) return rc;
+    if (p.keep_all && p.G * p.W >= 32) rc = launch_score_dense(p, s, f, st, &taken);
+    else if (!hardly_a_tile(p, alpha, sms)) rc = launch_score_cluster(p, s, f, st, &taken);
     if (rc || taken) return rc;
 
     // What the remaining kernels need.  A call over few KV groups (a layer at a time, a single sequence) would leave SMs

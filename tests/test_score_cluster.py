@@ -155,3 +155,24 @@ def test_scores_near_the_smallest(oracle_mod, n_visual, window, alpha):
     small = want > 2.0 ** -120
     assert small.sum() > want.size // 2
     assert (np.abs(got - want)[small] / want[small]).max() <= 2e-5
+
+
+@pytest.mark.parametrize("heads,d,window,alpha,n_visual", [
+    ((8, 4), 64, 16, 0.9, 32), ((8, 4), 64, 16, 0.9, 33), ((8, 4), 64, 16, 0.5, 96), ((8, 4), 64, 16, 0.5, 97),
+    ((4, 4), 128, 64, 0.9, 3), ((4, 4), 128, 70, 0.9, 3), ((32, 4), 64, 16, 0.3, 48), ((32, 4), 64, 16, 0.3, 49),
+    ((8, 4), 64, 16, 0.9, 31)])
+@pytest.mark.parametrize("batch,per_head", [(8, 0), (7, 0), (8, 1)])
+def test_many_groups_of_hardly_a_tile(oracle_mod, heads, d, window, alpha, n_visual, batch, per_head):
+    """Both sides of the lines between the cluster kernel and the older ones where a call covers many groups of few keys (896
+    groups on 148 SMs are enough, 784 are not).  Logits of a few units, some hundred terms to a sum: 2e-5."""
+    wl = Workload("hardly", 28, heads[0], heads[1], d, batch=batch, n_visual=n_visual, n_text=80, ratio=0.1, steps=1,
+                  window=window, alpha=alpha)
+    k, v, qw = gen_inputs(wl, "cpu")
+    score = oracle_mod.score_groups if per_head else oracle_mod.score
+    ref = score(oracle_dims(oracle_mod, wl), u16(logical(k)), u16(qw), wl.scale, alpha)
+    gp = GpuPath(wl, device=DEV, per_kv_head=per_head)
+    gp.set_full(logical(k.to(DEV)), logical(v.to(DEV)))
+    gp.score(qw.to(DEV), alpha=alpha)
+    assert gp.status() == 0
+    assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
+    assert rel_elem_err(gp.scores.cpu().numpy(), ref["scores"]) <= 2e-5
