@@ -24,6 +24,9 @@ tokens per sequence) at batch 64, 2 GB of compressed cache per decode launch, 25
                   config 4, config 5) with its full number of decode rounds, measured briefly after the main
                   run at N = 1: stage times, the three rooflines, clocks
 
+One line on stdout with the keys above down to cpu_baseline but without the rooflines of the compression; one line on
+stderr with everything.
+
 `python bench.py --impl reference` times the CPU oracle instead (there is no other implementation of the
 paper's method to run).  Under torchrun every rank runs the same workload on its own GPU with its own seeds
 (no data-path collective: requests are independent); times are device times, maximum over ranks.
@@ -603,7 +606,22 @@ def run_cuda(args):
         dist.barrier()
         dist.destroy_process_group()
     if rank == 0:
-        print(json.dumps(result))
+        print(json.dumps(result), file=sys.stderr)
+        print(json.dumps(short_line(result), separators=(",", ":")))
+
+
+# What the printed line holds.  It has to be read from the end of a log, so everything else (the other workloads, sweeps,
+# rooflines of the compression, ablations) goes to stderr, as one line of its own.
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+             "dtype", "data", "config", "decode_tok_s", "compress_us_per_layer", "roofline", "clocks", "gpu_launches", "e2e")
+
+
+def short_line(result):
+    line = {k: result[k] for k in LINE_KEYS if k in result}
+    line["clocks"] = {k: v for k, v in result["clocks"].items() if k in ("sm_mhz", "sm_max_mhz", "reasons")}
+    if "cpu_baseline" in result:
+        line["cpu_baseline"] = {k: result["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    return line
 
 
 def dense_window_score(wl, s, reps=10):
