@@ -324,10 +324,9 @@ def default_rotate(ac, wl):
 
 
 def kernels_per_step(wl, rotate, n_dec):
-    """Launches of this library's kernels in one step: elite + one-pass scoring + sum over the KV groups; budget;
-    select + gather; one decode kernel per call.  (alpha = 0 and sequences too long for the one-pass kernel
-    launch differently; no bench workload is either.)"""
-    score = 3
+    """Launches of this library's kernels in one step, at least: scoring (the sum over the KV groups that follows in calls
+    over few sequences is not counted); budget; select + gather; one decode kernel per call."""
+    score = 1
     return rotate * (score + 1 + 2 + n_dec)
 
 
