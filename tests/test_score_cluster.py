@@ -63,8 +63,8 @@ def test_ties_at_the_threshold(oracle_mod, window):
     (1000, (14, 2), 128, 64, 6.0, 0), (4097, (28, 4), 128, 16, 6.0, 1), (2500, (4, 4), 64, 128, 1.0, 0),
     (20000, (16, 1), 64, 9, 1.0, 0)])
 def test_whole_window_at_the_edges(oracle_mod, n_visual, heads, d, window, sharp, per_head):
-    """alpha = 0: one tile and fewer, query blocks that fill 128 rows and that do not, several of them, references that
-    have to move, and a sequence cut into many pieces."""
+    """alpha = 0: one tile and fewer, query blocks that fill 128 rows and that do not, several of them, logits up to six times
+    as sharp (no reference moves for them: test_score_paths.py), and a sequence cut into many pieces."""
     wl = Workload("edge0", 2, heads[0], heads[1], d, batch=2, n_visual=n_visual, n_text=130, ratio=0.1, steps=1,
                   window=window, alpha=0.0)
     scale = sharp / d ** 0.5
