@@ -36,11 +36,14 @@ constexpr int64_t kResetBytes = kStatusBytes + kPlanMemoBytes;
 // ---------------------------------------------------------------------------------------------
 void set_last_cuda_error(cudaError_t e);
 
+// (An error that was returned is taken out of the runtime's own record too: the check behind a later launch would
+// report it for that launch.)
 #define AIRCACHE_CUDA_TRY(expr)                         \
     do {                                                \
         cudaError_t _e = (expr);                        \
         if (_e != cudaSuccess) {                        \
             ::aircache::set_last_cuda_error(_e);        \
+            cudaGetLastError();                         \
             return AIRCACHE_ERR_CUDA;                   \
         }                                               \
     } while (0)
