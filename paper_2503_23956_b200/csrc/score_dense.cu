@@ -357,13 +357,19 @@ dense_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
                 const float4 *f4 = reinterpret_cast<const float4 *>(sm.tab.factor[v & 1]);
                 const int n32 = rows >> 5;               // whole sets of 32 rows; the rest, if any, in up to two of 16
                 const bool rest = (rows & 31) != 0, rest2 = (rows & 31) > 16;
+                const bool ragged = (rows & 15) != 0;    // rows of zeros fill the last sixteen: NaN beside a masked key's infinities
                 float2 a0, a1;
                 auto columns = [&](const uint32_t *x, int c, auto n) {
 #pragma unroll
                     for (int j = 0; j < decltype(n)::value; j += 4) {
                         const float4 nm = nm4[(c + j) >> 2], f = f4[(c + j) >> 2];
-                        const float2 u = fma2(pair(x, j), sl2, make_float2(nm.x, nm.y));
-                        const float2 w = fma2(pair(x, j + 2), sl2, make_float2(nm.z, nm.w));
+                        float2 xa = pair(x, j), xb = pair(x, j + 2);
+                        if (decltype(n)::value == 16 && ragged) {
+                            xa = make_float2(c + j < rows ? xa.x : 0.f, c + j + 1 < rows ? xa.y : 0.f);
+                            xb = make_float2(c + j + 2 < rows ? xb.x : 0.f, c + j + 3 < rows ? xb.y : 0.f);
+                        }
+                        const float2 u = fma2(xa, sl2, make_float2(nm.x, nm.y));
+                        const float2 w = fma2(xb, sl2, make_float2(nm.z, nm.w));
                         a0 = fma2(make_float2(fast_exp2(u.x), fast_exp2(u.y)), make_float2(f.x, f.y), a0);
                         a1 = fma2(make_float2(fast_exp2(w.x), fast_exp2(w.y)), make_float2(f.z, f.w), a1);
                     }

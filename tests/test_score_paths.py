@@ -134,3 +134,15 @@ def test_windows_wide_for_the_cluster(oracle_mod, heads, d, window, alpha):
     wl = workload(1, heads, d, 2, 900, window, alpha)
     k, v, qw = gen_inputs(wl, "cpu")
     compare(oracle_mod, wl, k, v, qw, 2e-5)
+
+
+@pytest.mark.parametrize("heads,window", [((14, 2), 5), ((14, 2), 9), ((16, 1), 19), ((14, 2), 16), ((3, 1), 43)])
+def test_whole_window_masked_keys(oracle_mod, heads, window):
+    """Keys of minus infinity in the whole-window passes score zero, also where the window rows of a KV group do not fill the
+    last sixteen columns of a query block (35, 63, 129 in two blocks of up to 66) or do (304 in three, 112)."""
+    wl = workload(2, heads, 128, 1, 700, window, 0.0)
+    k, v, qw = gen_inputs(wl, "cpu")
+    qw[..., 0], k[..., 0] = qw[..., 0].abs() + 0.125, 0.0
+    k[:, :, 3:6, :, 0] = float("-inf")
+    k[:, :, 128:450, :, 0] = float("-inf")
+    compare(oracle_mod, wl, k, v, qw, 2e-5)
