@@ -34,11 +34,14 @@
  *             issues many copies and launches, is the exception: see there).
  *             No exception crosses the ABI.
  * Threads.    The library keeps no mutable global state apart from a per-thread
- *             copy of the last CUDA error code, the device address of the
- *             built-in array of aircache_decode_attn_static and the number of
- *             blocks of the scoring kernel a device holds at once (each looked
- *             up once per device, under a lock); calls that share a workspace
- *             must be ordered on one stream.
+ *             copy of the last CUDA error code and what it has looked up or
+ *             set once: per device the number of SMs and of blocks and
+ *             clusters of the scoring kernels that it holds at once, per
+ *             context the kernels' shared-memory limits and the address of
+ *             the built-in array of aircache_decode_attn_static (so that a
+ *             program may go on after cudaDeviceReset).  All of it may be used
+ *             from several threads; calls that share a workspace must be
+ *             ordered on one stream.
  * Determinism. Same inputs give the same output bits on every run.
  */
 #ifndef AIRCACHE_H
@@ -175,13 +178,18 @@ int64_t aircache_workspace_bytes(const aircache_shape_t *shape);
  *   scores      fp32 [L, B, Nv]        output I_v
  *   elite_mask  u64  [L, B, Hq, ceil(W/64)]  output, candidate w is elite <=> bit w % 64 of word w / 64 is
  *                                      set (one word per head up to W = 64, two beyond); may be NULL
+ * A key whose logits are minus infinity (masked) scores zero, or NaN where blocks of
+ * one grid take the call (see below); the other keys' scores are not touched by it.
  * The blocks that share a KV group wait for one another: the blocks of one thread-
  * block cluster, which the hardware starts together, up to 16384 visual tokens;
- * beyond (and for caches that no tensor map describes) blocks of one grid, which
- * the library only lets do so when at most half of the blocks the GPU holds at
- * once are involved.  All waits are bounded; if one gives up (other work keeps
- * most of the GPU busy for a quarter of a second), the scores are incomplete and
- * aircache_check_status() reports AIRCACHE_ERR_TIMEOUT.
+ * beyond (and for caches that no tensor map describes, windows that do not fit a
+ * block - of 128 channels: 128 queries with 8 heads to a group, 110 with 16 - and
+ * calls over some 900 KV groups or more of up to about a hundred visual tokens)
+ * blocks of one grid, which the library only lets do so when at most half of the
+ * blocks the GPU holds at once are involved.  All waits are bounded, within a
+ * cluster to about a second, within a grid to a quarter of one; if one gives up
+ * (other work keeps most of the GPU busy for that long), the scores are incomplete
+ * and aircache_check_status() reports AIRCACHE_ERR_TIMEOUT.
  */
 int aircache_score(const aircache_shape_t *shape, const aircache_full_t *full, const void *q_window,
                    float alpha, float *scores, uint64_t *elite_mask, void *workspace, int64_t workspace_bytes,
@@ -209,7 +217,8 @@ int aircache_score_layers(const aircache_shape_t *shape, const aircache_full_t *
 /*
  * Section 3.4, Eq. 9-11 and the budget line of Algorithm 1.  Per region:
  * strength s_t = sum of I_v (Eq. 9) and skewness s_k = adjusted Fisher-Pearson
- * coefficient with the sample standard deviation (Eq. 10), both in fp64.  Per
+ * coefficient with the sample standard deviation (Eq. 10), both in fp64, in an order
+ * that depends on n_visual alone (a sequence has the same bits in every batch).  Per
  * sequence: both are divided by their mean over the layers (negative skewness
  * counts as 0, a zero mean makes the factor 1), w_l = (s't + s'k) / 2 (Eq. 11),
  * and T = aircache_kept_per_sequence() rows are split in proportion to w_l with
@@ -291,7 +300,7 @@ int aircache_decode_step(const aircache_shape_t *shape, aircache_ragged_t *cache
  *            bytes must fit in the array (7424 = 256 bytes of status + 1792 tickets;
  *            on a 148-SM B200: Hq * (d + 2) <= 10620, e.g. 80 heads of 128);
  *            larger problems get AIRCACHE_ERR_STATIC_SCRATCH and nothing is enqueued.
- *   Set-up.  The first call on each device looks up the array's device address
+ *   Set-up.  The first call in each context looks up the array's device address
  *            (with that device current).  Make that first call before any
  *            stream capture is begun.
  *   Sharing. All calls on a device use the one array, and the array keeps what

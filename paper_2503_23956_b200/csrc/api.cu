@@ -378,7 +378,7 @@ int aircache_pipeline_host(const aircache_shape_t *shape, const aircache_full_t 
     aircache_full_t d_full = *h_full;
     d_full.k = d_full_k;
     d_full.v = d_full_v;
-    // K is read twice in full by the scoring passes, so it is uploaded.  V is read once, and only the rows that
+    // K is read in full by the scoring kernels, so it is uploaded.  V is read once, and only the rows that
     // survive (kept visual rows and text rows): when the host buffer is page-locked and mapped, the gather
     // kernel reads those rows from it in place and the upload of the other rows never happens.
     void *v_in_place = mapped_host_range(h_full->v, full_elems * 2);

@@ -6,9 +6,9 @@
 //                  the k-th, until few enough are left to be ranked directly (mostly after one histogram).  Then
 //                  the kept token indices in ascending order, duplicates of the threshold value taken from the
 //                  lowest indices, by ballots and one scan.
-//   gather_kernel  one warp per output row [Hkv, d] of K' and of V': 16-byte loads along the source row's
-//                  head slices, 16-byte stores to the packed row.  Region of a row by binary search in the
-//                  offsets table.
+//   gather_kernel  one warp per four output rows [Hkv, d] of K' and of V': 16-byte loads along the source rows' head
+//                  slices, 16-byte stores to the packed rows.  Region of the first row by 32 probes at a time in the
+//                  offsets table, of the further ones by walking on.
 #include "common.cuh"
 
 namespace aircache {

@@ -3,8 +3,8 @@
 //
 // Sequences of up to 16384 visual tokens are scored by the cluster kernel of score_cluster.cu, alpha = 0 with 32 window
 // rows or more by the passes of score_dense.cu.  Here is the rest: longer sequences, windows too wide for the cluster
-// kernel's shared memory (128 channels, 128 window queries and 8 heads to a group), many groups of hardly a tile, and
-// caches that no tensor map describes.  Kernels on one stream:
+// kernel's shared memory (of 128 channels: 128 queries with 8 heads to a group, 110 with 16), many groups of hardly a tile,
+// and caches that no tensor map describes.  Kernels on one stream:
 //   elite_kernel       one CTA per (layer, sequence, KV head): the W candidate keys and the last text query
 //                      are staged in shared memory; Eq. 4 logits as fp64 dot products in element order (so
 //                      the Eq. 5 decision does not depend on a summation order), the elite set of each

@@ -1,21 +1,23 @@
 // Scoring by thread-block clusters: Eq. 4-8 in one launch with one read of the visual keys, for sequences that a
-// cluster of up to eight blocks holds (16384 visual tokens).
+// cluster of up to eight blocks holds (16384 visual tokens) and windows that fit a block beside two ring stages.
 //
 // A cluster of C blocks works on one KV group (layer, sequence, KV head) at a time, each block on a stretch of the
 // visual keys in tiles of 128.  Warp roles inside a block (two blocks share an SM):
 //   producer   one thread: key tiles by TMA (128-byte swizzle) through a ring of shared-memory stages
-//   tensor     one thread: tcgen05.mma M = 128 keys, N = 16 elite rows, D in a 16-column slot of tensor memory per
-//              tile, so the logits of all of a block's tiles stay on chip
-//   elite      four warps: Eq. 4-5 of the group (fp64 logits in element order, masks), the table of elite rows,
-//              16 query rows at a time into the swizzled operand layout, each row's softmax statistics over the
-//              elite text keys it sees.  Every block of the cluster does this for itself, one group ahead.
+//   tensor     one warp, of which an elected lane issues: tcgen05.mma M = 128 keys, N = 16 elite rows, D in a 16-column
+//              slot of tensor memory per tile, so the logits of all of a block's tiles stay on chip
+//   elite      four warps: Eq. 4-5 of the group (fp32 logits, and the defining fp64 ones in element order for heads with
+//              a candidate at the threshold), the masks, the table of elite rows, 16 query rows at a time into the
+//              swizzled operand layout, each row's softmax statistics over the elite text keys it sees.  Every block
+//              of the cluster does this for itself, one group ahead.
 //   epilogue   four warps, a thread owns a key (tensor-memory lane) of every tile and the 16 rows' values in
 //              registers:  e = exp2(logit - reference) as a tile arrives, written back over the logit, and the
 //              running sum per row; at the end of the stretch the sums meet (warp, block, then cluster through
 //              distributed shared memory), and p = e * F with F = weight / normaliser * exp2(reference - max) per
 //              thread and row: one exponential per logit, no reduction across lanes for Eq. 8.
 // The reference is the thread's first logit of the row.  It need not be the maximum, only near enough for fp32's
-// range: a logit more than 2^24 above it moves it (the stored values of the earlier tiles are rescaled; rare).
+// range: a logit more than 2^24 above it takes its place (the stored values of the earlier tiles are rescaled; rare).
+// A masked key (a logit of minus infinity) is no reference, and scores zero.
 //
 // More than 16 elite rows: the keys are read again (from L2) for every further 16.  The KV groups of a (layer,
 // sequence) either follow one another in the same cluster, each adding to the scores, or - when there are too few
@@ -23,8 +25,8 @@
 //
 // What it replaced (elite kernel, one-pass kernel on mma.sync with a wait between blocks, sum kernel) streamed keys
 // during half of a block's life and took three launches.  Measured, 28 layers of 28 query and 4 KV heads of 128
-// channels: 64 sequences of 2916 tokens 1180 -> 882 us (6.1 TB/s of keys: at the memory's rate); one of 7290 tokens
-// 75 -> 51 us; four of 6272, a call per layer, 33 -> 17 us a call.  A call of one layer is a chain of latencies: some
+// channels: 64 sequences of 2916 tokens 1196 -> 837 to 867 us by the box (6.2 TB/s of keys: at the memory's rate); one of
+// 7290 tokens 75 -> 47 us; four of 6272, a call per layer, 33 -> 17 us a call.  A call of one layer is a chain of latencies: some
 // 7 us until the first query block is ready (2 of them the first rows from memory), 4 us until the last tile has been
 // multiplied, 4 us for the exchange and Eq. 8.
 //

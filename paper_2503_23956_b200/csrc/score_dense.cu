@@ -14,7 +14,7 @@
 //
 // What bounds it: the keys, read twice, and the exponentials, two per logit.  28 layers of 28 query heads, 16 window
 // queries and 7290 tokens: 36 us a pass without the exponentials (33 at the memory's rate), 24 us a pass for the
-// exponentials alone (16 a clock and SM), 48 and 50 us as it is; with what it replaced 189 us a call, now 95.  (That had
+// exponentials alone (16 a clock and SM), 48 and 50 us as it is; with what it replaced 189 us a call, now 99 to 102.  (That had
 // a kernel for the table of rows, running maxima, sixteen microseconds and a quarter of each pass on merging statistics
 // in one block.)  Hence no work per logit but one multiply-add, the exponential and one addition, two logits to an
 // instruction: a row's reference is the largest logit of its first columns, and moves only when a sum of 32 passes
