@@ -236,7 +236,7 @@ int aircache_budget(const aircache_shape_t *shape, const float *scores, double r
 
 /*
  * Algorithm 1, second loop.  Per region: the n_r visual tokens of largest score
- * (radix select on the fp32 bit pattern; equal scores: the lower token index
+ * (histograms over the fp32 bit patterns; equal scores: the lower token index
  * wins), then K' = Concat(K_v[kept], K_t), V' = Concat(V_v[kept], V_t) are
  * gathered into the region's rows, kept tokens in ascending token order.
  * out->offsets and out->lens must hold what aircache_budget wrote for `budgets`.
