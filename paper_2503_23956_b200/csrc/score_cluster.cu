@@ -25,7 +25,7 @@
 //
 // What it replaced (elite kernel, one-pass kernel on mma.sync with a wait between blocks, sum kernel) streamed keys
 // during half of a block's life and took three launches.  Measured, 28 layers of 28 query and 4 KV heads of 128
-// channels: 64 sequences of 2916 tokens 1196 -> 837 to 867 us by the box (6.2 TB/s of keys: at the memory's rate); one of
+// channels: 64 sequences of 2916 tokens 1196 -> 835 to 870 us by the box (6.2 TB/s of keys: at the memory's rate); one of
 // 7290 tokens 75 -> 47 us; four of 6272, a call per layer, 33 -> 17 us a call.  A call of one layer is a chain of latencies: some
 // 7 us until the first query block is ready (2 of them the first rows from memory), 4 us until the last tile has been
 // multiplied, 4 us for the exchange and Eq. 8.
@@ -63,7 +63,7 @@ struct ClusterSmem {   // small state behind the ring and the query block
     uint64_t acc_full[kSlots], acc_empty[2], exchange[2];
     float2 stats[2][kMaxCluster][kRows];   // (max, sum) of every block of the cluster
     float2 warp_stats[2][4][kRows];
-    float2 fin[4][kRows];                  // per epilogue warp: (max, weight / normaliser)
+    float2 fin[4][kRows];                  // per epilogue warp: (max, 2^64 weight / normaliser)
     float2 text[2][kRows];
     float coef[2][kRows];
     int2 meta[2];                          // rows of the unit, last unit of its group
@@ -549,19 +549,13 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
 #pragma unroll
                             for (int r = 0; r < kRows; ++r) m[r] = valid ? fmaxf(x[r] * p.sl2, kNegBig) : kNegBig;   // (a masked key: -inf)
                         }
-                        // What is left of a logit beside the reference made from it: the rounding of the product.  (Of a masked
-                        // key's 1e29 that would be 1e21: nothing then.)
-                        auto beside = [&](float logit, float ref) {
-                            const float d = fmaf(logit, p.sl2, -ref);
-                            return fabsf(d) > 1.f && ref > kNegBig ? 0.f : d;
-                        };
                         float top = -INFINITY;
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             if (q < quads) {
 #pragma unroll
                                 for (int r = 4 * q; r < 4 * q + 4; ++r) {
-                                    x[r] = t == 0 ? beside(x[r], m[r]) : fmaf(x[r], p.sl2, -m[r]);
+                                    x[r] = fmaf(x[r], p.sl2, -m[r]);
                                     if (tail && !valid) x[r] = -INFINITY;
                                     top = fmaxf(top, x[r]);
                                 }
@@ -584,7 +578,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                                         const float mn = move ? raw[j] * p.sl2 : m[r];
                                         fac[j] = move ? fast_exp2(m[r] - mn) : 1.f;
                                         z[r] *= fac[j];
-                                        if (move) x[r] = beside(raw[j], mn);
+                                        // (what is left beside it: the rounding of the product, nothing of a masked key's 1e29)
+                                        const float d = fmaf(raw[j], p.sl2, -mn);
+                                        if (move) x[r] = fabsf(d) > 1.f ? 0.f : d;
                                         m[r] = mn;
                                     }
 #pragma unroll 1
@@ -669,7 +665,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                             const float2 o = sm.stats[par][c][lane];
                             sum = fmaf(o.y, fast_exp2(o.x - mx), sum);
                         }
-                        sm.fin[ew][lane] = make_float2(mx, sm.coef[par][lane] / sum);
+                        sm.fin[ew][lane] = make_float2(mx, sm.coef[par][lane] / sum * kScaleUp);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&sm.meta_empty[par]));
@@ -681,7 +677,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         const float2 f = sm.fin[ew][r];
                         const float below = m[r] - f.x;
                         const bool far = below < -100.f;
-                        m[r] = f.y * (fast_exp2(far ? below + 64.f : below) * (far ? 1.f : kScaleUp));
+                        m[r] = (far ? f.y * (1.f / kScaleUp) : f.y) * fast_exp2(far ? below + 64.f : below);
                     }
                     __syncwarp();
 
