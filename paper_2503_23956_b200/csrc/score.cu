@@ -177,10 +177,6 @@ __global__ void __launch_bounds__(128, QREG ? 2 : 6) elite_kernel(ScoreParams p)
 // (read straight from global memory) and for the query rows (shared memory).  A dot product does not
 // depend on the order of its terms' indices as long as both operands use the same order.
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void prefetch_l2(const void *ptr) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr) : "memory");
-}
-
 template <int D>
 struct KeyFrag {
     uint4 lo[D / 32];  // key row gid

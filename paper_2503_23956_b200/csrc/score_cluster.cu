@@ -26,9 +26,13 @@
 // What it replaced (elite kernel, one-pass kernel on mma.sync with a wait between blocks, sum kernel) streamed keys
 // during half of a block's life and took three launches.  Measured, 28 layers of 28 query and 4 KV heads of 128
 // channels: 64 sequences of 2916 tokens 1196 -> 835 to 870 us by the box (6.2 TB/s of keys: at the memory's rate); one of
-// 7290 tokens 75 -> 47 us; four of 6272, a call per layer, 33 -> 17 us a call.  A call of one layer is a chain of latencies: some
-// 7 us until the first query block is ready (2 of them the first rows from memory), 4 us until the last tile has been
-// multiplied, 4 us for the exchange and Eq. 8.
+// 7290 tokens 75 -> 45 us; four of 6272, a call per layer, 33 -> 15.5 us a call.  A call of one layer is a chain of latencies (us
+// behind the wait for what is before it in the stream): 1.4 until the rows of the first query block are staged, 4.2 until
+// the block is ready, 8.2 until the last tile has been multiplied, 12 at the end; then the sum over groups and the launches'
+// hand-over, 3.  What shortened it from 17: the first rows and tiles are asked into L2 and the addresses worked out ahead of
+// the wait, an idle warp's lanes ask for the window's queries (one thread took 1 us for the 16 copies), the text columns'
+// statistics and the masks are written behind the query block, which does not need them, and no block waits for its
+// cluster at its end: 16.9 -> 15.5 us; image 47.6 -> 45.3.
 //
 // With up to eight tiles per block the tensor memory holds two units of work and the tensor core runs ahead of the
 // epilogue; with up to sixteen the other block of the SM fills the gap.  All waits are bounded.
@@ -59,7 +63,7 @@ constexpr int kFirstAhead = 5;        // tiles asked into L2 behind the first fu
 
 struct ClusterSmem {   // small state behind the ring and the query block
     uint64_t full[kMaxStages], empty[kMaxStages];
-    uint64_t q_full[2], meta_empty[2], q_free, q_all, q_taken;
+    uint64_t q_full[2], text_full[2], meta_empty[2], q_free, q_all, q_taken;
     uint64_t acc_full[kSlots], acc_empty[2], exchange[2];
     float2 stats[2][kMaxCluster][kRows];   // (max, sum) of every block of the cluster
     float2 warp_stats[2][4][kRows];
@@ -125,6 +129,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
         for (int i = 0; i < S; ++i) { mbar_init(smem_u32(&sm.full[i]), 1); mbar_init(smem_u32(&sm.empty[i]), 1); }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&sm.q_full[i]), 1);
+            mbar_init(smem_u32(&sm.text_full[i]), kRows);
             mbar_init(smem_u32(&sm.meta_empty[i]), 5);   // producer and four epilogue warps
             mbar_init(smem_u32(&sm.acc_empty[i]), 4);
             mbar_init(smem_u32(&sm.exchange[i]), 1);
@@ -151,13 +156,50 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
     const int T = t1 - t0, key0 = t0 * 128;
     const int first_grp = p.lb0 * p.Hkv;
 
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // nothing above read global memory
+    // The block's first group: its rows and first tiles are asked into L2 while the block waits for what is before it in the
+    // stream (hints: they consume no value; the blocks of a cluster share the lines of the rows), and the addresses of its
+    // rows are worked out.
+    const bool preload = p.W * p.G <= kPreloadRows;
+    const int n_vec = (p.W + p.G) * (D / 8);   // 16-byte vectors of the candidate keys and the last queries
+    const uint4 *first_rows[4];
+    {
+        const int grp = first_grp + cid * plan.groups_per_item;
+        const int g = grp % p.Hkv, lb = grp / p.Hkv, l = lb / p.B, b = lb - l * p.B;
+        const uint16_t *k_cand = p.k + (int64_t)l * p.s_layer + (int64_t)b * p.s_batch + (int64_t)g * p.s_head +
+                                 (int64_t)(p.Nv + p.Nt - p.W) * p.s_token;
+        const uint16_t *q0 = p.qw + ((int64_t)lb * p.W * p.Hq + g * p.G) * D;
+        if (warp >= kEliteWarp0 && warp < kEpiWarp0) {
+            constexpr int LK = D * 2 / 128;   // 128-byte lines of a key
+            const int lines = LK + p.G * LK;  // and of a window slot's queries
+            for (int i = (tid - kEliteWarp0 * 32) * plan.cluster + (int)rank; i < p.W * lines; i += kEliteThreads * plan.cluster) {
+                const int w = i / lines, c = i - w * lines;
+                prefetch_l2(c < LK ? k_cand + (int64_t)w * p.s_token + c * 64 : q0 + (int64_t)w * p.Hq * D + (c - LK) * 64);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int idx = tid - kEliteWarp0 * 32 + i * kEliteThreads, row = idx / (D / 8), c = idx % (D / 8);
+                first_rows[i] = reinterpret_cast<const uint4 *>(row < p.W ? k_cand + (int64_t)row * p.s_token
+                                                                          : q0 + ((int64_t)(p.W - 1) * p.Hq + row - p.W) * D) + c;
+            }
+        } else if (tid == 0) {
+            for (int t = 0; t < T && t < S + kFirstAhead; ++t) prefetch_key_tile<D>(&tm_k, p, key0 + t * 128, g, b, l);
+        }
+        asm volatile("griddepcontrol.wait;" ::: "memory");   // no value above came from global memory
+        // First unit of the block: all of the window's queries of the group come into the last ring stage at once, since
+        // which of them are elite is known two steps later only.
+        if (warp == 2 && preload) {
+            if (lane == 0) mbar_expect_tx(smem_u32(&sm.q_all), p.W * p.G * D * 2);
+            for (int w = lane; w < p.W; w += 32)
+                bulk_load(smem_u32(s_ring + (S - 1) * C::TILE_BYTES + w * p.G * D * 2), q0 + (int64_t)w * p.Hq * D, p.G * D * 2,
+                          smem_u32(&sm.q_all));
+        }
+    }
 
     // Units of work, in the same order in every role: item (the cluster's share), KV group of the item, 16 rows.
     if (warp == 0) {
         // ================================ producer ================================
-        // The keys of all blocks together occupy the memory for microseconds: the few rows that the elite warps need
-        // first come in before them.
+        // The few rows that the elite warps need first come in before the keys of all blocks.  (Both at once: one-layer calls
+        // 15.5 -> 15.7 us, an image 45.3 either way.)
         named_bar(3, kEliteThreads + 32);
         if (lane == 0) {
             bool ok = p.W * p.G > kPreloadRows || mbar_wait(smem_u32(&sm.q_all), 0, abort_flag, p.status, 32);
@@ -234,7 +276,6 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
         // ================================ elite rows ================================
         const int et = tid - kEliteWarp0 * 32, ew = warp - kEliteWarp0;
         const int words = (p.W + 31) >> 5;
-        const int n_vec = (p.W + p.G) * (D / 8);   // 16-byte vectors of the candidate keys and the last queries
         bool ok = true;
         uint32_t u = 0;
         // four vectors per thread from `base` on: loaded, then stored with the norm of every row
@@ -309,16 +350,10 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
         constexpr float kSlack = 5.5e-6f;
 
         uint4 ahead[4];   // the first vectors of the next group, on their way while this one is worked on
-        load_rows(first_grp + cid * plan.groups_per_item, et, ahead);
-        // First unit of the block: all of the window's queries of the group come into the last ring stage at once, since
-        // which of them are elite is known two steps later only.
-        const bool preload = p.W * p.G <= kPreloadRows;
-        if (preload && et == 0) {
-            const int grp = first_grp + cid * plan.groups_per_item, g = grp % p.Hkv, lb = grp / p.Hkv;
-            mbar_expect_tx(smem_u32(&sm.q_all), p.W * p.G * D * 2);
-            for (int w = 0; w < p.W; ++w)
-                bulk_load(smem_u32(s_ring + (S - 1) * C::TILE_BYTES + w * p.G * D * 2),
-                          p.qw + (((int64_t)lb * p.W + w) * p.Hq + g * p.G) * D, p.G * D * 2, smem_u32(&sm.q_all));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            ahead[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (et + i * kEliteThreads < n_vec) ahead[i] = __ldg(first_rows[i]);
         }
 
         for (int item = cid; ok && item < plan.items; item += n_clusters) {
@@ -399,11 +434,6 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     }
                 }
                 named_bar(2, kEliteThreads);
-                if (p.elite_mask && rank == 0 && et < p.G * ((p.W + 63) >> 6)) {
-                    const int w64 = (p.W + 63) >> 6, hl = et / w64, j = et - hl * w64;
-                    p.elite_mask[((int64_t)lb * p.Hq + g * p.G + hl) * w64 + j] =
-                        (uint64_t)sm.mask[hl][2 * j] | ((uint64_t)sm.mask[hl][2 * j + 1] << 32);
-                }
                 // rows: elite rows of head 0 first, ascending window slot; lane hl holds the rows up to and with head hl
                 int count = 0;
                 if (lane < p.G)
@@ -456,6 +486,32 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                             for (int i = 0; i < D / 64; ++i) qv[i] = __ldg(src + i * 8 + sub);
                         }
                     }
+                    __syncwarp();
+                    // the query block is free when the previous unit's MMAs have completed, the small tables when
+                    // the unit before that has been read
+                    ok = ok && (u < 1 || mbar_wait(smem_u32(&sm.q_free), (u - 1) & 1, abort_flag, p.status, 25)) &&
+                         (u < 2 || mbar_wait(smem_u32(&sm.meta_empty[u & 1]), ((u >> 1) & 1) ^ 1, abort_flag, p.status, 26));
+                    if (ok) {
+#pragma unroll
+                        for (int i = 0; i < D / 64; ++i)
+                            *reinterpret_cast<uint4 *>(s_q + i * C::Q_SUB + rr * 128 + ((sub ^ (rr & 7)) << 4)) = qv[i];
+                        if (sub == 0) sm.coef[u & 1][rr] = real ? coef : 0.f;
+                        if (et == 0) sm.meta[u & 1] = make_int2(min(kRows, max(n_rows - row0, 0)), row0 + kRows >= n_rows);
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // read by the tensor core
+                    }
+                    ok = named_bar_and(2, kEliteThreads, ok);
+                    if (et == 0 && ok) {
+                        mbar_arrive(smem_u32(&sm.q_full[u & 1]));
+                        if (u == 0) mbar_arrive(smem_u32(&sm.q_taken));
+                    }
+                    if (!ok) break;
+                    if (row0 == 0) {
+                        if (p.elite_mask && rank == 0 && et < p.G * ((p.W + 63) >> 6)) {
+                            const int w64 = (p.W + 63) >> 6, hl = et / w64, j = et - hl * w64;
+                            p.elite_mask[((int64_t)lb * p.Hq + g * p.G + hl) * w64 + j] =
+                                (uint64_t)sm.mask[hl][2 * j] | ((uint64_t)sm.mask[hl][2 * j + 1] << 32);
+                        }
+                    }
                     // Eq. 6-7, text columns: row w sees the elite text keys w' <= w
                     float mm = kNegBig, zz = 0.f;
                     if (real) {
@@ -484,25 +540,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         }
                     }
                     __syncwarp();
-                    // the query block is free when the previous unit's MMAs have completed, the small tables when
-                    // the unit before that has been read
-                    ok = ok && (u < 1 || mbar_wait(smem_u32(&sm.q_free), (u - 1) & 1, abort_flag, p.status, 25)) &&
-                         (u < 2 || mbar_wait(smem_u32(&sm.meta_empty[u & 1]), ((u >> 1) & 1) ^ 1, abort_flag, p.status, 26));
-                    if (ok) {
-#pragma unroll
-                        for (int i = 0; i < D / 64; ++i)
-                            *reinterpret_cast<uint4 *>(s_q + i * C::Q_SUB + rr * 128 + ((sub ^ (rr & 7)) << 4)) = qv[i];
-                        if (sub == 0) {
-                            sm.text[u & 1][rr] = make_float2(mm, real ? zz : 1.f);
-                            sm.coef[u & 1][rr] = real ? coef : 0.f;
-                        }
-                        if (et == 0) sm.meta[u & 1] = make_int2(min(kRows, max(n_rows - row0, 0)), row0 + kRows >= n_rows);
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // read by the tensor core
-                    }
-                    ok = named_bar_and(2, kEliteThreads, ok);
-                    if (et == 0 && ok) {
-                        mbar_arrive(smem_u32(&sm.q_full[u & 1]));
-                        if (u == 0) mbar_arrive(smem_u32(&sm.q_taken));
+                    if (sub == 0) {
+                        sm.text[u & 1][rr] = make_float2(mm, real ? zz : 1.f);
+                        mbar_arrive(smem_u32(&sm.text_full[u & 1]));
                     }
                 }
             }
@@ -652,7 +692,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         st_async_f32x2(peer_smem(smem_u32(&sm.stats[par][rank][r]), peer), a.x, a.y,
                                        peer_smem(smem_u32(&sm.exchange[par]), peer));
                     }
-                    ok = mbar_wait_cluster(smem_u32(&sm.exchange[par]), (u >> 1) & 1, abort_flag, p.status, 29);
+                    ok = mbar_wait(smem_u32(&sm.text_full[par]), (u >> 1) & 1, abort_flag, p.status, 33) &&
+                         mbar_wait_cluster(smem_u32(&sm.exchange[par]), (u >> 1) & 1, abort_flag, p.status, 29);
                     __syncwarp();
                     if (lane < kRows) {
                         // the largest first, so that the blocks' exponentials do not wait for one another
@@ -712,12 +753,16 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
     }
 
     __syncthreads();
-    if (sm.abort) __nanosleep(100000);   // gave up: whatever neighbours still send lands before the block ends
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, kSlots * kRows);
     }
-    cluster_sync_all();
+    // A block that has had its last unit's sums from every other has all that will ever be sent to it, and may end.  One that
+    // gave up waits for the others (those that have ended count as arrived): what they still send lands before it ends.
+    if (sm.abort) {
+        __nanosleep(100000);
+        cluster_sync_all();
+    }
 }
 
 // Stands in for the kernel above in occupancy queries (same block, same shared memory): the runtime answers one block
