@@ -14,10 +14,11 @@
 //              registers:  e = exp2(logit - reference) as a tile arrives, written back over the logit, and the
 //              running sum per row; at the end of the stretch the sums meet (warp, block, then cluster through
 //              distributed shared memory), and p = e * F with F = weight / normaliser * exp2(reference - max) per
-//              thread and row: one exponential per logit, no reduction across lanes for Eq. 8.
-// The reference is the thread's first logit of the row.  It need not be the maximum, only near enough for fp32's
-// range: a logit more than 2^24 above it takes its place (the stored values of the earlier tiles are rescaled; rare).
-// A masked key (a logit of minus infinity) is no reference, and scores zero.
+//              warp and row: one exponential per logit, no reduction across lanes for Eq. 8.
+// The reference is the warp's largest logit of the row in its first tile, taken while the next tiles are on their way.  It
+// need not be the maximum, only near enough for fp32's range: when a logit is more than 2^24 above it, the warp's largest
+// takes its place (the stored values of the earlier tiles are rescaled; rare).  A masked key (a logit of minus infinity) is
+// no reference, and scores zero.
 //
 // More than 16 elite rows: the keys are read again (from L2) for every further 16.  The KV groups of a (layer,
 // sequence) either follow one another in the same cluster, each adding to the scores, or - when there are too few
@@ -26,13 +27,15 @@
 // What it replaced (elite kernel, one-pass kernel on mma.sync with a wait between blocks, sum kernel) streamed keys
 // during half of a block's life and took three launches.  Measured, 28 layers of 28 query and 4 KV heads of 128
 // channels: 64 sequences of 2916 tokens 1196 -> 835 to 870 us by the box (6.2 TB/s of keys: at the memory's rate); one of
-// 7290 tokens 75 -> 45 us; four of 6272, a call per layer, 33 -> 15.5 us a call.  A call of one layer is a chain of latencies (us
+// 7290 tokens 75 -> 43 us; four of 6272, a call per layer, 33 -> 14.6 us a call.  A call of one layer is a chain of latencies (us
 // behind the wait for what is before it in the stream): 1.4 until the rows of the first query block are staged, 4.2 until
 // the block is ready, 8.2 until the last tile has been multiplied, 12 at the end; then the sum over groups and the launches'
 // hand-over, 3.  What shortened it from 17: the first rows and tiles are asked into L2 and the addresses worked out ahead of
 // the wait, an idle warp's lanes ask for the window's queries (one thread took 1 us for the 16 copies), the text columns'
 // statistics and the masks are written behind the query block, which does not need them, and no block waits for its
-// cluster at its end: 16.9 -> 15.5 us; image 47.6 -> 45.3.
+// cluster at its end: 16.9 -> 15.5 us; image 47.6 -> 45.3.  A reference per warp (below) left no maxima to take behind the
+// last tile and the factors to one lane a row, and the first tile's exponentials come back beside the exchange: 14.6; 43.2.
+// (The next tile's beside the sums of one: 104 bytes of spills, image 53.)
 //
 // With up to eight tiles per block the tensor memory holds two units of work and the tensor core runs ahead of the
 // epilogue; with up to sixteen the other block of the SM fills the gap.  All waits are bounded.
@@ -66,8 +69,9 @@ struct ClusterSmem {   // small state behind the ring and the query block
     uint64_t q_full[2], text_full[2], meta_empty[2], q_free, q_all, q_taken;
     uint64_t acc_full[kSlots], acc_empty[2], exchange[2];
     float2 stats[2][kMaxCluster][kRows];   // (max, sum) of every block of the cluster
-    float2 warp_stats[2][4][kRows];
-    float2 fin[4][kRows];                  // per epilogue warp: (max, 2^64 weight / normaliser)
+    alignas(16) float warp_ref[2][4][kRows];
+    float warp_sum[2][4][kRows];
+    alignas(16) float fin[4][kRows];                   // per epilogue warp: 2^64 times the factor of its rows
     float2 text[2][kRows];
     float coef[2][kRows];
     int2 meta[2];                          // rows of the unit, last unit of its group
@@ -587,7 +591,13 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         const bool valid = key0 + t * 128 + own < p.Nv;
                         if (t == 0) {
 #pragma unroll
-                            for (int r = 0; r < kRows; ++r) m[r] = valid ? fmaxf(x[r] * p.sl2, kNegBig) : kNegBig;   // (a masked key: -inf)
+                            for (int q = 0; q < 4; ++q) {
+                                if (q < quads) {
+#pragma unroll
+                                    for (int r = 4 * q; r < 4 * q + 4; ++r)   // (a masked key: -inf)
+                                        m[r] = fmaxf(warp_max(valid ? x[r] * p.sl2 : -INFINITY), kNegBig);
+                                }
+                            }
                         }
                         float top = -INFINITY;
 #pragma unroll
@@ -603,8 +613,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         }
                         if (__any_sync(0xffffffffu, top > kRescale)) {
                             // Move the references of the rows that outgrew them and rescale what is stored.  The new one is
-                            // the logit itself, read again: reference plus difference has only the bits that are left beside
-                            // the old reference, which may be a masked key's.
+                            // the warp's largest logit itself, read again: reference plus difference has only the bits that
+                            // are left beside the old reference, which may be a masked key's.
                             tmem_st_wait();
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
@@ -614,22 +624,23 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
 #pragma unroll
                                     for (int j = 0; j < 4; ++j) {
                                         const int r = 4 * q + j;
-                                        const bool move = x[r] > kRescale;
-                                        const float mn = move ? raw[j] * p.sl2 : m[r];
+                                        const bool move = warp_max(x[r]) > kRescale;
+                                        const float y = tail && !valid ? -INFINITY : raw[j] * p.sl2, top_r = warp_max(y);
+                                        const float mn = move ? top_r : m[r];
                                         fac[j] = move ? fast_exp2(m[r] - mn) : 1.f;
                                         z[r] *= fac[j];
-                                        // (what is left beside it: the rounding of the product, nothing of a masked key's 1e29)
+                                        // (beside a masked key's 1e29 nothing is left of a difference but the product's rounding)
                                         const float d = fmaf(raw[j], p.sl2, -mn);
-                                        if (move) x[r] = fabsf(d) > 1.f ? 0.f : d;
+                                        if (move) x[r] = y == -INFINITY ? y : (d > 1.f || (d < -1.f && y == mn)) ? 0.f : d;
                                         m[r] = mn;
                                     }
 #pragma unroll 1
                                     for (int t2 = 0; t2 < t; ++t2) {
-                                        float y[4];
-                                        tmem_ld4(base + t2 * kRows + 4 * q, y);
+                                        float o[4];
+                                        tmem_ld4(base + t2 * kRows + 4 * q, o);
 #pragma unroll
-                                        for (int j = 0; j < 4; ++j) y[j] *= fac[j];
-                                        tmem_st4(base + t2 * kRows + 4 * q, y);
+                                        for (int j = 0; j < 4; ++j) o[j] *= fac[j];
+                                        tmem_st4(base + t2 * kRows + 4 * q, o);
                                     }
                                 }
                             }
@@ -648,14 +659,10 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     }
 
                     // ---- (max, sum) of every row: warp, block, cluster ----
-                    float top_mine = kNegBig;   // lanes 2r, 2r + 1 end up with row r
+                    if (lane == 0) {
 #pragma unroll
-                    for (int r = 0; r < kRows; ++r) {
-                        if ((r >> 2) < quads) {
-                            const float top_r = warp_max(m[r]);
-                            z[r] *= fast_exp2(m[r] - top_r);
-                            if ((lane >> 1) == r) top_mine = top_r;
-                        }
+                        for (int q = 0; q < 4; ++q)
+                            reinterpret_cast<float4 *>(sm.warp_ref[par][ew])[q] = make_float4(m[4 * q], m[4 * q + 1], m[4 * q + 2], m[4 * q + 3]);
                     }
                     float s8[8], s4[4], s2[2];   // 16 sums over 32 lanes: halves of the rows change hands
 #pragma unroll
@@ -675,21 +682,20 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     }
                     float s1 = (lane & 2 ? s2[1] : s2[0]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? s2[0] : s2[1], 2);
                     s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
-                    if ((lane & 1) == 0) sm.warp_stats[par][ew][lane >> 1] = make_float2(top_mine, s1);
+                    if ((lane & 1) == 0) sm.warp_sum[par][ew][lane >> 1] = s1;
                     tmem_st_wait();
                     leave = !named_bar_and(1, kEpiThreads, ok);
                     if (leave) break;
+                    float xa[kRows];   // the exponentials come back beside the exchange
+                    tmem_ld16_issue(base, xa);
                     if ((et >> 4) < plan.cluster) {
                         const int r = et & 15, peer = et >> 4;
-                        float2 a = make_float2(kNegBig, 0.f);
+                        float top = kNegBig, sum = 0.f;
 #pragma unroll
-                        for (int w2 = 0; w2 < 4; ++w2) a.x = fmaxf(a.x, sm.warp_stats[par][w2][r].x);
+                        for (int w2 = 0; w2 < 4; ++w2) top = fmaxf(top, sm.warp_ref[par][w2][r]);
 #pragma unroll
-                        for (int w2 = 0; w2 < 4; ++w2) {
-                            const float2 o = sm.warp_stats[par][w2][r];
-                            a.y = fmaf(o.y, fast_exp2(o.x - a.x), a.y);
-                        }
-                        st_async_f32x2(peer_smem(smem_u32(&sm.stats[par][rank][r]), peer), a.x, a.y,
+                        for (int w2 = 0; w2 < 4; ++w2) sum = fmaf(sm.warp_sum[par][w2][r], fast_exp2(sm.warp_ref[par][w2][r] - top), sum);
+                        st_async_f32x2(peer_smem(smem_u32(&sm.stats[par][rank][r]), peer), top, sum,
                                        peer_smem(smem_u32(&sm.exchange[par]), peer));
                     }
                     ok = mbar_wait(smem_u32(&sm.text_full[par]), (u >> 1) & 1, abort_flag, p.status, 33) &&
@@ -698,6 +704,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     if (lane < kRows) {
                         // the largest first, so that the blocks' exponentials do not wait for one another
                         const float2 tx = sm.text[par][lane];
+                        const float ref = sm.warp_ref[par][ew][lane];
                         float mx = tx.x;
                         for (int c = 0; c < plan.cluster; ++c) mx = fmaxf(mx, sm.stats[par][c][lane].x);
                         float sum = tx.y * fast_exp2(tx.x - mx);
@@ -706,28 +713,25 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                             const float2 o = sm.stats[par][c][lane];
                             sum = fmaf(o.y, fast_exp2(o.x - mx), sum);
                         }
-                        sm.fin[ew][lane] = make_float2(mx, sm.coef[par][lane] / sum * kScaleUp);
+                        // 2^64 times the factor: where a warp's reference is 2^126 below the row's maximum, its keys may still be
+                        // 2^24 above the reference and their scores in range.  (Exact: powers of two, and the sum in the exponent
+                        // loses no bits where it is taken.)
+                        const float f = sm.coef[par][lane] / sum * kScaleUp, below = ref - mx;
+                        const bool far = below < -100.f;
+                        sm.fin[ew][lane] = (far ? f * (1.f / kScaleUp) : f) * fast_exp2(far ? below + 64.f : below);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&sm.meta_empty[par]));
 #pragma unroll
-                    for (int r = 0; r < kRows; ++r) {
-                        // 2^64 times the factor: where a thread's reference is 2^126 below the row's maximum, its keys may still
-                        // be 2^24 above the reference and their scores in range.  (Exact: powers of two, and the sum in the
-                        // exponent loses no bits where it is taken.)
-                        const float2 f = sm.fin[ew][r];
-                        const float below = m[r] - f.x;
-                        const bool far = below < -100.f;
-                        m[r] = (far ? f.y * (1.f / kScaleUp) : f.y) * fast_exp2(far ? below + 64.f : below);
+                    for (int q = 0; q < 4; ++q) {
+                        const float4 f = reinterpret_cast<const float4 *>(sm.fin[ew])[q];
+                        m[4 * q] = f.x; m[4 * q + 1] = f.y; m[4 * q + 2] = f.z; m[4 * q + 3] = f.w;
                     }
                     __syncwarp();
 
-                    // ---- Eq. 8: one key per thread and tile ----
-                    for (int t = 0; t < T; ++t) {
-                        float x[kRows];
-                        tmem_ld16_issue(base + t * kRows, x);
+                    // ---- Eq. 8: one key per thread and tile, the next tile's values on their way ----
+                    auto weigh = [&](const float (&x)[kRows], int t) {
                         const int key = key0 + t * 128 + own;
-                        tmem_ld_wait(x);
                         float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
@@ -743,6 +747,12 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                             if (add) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(out + key), "f"(v) : "memory");
                             else out[key] = v;
                         }
+                    };
+#pragma unroll 1
+                    for (int t = 0; t < T; ++t) {
+                        tmem_ld_wait(xa);
+                        weigh(xa, t);
+                        if (t + 1 < T) tmem_ld16_issue(base + (t + 1) * kRows, xa);
                     }
                     tc_fence_before();
                     __syncwarp();
