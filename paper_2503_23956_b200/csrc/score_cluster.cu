@@ -27,7 +27,7 @@
 // What it replaced (elite kernel, one-pass kernel on mma.sync with a wait between blocks, sum kernel) streamed keys
 // during half of a block's life and took three launches.  Measured, 28 layers of 28 query and 4 KV heads of 128
 // channels: 64 sequences of 2916 tokens 1196 -> 835 to 870 us by the box (6.2 TB/s of keys: at the memory's rate); one of
-// 7290 tokens 75 -> 43 us; four of 6272, a call per layer, 33 -> 14.6 us a call.  A call of one layer is a chain of latencies (us
+// 7290 tokens 75 -> 42.6 us; four of 6272, a call per layer, 33 -> 14.3 us a call.  A call of one layer is a chain of latencies (us
 // behind the wait for what is before it in the stream): 1.4 until the rows of the first query block are staged, 4.2 until
 // the block is ready, 8.2 until the last tile has been multiplied, 12 at the end; then the sum over groups and the launches'
 // hand-over, 3.  What shortened it from 17: the first rows and tiles are asked into L2 and the addresses worked out ahead of
@@ -321,7 +321,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
             const uint4 *q = reinterpret_cast<const uint4 *>(s_k + (p.W + hl) * C::KS);
             const uint4 *kk = reinterpret_cast<const uint4 *>(s_k + w * C::KS);
             float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 8
+            // (not unrolled: a block passes here first with its instructions still to be fetched, and 7 KB of them took longer
+            // than the loop does: an image 43.2 -> 42.6 us)
+#pragma unroll 1
             for (int c = 0; c < D / 8; ++c) {
                 const uint4 a = q[c], bb = kk[c];
                 a0 = fmaf(bf16lo(a.x), bf16lo(bb.x), a0); a1 = fmaf(bf16hi(a.x), bf16hi(bb.x), a1);
@@ -706,6 +708,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         const float2 tx = sm.text[par][lane];
                         const float ref = sm.warp_ref[par][ew][lane];
                         float mx = tx.x;
+#pragma unroll 4
                         for (int c = 0; c < plan.cluster; ++c) mx = fmaxf(mx, sm.stats[par][c][lane].x);
                         float sum = tx.y * fast_exp2(tx.x - mx);
 #pragma unroll 4
