@@ -48,10 +48,9 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *s_warp
 // The chain of latencies is what it costs.  Four 256-bin passes over shared memory took 14 us for 28 regions of 7290
 // tokens and 47 us for 1792 of 2916 (512 threads); this takes 6 and 20.
 template <int T, int PER>
-__global__ void __launch_bounds__(T, T == 256 ? 5 : T == 512 ? 2 : 1) select_kernel(const float *__restrict__ scores, const int32_t *__restrict__ budgets,
-                                                   const int64_t *__restrict__ offsets, int n_visual, int n_text, int slack,
-                                                   int64_t first_row, int32_t *__restrict__ kept, int64_t kept_cap,
-                                                   uint32_t *status) {
+__device__ __forceinline__ void select_region(int r, const float *__restrict__ scores, const int32_t *__restrict__ budgets,
+                                              const int64_t *__restrict__ offsets, int n_visual, int n_text, int slack,
+                                              int64_t first_row, int32_t *__restrict__ kept, int64_t kept_cap, uint32_t *status) {
     constexpr int WARPS = T / 32;
     __shared__ uint32_t s_hist[kSelBins];
     __shared__ uint32_t s_warp[32], s_lo[32], s_hi[32];
@@ -60,11 +59,6 @@ __global__ void __launch_bounds__(T, T == 256 ? 5 : T == 512 ? 2 : 1) select_ker
     __shared__ uint32_t s_n;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    // What is before in the stream has ended when this kernel lets the gather kernel start: that one copies its text
-    // rows by the budgets at once, and waits before it reads the lists.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int r = blockIdx.x;
     const int k = budgets[r];
     // the region's list starts after the kept rows of the regions before it; budgets and offsets come from
     // device memory, so a pair that does not fit the list buffer is reported instead of followed
@@ -220,6 +214,21 @@ __global__ void __launch_bounds__(T, T == 256 ? 5 : T == 512 ? 2 : 1) select_ker
     }
 }
 
+template <int T, int PER>
+__global__ void __launch_bounds__(T, T == 256 ? 5 : T == 512 ? 2 : 1) select_kernel(const float *__restrict__ scores, const int32_t *__restrict__ budgets,
+                                                   const int64_t *__restrict__ offsets, int n_regions, int n_visual, int n_text,
+                                                   int slack, int64_t first_row, int32_t *__restrict__ kept, int64_t kept_cap,
+                                                   uint32_t *status) {
+    // What is before in the stream has ended when this kernel lets the gather kernel start: that one copies its text
+    // rows by the budgets at once, and waits before it reads the lists.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int r = blockIdx.x; r < n_regions; r += gridDim.x) {
+        select_region<T, PER>(r, scores, budgets, offsets, n_visual, n_text, slack, first_row, kept, kept_cap, status);
+        __syncthreads();   // the shared memory has been read
+    }
+}
+
 struct GatherParams {
     const uint16_t *k, *v;
     int64_t s_layer, s_batch, s_head, s_token;
@@ -228,7 +237,7 @@ struct GatherParams {
     const int32_t *lens;
     const int32_t *budgets;
     const int32_t *kept;
-    int64_t rows_cap;  // rows covered by the launch
+    int text_blocks;   // blocks of text rows; those behind them take the kept rows
     int64_t total_rows;  // rows the output buffers hold
     int64_t kept_cap;    // entries the kept-list buffer holds
     uint32_t *status;
@@ -239,17 +248,17 @@ struct GatherParams {
 
 constexpr int kGatherThreads = 256;
 constexpr int kGatherRowsPerWarp = 4;
+constexpr int kGatherRowsPerBlock = kGatherThreads / 32 * kGatherRowsPerWarp;
 
 // Copies the rows of the ragged cache: for region r first the kept visual rows in ascending token order, then
 // the text rows (Algorithm 1's C^l = Concat(K_v[kept], K_t)).  A warp moves four rows at a time.
-// The text rows need no selection result - their place follows from the budgets alone - so they are copied
-// before the kernel waits for its predecessor in the stream (the selection kernel, which releases its
-// dependents at once): that part of the traffic runs beside the selection, which occupies one CTA per region
-// and is bound by latency, not by bandwidth.
+// The text rows need no selection result - their place follows from the budgets alone - so the first blocks, which
+// copy them, do not wait for the predecessor in the stream (the selection kernel, which releases its dependents when its
+// last block has started): that part of the traffic runs beside the selection, which is bound by latency, not by
+// bandwidth.  When every block copied some text rows and then waited, the first ones on the SMs held up the text rows of the
+// others: 28 layers of 7290 + 128 tokens 32.3 -> 30.7 us a pass with the budgets.  Bound by the memory.
 __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams p) {
     const int lane = threadIdx.x & 31;
-    const int64_t warp0 = ((int64_t)blockIdx.x * kGatherThreads + threadIdx.x) >> 5;
-    const int64_t row_step = (int64_t)gridDim.x * (kGatherThreads / 32) * kGatherRowsPerWarp;
     const int n_regions = p.L * p.B * p.Hc;       // cells
     const int row_heads = p.Hc > 1 ? 1 : p.Hkv;   // KV heads in one row of the ragged cache
     const int vec_per_head = p.d / 8;             // 16-byte vectors per head slice
@@ -282,13 +291,14 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams 
         }
     };
 
-    // ---- text rows: row j of region r goes to offsets[r] + budgets[r] + j ----
-    const int n_text_rows = n_regions * p.Nt;   // below 2^31: the cache has fewer rows than that
-    for (int64_t first = warp0 * kGatherRowsPerWarp; first < n_text_rows; first += row_step) {
+    if ((int)blockIdx.x < p.text_blocks) {
+        // ---- text rows: row j of region r goes to offsets[r] + budgets[r] + j ----
+        const int n_text_rows = n_regions * p.Nt;   // below 2^31: the cache has fewer rows than that
+        const int first = (int)blockIdx.x * kGatherRowsPerBlock + (threadIdx.x >> 5) * kGatherRowsPerWarp;
         int64_t src_off[kGatherRowsPerWarp], dst_row[kGatherRowsPerWarp];
 #pragma unroll
         for (int i = 0; i < kGatherRowsPerWarp; ++i) {
-            const int idx = (int)first + i;
+            const int idx = first + i;
             dst_row[i] = -1;
             src_off[i] = 0;
             if (idx >= n_text_rows) continue;
@@ -299,6 +309,7 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams 
             else dst_row[i] = dst;
         }
         copy_rows(src_off, dst_row);
+        return;
     }
 
     // ---- kept visual rows: where they go follows from the offsets, what goes there from the selection's lists ----
@@ -309,8 +320,8 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams 
         if (threadIdx.x == 0) atomicExch(p.status, kStatusInconsistent);
         n_kept = 0;
     }
-    bool waited = false;
-    for (int64_t first = warp0 * kGatherRowsPerWarp; first < n_kept; first += row_step) {
+    const int64_t first = (int64_t)((int)blockIdx.x - p.text_blocks) * kGatherRowsPerBlock + (threadIdx.x >> 5) * kGatherRowsPerWarp;
+    if (first < n_kept) {
         // Largest r with (kept rows before r) <= first (regions without kept rows are passed over), 32 probes at a
         // time; the further rows are found by walking on.  (A binary search per row and behind the wait
         // took 2 to 6 us of a warp's time.)
@@ -338,8 +349,7 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams 
             region[i] = r;
             dst_row[i] = begin + p.first_row + r * per + (idx - begin);
         }
-        if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
-        waited = true;
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         int tok[kGatherRowsPerWarp];
 #pragma unroll
         for (int i = 0; i < kGatherRowsPerWarp; ++i) tok[i] = first + i < n_kept ? p.kept[first + i] : 0;
@@ -354,8 +364,9 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams 
             }
         }
         copy_rows(src_off, dst_row);
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
     }
-    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 __global__ void append_kernel(uint16_t *k_out, uint16_t *v_out, const int64_t *offsets, int32_t *lens,
@@ -375,7 +386,7 @@ struct SelectArgs {
     const float *scores;
     const int32_t *budgets;
     const int64_t *offsets;
-    int n_visual, n_text, slack;
+    int n_regions, n_visual, n_text, slack;
     int64_t first_row;
     int32_t *kept;
     int64_t kept_cap;
@@ -383,9 +394,9 @@ struct SelectArgs {
 };
 
 template <int T, int PER>
-cudaError_t launch_select(const SelectArgs &a, int regions, cudaStream_t st) {
+cudaError_t launch_select(const SelectArgs &a, int blocks, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)regions);
+    cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(T);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -393,7 +404,7 @@ cudaError_t launch_select(const SelectArgs &a, int regions, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, select_kernel<T, PER>, a.scores, a.budgets, a.offsets, a.n_visual, a.n_text, a.slack,
+    return cudaLaunchKernelEx(&cfg, select_kernel<T, PER>, a.scores, a.budgets, a.offsets, a.n_regions, a.n_visual, a.n_text, a.slack,
                               a.first_row, a.kept, a.kept_cap, a.status);
 }
 
@@ -412,11 +423,21 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
     int dev = 0, sms = 0;
     const int rc = current_device(&dev, &sms);
     if (rc) return rc;
-    const SelectArgs a = {scores, budgets, out->offsets, s->n_visual, s->n_text, s->slack, out->first_row, kept, kept_cap, status};
+    const SelectArgs a = {scores, budgets, out->offsets, LB, s->n_visual, s->n_text, s->slack, out->first_row, kept, kept_cap, status};
     const bool many = LB > sms;
+    // The gather kernel starts when the last block of the selection has.  Where its text rows keep the memory busy for longer
+    // than a selection by 512 threads an SM takes (9 us a region), there are no more blocks than that: the rest of the SM
+    // copies text rows meanwhile.  64 sequences of 2916 + 256 tokens, 28 layers: 692 -> 652 us a pass with the budgets (for
+    // 50 us the memory was idle); with 24 text tokens the selection is what is waited for, and takes 33 us by as many blocks as
+    // there are regions and 54 by these.
+    const double text_us = (double)LB * s->n_text * row_heads_of(s) * s->head_dim * 8 / 6.0e6;
+    auto blocks_of = [&](int threads) {
+        const int few = sms * (512 / threads);
+        return text_us > 9.0 * ((LB + few - 1) / few) ? (LB < few ? LB : few) : LB;
+    };
     cudaError_t e;
-    if (many && s->n_visual <= 256 * 16) e = launch_select<256, 16>(a, LB, st);
-    else if (many && s->n_visual <= 512 * 16) e = launch_select<512, 16>(a, LB, st);
+    if (many && s->n_visual <= 256 * 16) e = launch_select<256, 16>(a, blocks_of(256), st);
+    else if (many && s->n_visual <= 512 * 16) e = launch_select<512, 16>(a, blocks_of(512), st);
     else if (s->n_visual <= 1024 * 8) e = launch_select<1024, 8>(a, LB, st);
     else if (s->n_visual <= 1024 * 16) e = launch_select<1024, 16>(a, LB, st);
     else e = launch_select<1024, 0>(a, LB, st);
@@ -428,22 +449,16 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
     p.k_out = (uint16_t *)out->k; p.v_out = (uint16_t *)out->v;
     p.offsets = out->offsets; p.lens = out->lens; p.budgets = budgets; p.kept = kept;
     p.first_row = out->first_row;
-    p.rows_cap = kept_cap + (int64_t)LB * (s->n_text + s->slack);
     p.total_rows = out->total_rows;
     p.kept_cap = kept_cap;
     p.status = status;
     p.Hc = cells_of(s);
     p.L = s->n_layers; p.B = s->batch; p.Hkv = s->n_kv_heads; p.d = s->head_dim;
     p.Nv = s->n_visual; p.Nt = s->n_text; p.slack = s->slack;
-    const int64_t rows_per_block = (kGatherThreads / 32) * kGatherRowsPerWarp;
-    const int64_t text_rows = (int64_t)LB * s->n_text;
-    const int64_t kept_rows = p.rows_cap - (int64_t)LB * (s->n_text + s->slack);
-    const int64_t most = text_rows > kept_rows ? text_rows : kept_rows;
-    // One block per 32 rows of the longer phase (a grid limited to the resident blocks, each striding through
-    // the rows, measured 20 % slower on the large configurations).  Blocks that start after the selection has
-    // finished pass the wait at once.
-    int64_t blocks = (most + rows_per_block - 1) / rows_per_block;
-    if (blocks < 1) blocks = 1;
+    // One block per 32 rows (a grid limited to the resident blocks, each striding through the rows, measured 20 % slower on
+    // the large configurations).  The text rows' blocks come first and do not wait for the selection; at least one block does.
+    p.text_blocks = (int)(((int64_t)LB * s->n_text + kGatherRowsPerBlock - 1) / kGatherRowsPerBlock);
+    const int64_t blocks = p.text_blocks + (kept_cap > 0 ? (kept_cap + kGatherRowsPerBlock - 1) / kGatherRowsPerBlock : 1);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(kGatherThreads);
