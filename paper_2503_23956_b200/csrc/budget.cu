@@ -80,10 +80,11 @@ __device__ __forceinline__ double warp_bcast(double v, int src) {
     return __shfl_sync(0xffffffffu, v, src);
 }
 
-// Eq. 11 and the integer budgets of one sequence, by one warp.  st/sk/w/share/bud/act are arrays in shared memory
-// over the sequence's cells - its layers, or its (layer, KV head) pairs in per-KV-head mode, layer-major -
+// Eq. 11 of one sequence, by one warp: the floors of the cells' shares, and how many rows are left for the largest fractional
+// parts (returned; the fractions are in share, -1 for cells outside the split).  st/sk/w/share/bud/act are arrays in shared
+// memory over the sequence's cells - its layers, or its (layer, KV head) pairs in per-KV-head mode, layer-major -
 // numbered l = 0 .. n - 1; act flags cells that still take part in the proportional split.
-__device__ void allocate_sequence(const BudgetParams &p, int n, const double *st, const double *sk, double *w,
+__device__ long long split_sequence(const BudgetParams &p, int n, const double *st, const double *sk, double *w,
                                   double *share, unsigned char *act, int *bud) {
     const int L = n, lane = threadIdx.x & 31;
     // across-layer means: one lane, layer order (this fixes the rounding of the sums)
@@ -151,7 +152,10 @@ __device__ void allocate_sequence(const BudgetParams &p, int n, const double *st
     // floors, then the largest fractional parts (ties to the lower layer) take one more row each
     int given = 0;
     for (int l = lane; l < L; l += 32) {
-        if (!act[l]) continue;
+        if (!act[l]) {
+            share[l] = -1.0;
+            continue;
+        }
         const double sh = share[l];
         const int f = (int)floor(sh);
         bud[l] = f;
@@ -161,22 +165,7 @@ __device__ void allocate_sequence(const BudgetParams &p, int n, const double *st
     long long given_all = given;
 #pragma unroll
     for (int s = 16; s > 0; s >>= 1) given_all += __shfl_xor_sync(0xffffffffu, given_all, s);
-    __syncwarp();
-    const long long left = R - given_all;
-    // a layer gets the extra row iff fewer than `left` active layers precede it in the order
-    // (fraction descending, layer ascending): the same set the one-at-a-time selection picks
-    for (int l = lane; l < L; l += 32) {
-        if (!act[l]) continue;
-        const double fr = share[l];
-        long long rank = 0;
-        for (int l2 = 0; l2 < L; ++l2) {
-            if (!act[l2]) continue;
-            const double f2 = share[l2];
-            rank += (f2 > fr) || (f2 == fr && l2 < l);
-        }
-        if (rank < left) bud[l] += 1;
-    }
-    __syncwarp();
+    return R - given_all;
 }
 
 template <int T, int PER>
@@ -252,11 +241,26 @@ __global__ void __launch_bounds__(T, 1024 / T) budget_kernel(BudgetParams p) {
         sk[l] = __ldcg(p.skewness + at(l));
     }
     __syncthreads();
-    if (tid < 32) allocate_sequence(p, n, st, sk, w, share, act, bud);
+    __shared__ long long s_left;
+    if (tid < 32) {
+        const long long left = split_sequence(p, n, st, sk, w, share, act, bud);
+        if (tid == 0) s_left = left;
+    }
     __syncthreads();
+    // A cell gets an extra row iff fewer than `left` cells of the split precede it in the order (fraction descending, cell
+    // ascending): the same set the one-at-a-time selection picks.  By all of the block: n comparisons a cell, which took one
+    // warp 200 us for the 640 cells of a sequence (80 layers, 8 KV heads): 261 -> 62 us a call.
     for (int l = tid; l < n; l += T) {
-        __stcg(p.budgets + at(l), bud[l]);
-        p.lens[at(l)] = bud[l] + p.Nt;
+        const double fr = share[l];
+        int rank = 0;
+#pragma unroll 4
+        for (int l2 = 0; l2 < n; ++l2) {
+            const double f2 = share[l2];
+            rank += (f2 > fr) || (f2 == fr && l2 < l);
+        }
+        const int b_l = bud[l] + (act[l] && rank < s_left);
+        __stcg(p.budgets + at(l), b_l);
+        p.lens[at(l)] = b_l + p.Nt;
     }
     __syncthreads();
     if (tid == 0) {
