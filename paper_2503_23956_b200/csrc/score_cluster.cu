@@ -27,7 +27,7 @@
 // What it replaced (elite kernel, one-pass kernel on mma.sync with a wait between blocks, sum kernel) streamed keys
 // during half of a block's life and took three launches.  Measured, 28 layers of 28 query and 4 KV heads of 128
 // channels: 64 sequences of 2916 tokens 1196 -> 835 to 870 us by the box (6.2 TB/s of keys: at the memory's rate); one of
-// 7290 tokens 75 -> 42.6 us; four of 6272, a call per layer, 33 -> 14.3 us a call.  A call of one layer is a chain of latencies (us
+// 7290 tokens 75 -> 41.4 us; four of 6272, a call per layer, 33 -> 13.9 us a call.  A call of one layer is a chain of latencies (us
 // behind the wait for what is before it in the stream): 1.4 until the rows of the first query block are staged, 4.2 until
 // the block is ready, 8.2 until the last tile has been multiplied, 12 at the end; then the sum over groups and the launches'
 // hand-over, 3.  What shortened it from 17: the first rows and tiles are asked into L2 and the addresses worked out ahead of
@@ -35,7 +35,9 @@
 // statistics and the masks are written behind the query block, which does not need them, and no block waits for its
 // cluster at its end: 16.9 -> 15.5 us; image 47.6 -> 45.3.  A reference per warp (below) left no maxima to take behind the
 // last tile and the factors to one lane a row, and the first tile's exponentials come back beside the exchange: 14.6; 43.2.
-// (The next tile's beside the sums of one: 104 bytes of spills, image 53.)
+// (The next tile's beside the sums of one: 104 bytes of spills, image 53.)  The bound that decides whether a head needs its
+// fp64 sums comes out of the fp32 dot products themselves and no longer from norms taken while the rows were stored: 14.3 ->
+// 13.9; 42.4 -> 41.4.
 //
 // With up to eight tiles per block the tensor memory holds two units of work and the tensor core runs ahead of the
 // epilogue; with up to sixteen the other block of the SM fills the gap.  All waits are bounded.
@@ -121,8 +123,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
     uint8_t *s_q = smem + S * C::TILE_BYTES;
     ClusterSmem &sm = *reinterpret_cast<ClusterSmem *>(s_q + C::Q_BYTES);
     uint16_t *s_k = reinterpret_cast<uint16_t *>(&sm + 1);   // [W][KS] candidate keys, then [G][KS] last queries
-    float *s_logit = reinterpret_cast<float *>(s_k + (p.W + p.G) * C::KS);   // [G][W]
-    float *s_norm = s_logit + p.G * p.W;                                     // 2-norm of every staged row
+    float *s_logit = reinterpret_cast<float *>(s_k + (p.W + p.G) * C::KS);   // [G][W], for W > 32
+    int *s_size = reinterpret_cast<int *>(s_logit + p.G * p.W);              // [G] largest sum of magnitudes of a head, its bits
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank();
@@ -282,7 +284,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
         const int words = (p.W + 31) >> 5;
         bool ok = true;
         uint32_t u = 0;
-        // four vectors per thread from `base` on: loaded, then stored with the norm of every row
+        // four vectors per thread from `base` on: loaded, then stored
         auto load_rows = [&](int grp, int base, uint4 (&v)[4]) {
             const int g = grp % p.Hkv, lb = grp / p.Hkv, l = lb / p.B, b = lb - l * p.B;
             const uint16_t *k_cand = p.k + (int64_t)l * p.s_layer + (int64_t)b * p.s_batch + (int64_t)g * p.s_head +
@@ -301,37 +303,32 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int idx = base + i * kEliteThreads, row = idx / (D / 8), c = idx % (D / 8);
-                const uint32_t w4[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-                float sq = 0.f;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) sq = fmaf(bf16lo(w4[e]), bf16lo(w4[e]), fmaf(bf16hi(w4[e]), bf16hi(w4[e]), sq));
-#pragma unroll
-                for (int sh = 1; sh < D / 8; sh <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, sh);
-                if (idx < n_vec) {
-                    *reinterpret_cast<uint4 *>(s_k + row * C::KS + c * 8) = v[i];
-                    if (c == 0) s_norm[row] = sqrtf(sq + 1e-30f);   // (squares below fp32's range: still a bound)
-                }
+                if (idx < n_vec) *reinterpret_cast<uint4 *>(s_k + row * C::KS + c * 8) = v[i];
             }
         };
         // Eq. 4, last row only: the logit of candidate w for head hl.  The decision of Eq. 5 is defined on fp64 dot
         // products in element order, rounded to fp32.  fp32 dot products settle it wherever the difference to the
         // threshold exceeds what the two can differ by; a head with a candidate closer than that is done again in fp64
         // (about one group in 200).  The fp64 chain alone took 2-4 us of a one-layer call's 19.
-        auto logit_fp32 = [&](int hl, int w) {
+        auto logit_fp32 = [&](int hl, int w, float &size) {   // size: the sum of the products' magnitudes
             const uint4 *q = reinterpret_cast<const uint4 *>(s_k + (p.W + hl) * C::KS);
             const uint4 *kk = reinterpret_cast<const uint4 *>(s_k + w * C::KS);
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
             // (not unrolled: a block passes here first with its instructions still to be fetched, and 7 KB of them took longer
             // than the loop does: an image 43.2 -> 42.6 us)
+            float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
 #pragma unroll 1
             for (int c = 0; c < D / 8; ++c) {
                 const uint4 a = q[c], bb = kk[c];
-                a0 = fmaf(bf16lo(a.x), bf16lo(bb.x), a0); a1 = fmaf(bf16hi(a.x), bf16hi(bb.x), a1);
-                a2 = fmaf(bf16lo(a.y), bf16lo(bb.y), a2); a3 = fmaf(bf16hi(a.y), bf16hi(bb.y), a3);
-                a0 = fmaf(bf16lo(a.z), bf16lo(bb.z), a0); a1 = fmaf(bf16hi(a.z), bf16hi(bb.z), a1);
-                a2 = fmaf(bf16lo(a.w), bf16lo(bb.w), a2); a3 = fmaf(bf16hi(a.w), bf16hi(bb.w), a3);
+                const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float ql = bf16lo(av[e]), qh = bf16hi(av[e]), kl = bf16lo(bv[e]), kh = bf16hi(bv[e]);
+                    a0 = fmaf(ql, kl, a0); a1 = fmaf(qh, kh, a1);
+                    b0 = fmaf(fabsf(ql), fabsf(kl), b0); b1 = fmaf(fabsf(qh), fabsf(kh), b1);
+                }
             }
-            return ((a0 + a1) + (a2 + a3)) * p.scale;
+            size = (b0 + b1) * p.scale;
+            return (a0 + a1) * p.scale;
         };
         auto logit_fp64 = [&](int hl, int w) {
             const uint4 *q = reinterpret_cast<const uint4 *>(s_k + (p.W + hl) * C::KS);
@@ -351,9 +348,10 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
             }
             return __fmul_rn((float)acc, p.scale);
         };
-        // How far (logit - best) can be off in fp32: per logit 34 roundings of the sum and 2 each for the scaled products,
-        // relative to |q| |k| scale (Cauchy-Schwarz), for two logits, plus the norms' own: 2 * 40 / 2^24 and a margin.
-        constexpr float kSlack = 5.5e-6f;
+        // How far (logit - best) can be off in fp32: per logit 66 roundings of the sum and 2 each for the scaled products,
+        // relative to the sum of the products' magnitudes, for two logits: 2 * 68 / 2^24 and a margin, of the head's largest such
+        // sum.  (Products below fp32's range: their sum is off by 128 * 2^-126 at most.)
+        constexpr float kSlack = 9e-6f, kSlackLeast = 1e-30f;
 
         uint4 ahead[4];   // the first vectors of the next group, on their way while this one is worked on
 #pragma unroll
@@ -368,6 +366,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                 const int g = grp % p.Hkv, lb = grp / p.Hkv;
                 const uint16_t *q_lb = p.qw + (int64_t)lb * p.W * p.Hq * D;
                 named_bar(2, kEliteThreads);   // the previous group's keys and masks have been used
+                if (p.W > 32 && et < p.G) s_size[et] = 0;
                 store_rows(et, ahead);
                 if (u == 0) asm volatile("bar.arrive 3, %0;" ::"n"(kEliteThreads + 32) : "memory");
                 for (int base = et + 4 * kEliteThreads; base - et < n_vec; base += 4 * kEliteThreads) {
@@ -387,15 +386,15 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     for (int h0 = 0; h0 < p.G; h0 += per_pass) {
                         const int hl = h0 + et / seg;
                         const bool in = hl < p.G && w < p.W;
-                        float t = in ? logit_fp32(hl, w) : -INFINITY;
-                        float kn = in ? s_norm[w] : 0.f;
+                        float size = 0.f, t = -INFINITY;
+                        if (in) t = logit_fp32(hl, w, size);
                         float top = t;
                         for (int sh = 1; sh < seg; sh <<= 1) {
                             top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, sh));
-                            kn = fmaxf(kn, __shfl_xor_sync(0xffffffffu, kn, sh));
+                            size = fmaxf(size, __shfl_xor_sync(0xffffffffu, size, sh));
                         }
                         float diff = __fsub_rn(t, top);
-                        const bool near = in && !(fabsf(diff - p.ln_alpha) > kSlack * p.scale * s_norm[p.W + hl] * kn);
+                        const bool near = in && !(fabsf(diff - p.ln_alpha) > fmaf(kSlack, size, kSlackLeast));
                         if (__any_sync(0xffffffffu, near)) {
                             t = in ? logit_fp64(hl, w) : -INFINITY;
                             top = t;
@@ -411,14 +410,15 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         sm.mask[i >> 2][i & 3] = left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1 : 0u);
                     }
                 } else {
-                    for (int idx = et; idx < p.G * p.W; idx += kEliteThreads) s_logit[idx] = logit_fp32(idx / p.W, idx % p.W);
+                    for (int idx = et; idx < p.G * p.W; idx += kEliteThreads) {
+                        float size;
+                        s_logit[idx] = logit_fp32(idx / p.W, idx % p.W, size);
+                        atomicMax(s_size + idx / p.W, __float_as_int(size));   // (not negative: ordered like the bits)
+                    }
                     named_bar(2, kEliteThreads);
                     // a warp per head; a warp that has to look closer does its head again by itself
-                    float kn = 0.f;
-                    for (int w = lane; w < p.W; w += 32) kn = fmaxf(kn, s_norm[w]);
-                    kn = warp_max(kn);
                     for (int hl = ew; hl < p.G; hl += 4) {
-                        const float slack = kSlack * p.scale * s_norm[p.W + hl] * kn;
+                        const float slack = fmaf(kSlack, __int_as_float(s_size[hl]), kSlackLeast);
                         for (bool again = true, exact = false; again; exact = true) {
                             float top = -INFINITY;
                             for (int w = lane; w < p.W; w += 32) top = fmaxf(top, s_logit[hl * p.W + w]);
