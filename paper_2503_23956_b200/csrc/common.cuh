@@ -192,6 +192,27 @@ __device__ __forceinline__ float fast_exp2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// The same without the flush: results below 2^-126 are subnormal numbers.  (volatile: stays in the rare branch it is written in)
+__device__ __forceinline__ float subnormal_exp2(float x) {
+    float y;
+    asm volatile("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// x * y + a and x + a, two at a time
+__device__ __forceinline__ float2 fma2(float2 x, float2 y, float2 a) {
+    float2 r;
+    asm("{\n.reg .b64 x, y, a;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nmov.b64 a, {%6, %7};\n"
+        "fma.rn.f32x2 x, x, y, a;\nmov.b64 {%0, %1}, x;\n}\n"
+        : "=f"(r.x), "=f"(r.y) : "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y), "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 add2(float2 x, float2 a) {
+    float2 r;
+    asm("{\n.reg .b64 x, a;\nmov.b64 x, {%2, %3};\nmov.b64 a, {%4, %5};\nadd.rn.f32x2 x, x, a;\nmov.b64 {%0, %1}, x;\n}\n"
+        : "=f"(r.x), "=f"(r.y) : "f"(x.x), "f"(x.y), "f"(a.x), "f"(a.y));
+    return r;
+}
 
 // Merge two (max, sum-of-exp2) pairs of the same softmax row.
 __device__ __forceinline__ void merge_stats(float &m, float &z, float m2, float z2) {

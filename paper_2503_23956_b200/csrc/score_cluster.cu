@@ -18,7 +18,9 @@
 // The reference is the warp's largest logit of the row in its first tile, taken while the next tiles are on their way.  It
 // need not be the maximum, only near enough for fp32's range: when a logit is more than 2^24 above it, the warp's largest
 // takes its place (the stored values of the earlier tiles are rescaled; rare).  A masked key (a logit of minus infinity) is
-// no reference, and scores zero.
+// no reference, and scores zero.  A key 2^126 below its warp's reference has a subnormal exponential, taken without the flush
+// in the same rare branch, so that a score keeps its bits down to 2^-149 (but for the additions of further units and groups
+// in global memory, which flush).
 //
 // More than 16 elite rows: the keys are read again (from L2) for every further 16.  The KV groups of a (layer,
 // sequence) either follow one another in the same cluster, each adding to the scores, or - when there are too few
@@ -62,6 +64,8 @@ constexpr int kEliteThreads = 128, kEpiThreads = 128;
 constexpr int kEliteWarp0 = 4, kEpiWarp0 = 8;
 constexpr int kSmemPerBlock = (228 * 1024) / 2 - 1024;   // two blocks per SM, 1 KB each is the system's
 constexpr float kRescale = 24.f;
+constexpr float kMiddle = 0.5f * (kRescale - 126.f);   // of the exponents that need no care
+constexpr float kFarDown = 7.888609052210118e-31f;   // 2^-100
 constexpr float kScaleUp = 18446744073709551616.f;   // 2^64
 constexpr int kPreloadRows = 128;     // window queries of a group that fit a ring stage
 constexpr int kFirstAhead = 5;        // tiles asked into L2 behind the first full ring
@@ -576,9 +580,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     const int2 meta = sm.meta[par];
                     last = meta.y != 0;
                     const int quads = (meta.x + 3) >> 2;   // rows in use, in fours
-                    float m[kRows], z[kRows];
+                    float m[kRows], z[kRows];   // minus the reference, and the sum of the row
 #pragma unroll
-                    for (int r = 0; r < kRows; ++r) { m[r] = kNegBig; z[r] = 0.f; }
+                    for (int r = 0; r < kRows; ++r) { m[r] = -kNegBig; z[r] = 0.f; }
 
                     // ---- exponentials as the tiles arrive ----
                     for (int t = 0; t < T; ++t) {
@@ -597,23 +601,43 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                                 if (q < quads) {
 #pragma unroll
                                     for (int r = 4 * q; r < 4 * q + 4; ++r)   // (a masked key: -inf)
-                                        m[r] = fmaxf(warp_max(valid ? x[r] * p.sl2 : -INFINITY), kNegBig);
+                                        m[r] = -fmaxf(warp_max(valid ? x[r] * p.sl2 : -INFINITY), kNegBig);
                                 }
                             }
                         }
-                        float top = -INFINITY;
+                        float top = 0.f;
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             if (q < quads) {
 #pragma unroll
-                                for (int r = 4 * q; r < 4 * q + 4; ++r) {
-                                    x[r] = fmaf(x[r], p.sl2, -m[r]);
-                                    if (tail && !valid) x[r] = -INFINITY;
-                                    top = fmaxf(top, x[r]);
+                                for (int r = 4 * q; r < 4 * q + 4; r += 2) {
+                                    const float2 y = fma2(make_float2(x[r], x[r + 1]), make_float2(p.sl2, p.sl2), make_float2(m[r], m[r + 1]));
+                                    x[r] = y.x; x[r + 1] = y.y;
+                                    const float2 o = add2(y, make_float2(-kMiddle, -kMiddle));
+                                    top = fmaxf(top, fmaxf(fabsf(o.x), fabsf(o.y)));
                                 }
                             }
                         }
-                        if (__any_sync(0xffffffffu, top > kRescale)) {
+                        if (tail) {   // (volatile: a branch, and not sixteen selects in every tile)
+#pragma unroll
+                            for (int r = 0; r < kRows; ++r) {
+                                asm volatile("" : "+f"(x[r]));
+                                x[r] = valid ? x[r] : -INFINITY;
+                            }
+                        }
+                        // Rare: a reference has to move, or the exponential of a key 2^126 below its warp's reference is a subnormal
+                        // number.  One bound covers both: -126 <= x <= 24.  (With a minimum beside the maximum and the products one at a
+                        // time an image took 43.4 us; so 41.6, as without the lower bound.)
+                        bool rare = __any_sync(0xffffffffu, valid && top > kRescale - kMiddle);
+                        if (rare) {   // not for keys that score zero in all rows (a third of the keys masked: 42.6 us, else 47)
+                            float most = -INFINITY;
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                if (q < quads) most = fmaxf(most, fmaxf(fmaxf(x[4 * q], x[4 * q + 1]), fmaxf(x[4 * q + 2], x[4 * q + 3])));
+                            }
+                            rare = __any_sync(0xffffffffu, top > kRescale - kMiddle && most > -150.f);
+                        }
+                        if (rare) {
                             // Move the references of the rows that outgrew them and rescale what is stored.  The new one is
                             // the warp's largest logit itself, read again: reference plus difference has only the bits that
                             // are left beside the old reference, which may be a masked key's.
@@ -628,22 +652,42 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                                         const int r = 4 * q + j;
                                         const bool move = warp_max(x[r]) > kRescale;
                                         const float y = tail && !valid ? -INFINITY : raw[j] * p.sl2, top_r = warp_max(y);
-                                        const float mn = move ? top_r : m[r];
-                                        fac[j] = move ? fast_exp2(m[r] - mn) : 1.f;
-                                        z[r] *= fac[j];
+                                        const float mn = move ? top_r : -m[r];
+                                        // (a stored value may be 2^24, so a factor below 2^-126 still counts: it is taken 2^100 times
+                                        // larger, with a minus for a mark, and these rows go down by that in a second round)
+                                        const float below = -m[r] - mn;
+                                        fac[j] = !move ? 1.f : below < -100.f ? -fast_exp2(below + 100.f) : fast_exp2(below);
+                                        z[r] *= fabsf(fac[j]);
+                                        if (fac[j] < 0.f) z[r] *= kFarDown;
                                         // (beside a masked key's 1e29 nothing is left of a difference but the product's rounding)
                                         const float d = fmaf(raw[j], p.sl2, -mn);
                                         if (move) x[r] = y == -INFINITY ? y : (d > 1.f || (d < -1.f && y == mn)) ? 0.f : d;
-                                        m[r] = mn;
+                                        m[r] = -mn;
                                     }
 #pragma unroll 1
-                                    for (int t2 = 0; t2 < t; ++t2) {
-                                        float o[4];
-                                        tmem_ld4(base + t2 * kRows + 4 * q, o);
+                                    while (__any_sync(0xffffffffu, fminf(fminf(fac[0], fac[1]), fminf(fac[2], fac[3])) < 1.f)) {
+#pragma unroll 1
+                                        for (int t2 = 0; t2 < t; ++t2) {
+                                            float o[4];
+                                            tmem_ld4(base + t2 * kRows + 4 * q, o);
 #pragma unroll
-                                        for (int j = 0; j < 4; ++j) o[j] *= fac[j];
-                                        tmem_st4(base + t2 * kRows + 4 * q, o);
+                                            for (int j = 0; j < 4; ++j) o[j] *= fabsf(fac[j]);
+                                            tmem_st4(base + t2 * kRows + 4 * q, o);
+                                        }
+                                        tmem_st_wait();   // what was stored is read again
+#pragma unroll
+                                        for (int j = 0; j < 4; ++j) fac[j] = fac[j] < 0.f ? kFarDown : 1.f;
                                     }
+                                }
+                            }
+#pragma unroll
+                            for (int r = 0; r < kRows; ++r) x[r] = subnormal_exp2(x[r]);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                if (q < quads) {
+#pragma unroll
+                                    for (int r = 4 * q; r < 4 * q + 4; ++r) x[r] = fast_exp2(x[r]);
                                 }
                             }
                         }
@@ -651,9 +695,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                         for (int q = 0; q < 4; ++q) {
                             if (q < quads) {
 #pragma unroll
-                                for (int r = 4 * q; r < 4 * q + 4; ++r) {
-                                    x[r] = fast_exp2(x[r]);
-                                    z[r] += x[r];
+                                for (int r = 4 * q; r < 4 * q + 4; r += 2) {
+                                    const float2 s2 = add2(make_float2(z[r], z[r + 1]), make_float2(x[r], x[r + 1]));
+                                    z[r] = s2.x; z[r + 1] = s2.y;
                                 }
                             }
                         }
@@ -664,7 +708,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     if (lane == 0) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            reinterpret_cast<float4 *>(sm.warp_ref[par][ew])[q] = make_float4(m[4 * q], m[4 * q + 1], m[4 * q + 2], m[4 * q + 3]);
+                            reinterpret_cast<float4 *>(sm.warp_ref[par][ew])[q] = make_float4(-m[4 * q], -m[4 * q + 1], -m[4 * q + 2], -m[4 * q + 3]);
                     }
                     float s8[8], s4[4], s2[2];   // 16 sums over 32 lanes: halves of the rows change hands
 #pragma unroll

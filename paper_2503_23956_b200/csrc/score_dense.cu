@@ -90,21 +90,6 @@ __device__ __forceinline__ void for_each_step(const ScoreParams &p, const DenseP
     }
 }
 
-// x = x * s + a and x = x * y + a, two at a time
-__device__ __forceinline__ float2 fma2(float2 x, float2 y, float2 a) {
-    float2 r;
-    asm("{\n.reg .b64 x, y, a;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nmov.b64 a, {%6, %7};\n"
-        "fma.rn.f32x2 x, x, y, a;\nmov.b64 {%0, %1}, x;\n}\n"
-        : "=f"(r.x), "=f"(r.y) : "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y), "f"(a.x), "f"(a.y));
-    return r;
-}
-__device__ __forceinline__ float2 add2(float2 x, float2 a) {
-    float2 r;
-    asm("{\n.reg .b64 x, a;\nmov.b64 x, {%2, %3};\nmov.b64 a, {%4, %5};\nadd.rn.f32x2 x, x, a;\nmov.b64 {%0, %1}, x;\n}\n"
-        : "=f"(r.x), "=f"(r.y) : "f"(x.x), "f"(x.y), "f"(a.x), "f"(a.y));
-    return r;
-}
-
 __device__ __forceinline__ float2 pair(const uint32_t *x, int j) { return make_float2(__uint_as_float(x[j]), __uint_as_float(x[j + 1])); }
 template <int N> struct Int { static constexpr int value = N; };
 

@@ -135,13 +135,6 @@ def test_scores_near_the_smallest(oracle_mod, n_visual, window, alpha):
     """Keys of 2^-104 of the largest weight, met by threads whose reference is 2^-127 of it: such a reference's own factor is
     below the smallest 32-bit number, the scores are not (5e-32), and a ranking of the tokens depends on them.  The oracle
     is compared above 1e-30 only, so the error of these scores is taken relative to themselves."""
-    unit = np.log(2) * 128 ** 0.5   # a logit of 1 in the log2 domain, in two channels for the bits
-
-    def put(k, tokens, x):
-        hi = torch.tensor(x * unit).to(torch.bfloat16)
-        k[:, :, tokens, :, 0] = hi
-        k[:, :, tokens, :, 1] = (torch.tensor(x * unit) - hi.double()).to(torch.bfloat16)
-
     def edit(k, qw):
         k.zero_()
         qw.zero_()
@@ -155,6 +148,37 @@ def test_scores_near_the_smallest(oracle_mod, n_visual, window, alpha):
     small = want > 2.0 ** -120
     assert small.sum() > want.size // 2
     assert (np.abs(got - want)[small] / want[small]).max() <= 2e-5
+
+
+def put(k, tokens, x):
+    """Keys whose logit is x in the log2 domain where the queries are one in two channels (the second for the bits) and zero
+    in the others."""
+    unit = np.log(2) * 128 ** 0.5
+    hi = torch.tensor(x * unit).to(torch.bfloat16)
+    k[:, :, tokens, :, 0] = hi
+    k[:, :, tokens, :, 1] = (torch.tensor(x * unit) - hi.double()).to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("n_visual,loud", [(300, 10), (9000, 10), (300, 138), (3000, 266), (9000, 266)])
+@pytest.mark.parametrize("below", [104, 124, 127, 135, 147])
+def test_scores_far_below_a_key_of_the_same_warp(oracle_mod, n_visual, loud, below):
+    """Keys of 2^-below of the largest weight, which a key of the same warp has, in its first tile (the reference from the
+    start) or in a later one (the reference moves there), beside a few masked ones.  Subnormal scores are scores too: they are rounded to 2^-149 where
+    an exponential is (weighted by the group's half), in the sum of a group and in the oracle, so two steps for two groups;
+    beside that the 2e-5 of the other cases."""
+    def edit(k, qw):
+        k.zero_()
+        qw.zero_()
+        qw[..., :2] = 1.0
+        put(k, slice(0, n_visual), -float(below))
+        for tile in range(0, n_visual, 384):
+            put(k, slice(tile, min(tile + 128, n_visual)), -127.0)
+        put(k, loud, 0.0)
+        put(k, slice(n_visual, None), -30.0)
+        k[:, :, loud + 3:loud + 6, :, 0] = float("-inf")
+    got, want = masked_case(oracle_mod, edit, n_visual, 2, 0.0)
+    assert ((want > 0).sum(-1) == n_visual - 3).all()
+    assert (np.abs(got.astype(np.float64) - want) <= 2 * 2.0 ** -149 + 2e-5 * want.astype(np.float64)).all()
 
 
 @pytest.mark.parametrize("heads,d,window,alpha,n_visual", [
