@@ -1,7 +1,7 @@
 // aircache_compact: per-region top-k of the importance scores and the gather that packs the kept
 // visual rows and all text rows into the ragged cache (Algorithm 1, second loop); aircache_append (Eq. 2).
 //
-//   select_kernel  one CTA per region.  The k-th largest score by histograms over an order-preserving integer image
+//   select_kernel  one CTA per region, or region after region.  The k-th largest score by histograms over an order-preserving integer image
 //                  of the fp32 scores: 2048 bins over the range the keys really have, then over the bin that holds
 //                  the k-th, until few enough are left to be ranked directly (mostly after one histogram).  Then
 //                  the kept token indices in ascending order, duplicates of the threshold value taken from the
@@ -214,7 +214,9 @@ __device__ __forceinline__ void select_region(int r, const float *__restrict__ s
     }
 }
 
-template <int T, int PER>
+// LOOP: a block takes region after region.  Blocks of 256 threads that take one region have no loop around it: with it they
+// spill (76 bytes of loads), 168 regions of 2000 + 16 tokens 34.1 -> 35.9 us a call.  Those of 512 spill without it.
+template <int T, int PER, bool LOOP>
 __global__ void __launch_bounds__(T, T == 256 ? 5 : T == 512 ? 2 : 1) select_kernel(const float *__restrict__ scores, const int32_t *__restrict__ budgets,
                                                    const int64_t *__restrict__ offsets, int n_regions, int n_visual, int n_text,
                                                    int slack, int64_t first_row, int32_t *__restrict__ kept, int64_t kept_cap,
@@ -223,6 +225,10 @@ __global__ void __launch_bounds__(T, T == 256 ? 5 : T == 512 ? 2 : 1) select_ker
     // rows by the budgets at once, and waits before it reads the lists.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!LOOP) {
+        select_region<T, PER>(blockIdx.x, scores, budgets, offsets, n_visual, n_text, slack, first_row, kept, kept_cap, status);
+        return;
+    }
     for (int r = blockIdx.x; r < n_regions; r += gridDim.x) {
         select_region<T, PER>(r, scores, budgets, offsets, n_visual, n_text, slack, first_row, kept, kept_cap, status);
         __syncthreads();   // the shared memory has been read
@@ -400,7 +406,7 @@ struct SelectArgs {
     uint32_t *status;
 };
 
-template <int T, int PER>
+template <int T, int PER, bool LOOP = false>
 cudaError_t launch_select(const SelectArgs &a, int blocks, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
@@ -411,7 +417,7 @@ cudaError_t launch_select(const SelectArgs &a, int blocks, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, select_kernel<T, PER>, a.scores, a.budgets, a.offsets, a.n_regions, a.n_visual, a.n_text, a.slack,
+    return cudaLaunchKernelEx(&cfg, select_kernel<T, PER, LOOP>, a.scores, a.budgets, a.offsets, a.n_regions, a.n_visual, a.n_text, a.slack,
                               a.first_row, a.kept, a.kept_cap, a.status);
 }
 
@@ -443,8 +449,10 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
         return text_us > 9.0 * ((LB + few - 1) / few) ? (LB < few ? LB : few) : LB;
     };
     cudaError_t e;
-    if (many && s->n_visual <= 256 * 16) e = launch_select<256, 16>(a, blocks_of(256), st);
-    else if (many && s->n_visual <= 512 * 16) e = launch_select<512, 16>(a, blocks_of(512), st);
+    const int select_blocks = many && s->n_visual <= 256 * 16 ? blocks_of(256) : many && s->n_visual <= 512 * 16 ? blocks_of(512) : LB;
+    if (many && s->n_visual <= 256 * 16)
+        e = select_blocks < LB ? launch_select<256, 16, true>(a, select_blocks, st) : launch_select<256, 16>(a, LB, st);
+    else if (many && s->n_visual <= 512 * 16) e = launch_select<512, 16, true>(a, select_blocks, st);
     else if (s->n_visual <= 1024 * 8) e = launch_select<1024, 8>(a, LB, st);
     else if (s->n_visual <= 1024 * 16) e = launch_select<1024, 16>(a, LB, st);
     else e = launch_select<1024, 0>(a, LB, st);
