@@ -442,11 +442,12 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
     // than a selection by 512 threads an SM takes (9 us a region), there are no more blocks than that: the rest of the SM
     // copies text rows meanwhile.  64 sequences of 2916 + 256 tokens, 28 layers: 692 -> 652 us a pass with the budgets (for
     // 50 us the memory was idle); with 24 text tokens the selection is what is waited for, and takes 33 us by as many blocks as
-    // there are regions and 54 by these.
+    // there are regions and 54 by these.  From twice as many regions on: fewer leave text rows their room anyway, and a
+    // second round costs more (300 regions of 4096 + 95 tokens 104.4 us by a block each, 109.8; 300 of 4097 + 140: 118.2, 114.5).
     const double text_us = (double)LB * s->n_text * row_heads_of(s) * s->head_dim * 8 / 6.0e6;
     auto blocks_of = [&](int threads) {
         const int few = sms * (512 / threads);
-        return text_us > 9.0 * ((LB + few - 1) / few) ? (LB < few ? LB : few) : LB;
+        return LB >= 2 * few && text_us > 9.0 * ((LB + few - 1) / few) ? few : LB;
     };
     cudaError_t e;
     const int select_blocks = many && s->n_visual <= 256 * 16 ? blocks_of(256) : many && s->n_visual <= 512 * 16 ? blocks_of(512) : LB;

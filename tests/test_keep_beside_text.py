@@ -1,6 +1,6 @@
-"""Selection by fewer blocks than regions, beside the copying of many text rows: blocks of 256 and 512 threads that take two
-regions one after the other, and as many regions as blocks.  Lists and rows against a library sort and plain indexing
-(whole numbers and copies: equal)."""
+"""Copying of text rows beside the selection: selection by fewer blocks than regions (blocks of 256 and 512 threads that take
+two regions one after the other, and as many regions as blocks), and text rows beside it.  Lists and rows against a library
+sort and plain indexing (whole numbers and copies: equal)."""
 import pytest
 import torch
 
@@ -11,19 +11,13 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.mark.parametrize("layers,batch,d,n_visual,n_text", [
-    (19, 16, 128, 300, 60),     # 304 regions, 256 threads
-    (37, 8, 128, 4096, 50),     # 296 regions
-    (30, 5, 64, 4097, 260),     # 150 regions, 512 threads
-    (37, 4, 64, 4500, 140)])    # 148 regions: a block of 1024 threads each
-def test_compaction_with_many_text_rows(layers, batch, d, n_visual, n_text):
-    heads = 8
-    wl = Workload("text", layers, heads, heads, d, batch=batch, n_visual=n_visual, n_text=n_text, ratio=0.07, steps=1, window=2)
+def check_compaction(layers, batch, heads, d, n_visual, n_text, ratio, per_head=0):
+    wl = Workload("text", layers, heads, heads, d, batch=batch, n_visual=n_visual, n_text=n_text, ratio=ratio, steps=1, window=2)
     gen = torch.Generator(device=DEV).manual_seed(n_visual)
     full = [torch.empty((layers, batch, heads, n_visual + n_text, d), dtype=torch.bfloat16, device=DEV).normal_(generator=gen)
             for _ in range(2)]
-    scores = torch.exp(torch.randn((layers, batch, n_visual), generator=gen, device=DEV))
-    gp = GpuPath(wl, device=DEV)
+    gp = GpuPath(wl, device=DEV, per_kv_head=per_head)
+    scores = torch.exp(torch.randn(tuple(gp.scores.shape), generator=gen, device=DEV))
     gp.set_full(*full)
     gp.budget(scores=scores)
     for _ in range(2):
@@ -34,12 +28,25 @@ def test_compaction_with_many_text_rows(layers, batch, d, n_visual, n_text):
     assert gp.status() == 0
     order = torch.sort(scores.view(-1, n_visual), dim=1, descending=True, stable=True).indices
     budgets, offsets = gp.budgets.view(-1).tolist(), gp.offsets.tolist()
+    cells = heads if per_head else 1
     at = 0
     for r, k in enumerate(budgets):
         kept = torch.sort(order[r, :k]).values
         assert torch.equal(gp.kept[at:at + k].long(), kept)
         at += k
         rows = torch.cat([kept, torch.arange(n_visual, n_visual + n_text, device=DEV)])
+        l, b, g = r // cells // batch, r // cells % batch, r % cells
         for have, src in ((gp.k_c, full[0]), (gp.v_c, full[1])):
-            want = src[r // batch, r % batch][:, rows].transpose(0, 1)
-            assert torch.equal(have[offsets[r]:offsets[r] + k + n_text], want)
+            want = src[l, b, g:g + 1 if per_head else heads][:, rows].transpose(0, 1)
+            assert torch.equal(have[offsets[r]:offsets[r] + k + n_text].view(-1), want.reshape(-1))
+
+
+@pytest.mark.parametrize("layers,batch,d,n_visual,n_text", [
+    (19, 16, 128, 300, 60),     # 304 regions, 256 threads
+    (37, 8, 128, 4096, 50),     # 296 regions
+    (37, 16, 128, 2000, 40),    # 592 regions by 296 blocks: exactly two each
+    (30, 10, 128, 4097, 100),   # 300 regions by 148 blocks of 512 threads
+    (30, 5, 64, 4097, 260),     # 150 regions, 512 threads
+    (37, 4, 64, 4500, 140)])    # 148 regions: a block of 1024 threads each
+def test_compaction_with_many_text_rows(layers, batch, d, n_visual, n_text):
+    check_compaction(layers, batch, 8, d, n_visual, n_text, 0.07)
