@@ -6,8 +6,8 @@
 //                  the k-th, until few enough are left to be ranked directly (mostly after one histogram).  Then
 //                  the kept token indices in ascending order, duplicates of the threshold value taken from the
 //                  lowest indices, by ballots and one scan.
-//   gather_kernel  one warp per four output rows [Hkv, d] of K' and of V': 16-byte loads along the source rows' head
-//                  slices, 16-byte stores to the packed rows.  Region of the first row by 32 probes at a time in the
+//   gather_kernel  one warp per four output rows [Hkv, d] of K' and of V' (short rows: eight or sixteen): 16-byte loads along
+//                  the source rows' head slices, 16-byte stores to the packed rows.  Region of the first row by 32 probes at a time in the
 //                  offsets table, of the further ones by walking on.
 #include "common.cuh"
 
@@ -243,7 +243,7 @@ struct GatherParams {
     const int32_t *lens;
     const int32_t *budgets;
     const int32_t *kept;
-    int text_blocks;   // blocks of text rows; those behind them take the kept rows
+    int text_blocks;   // blocks of text rows; those behind them, or all, take the kept rows
     int64_t total_rows;  // rows the output buffers hold
     int64_t kept_cap;    // entries the kept-list buffer holds
     uint32_t *status;
@@ -261,11 +261,14 @@ __host__ __device__ inline int gather_rows_abreast(int vec_per_row) { return vec
 // the text rows (Algorithm 1's C^l = Concat(K_v[kept], K_t)).  A lane moves a part of four rows at a
 // time; short rows (of one head: budgets per KV head) lie side by side in a warp, whose lanes are all at work then: 1280 cells
 // of 3000 + 300 tokens, one head of 128 channels 211 -> 148 us a call.
-// The text rows need no selection result - their place follows from the budgets alone - so the first blocks, which
-// copy them, do not wait for the predecessor in the stream (the selection kernel, which releases its dependents when its
-// last block has started): that part of the traffic runs beside the selection, which is bound by latency, not by
-// bandwidth.  When every block copied some text rows and then waited, the first ones on the SMs held up the text rows of the
-// others: 28 layers of 7290 + 128 tokens 32.3 -> 30.7 us a pass with the budgets.  Bound by the memory.
+// The text rows need no selection result - their place follows from the budgets alone - so they are copied without a wait
+// for the predecessor in the stream (the selection kernel, which releases its dependents when its last block has started):
+// that part of the traffic runs beside the selection, which is bound by latency, not by bandwidth.  They have blocks of
+// their own, in front, or in small calls are copied by the blocks that take the kept rows afterwards (rule: launch_compact).
+// Bound by the memory.
+// SHARED: a block copies text rows, then kept rows.  (An instantiation of its own: the others spill 56 bytes with it, 300
+// regions of 4097 + 24 tokens 97.2 -> 98.7 us a call.)
+template <bool SHARED>
 __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams p) {
     const int lane = threadIdx.x & 31;
     const int n_regions = p.L * p.B * p.Hc;       // cells
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams 
             else dst_row[i] = dst;
         }
         copy_rows(src_off, dst_row);
-        return;
+        if (!SHARED) return;
     }
 
     // ---- kept visual rows: where they go follows from the offsets, what goes there from the selection's lists ----
@@ -333,7 +336,7 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(GatherParams 
         if (threadIdx.x == 0) atomicExch(p.status, kStatusInconsistent);
         n_kept = 0;
     }
-    const int64_t first = (int64_t)((int)blockIdx.x - p.text_blocks) * rows_per_block + (threadIdx.x >> 5) * rows_per_warp;
+    const int64_t first = (int64_t)((int)blockIdx.x - (SHARED ? 0 : p.text_blocks)) * rows_per_block + (threadIdx.x >> 5) * rows_per_warp;
     if (first < n_kept) {
         // Largest r with (kept rows before r) <= first (regions without kept rows are passed over), 32 probes at a
         // time; the further rows are found by walking on.  (A binary search per row and behind the wait
@@ -421,6 +424,26 @@ cudaError_t launch_select(const SelectArgs &a, int blocks, cudaStream_t st) {
                               a.first_row, a.kept, a.kept_cap, a.status);
 }
 
+// Whether the gather kernel's blocks copy text rows and then kept rows, instead of blocks of their own for either.  Separate
+// blocks do not keep kept rows waiting behind text rows, and win wherever there are more blocks than start beside the
+// selection (28 layers of 7290 + 128 tokens 32.3 -> 30.7 us a pass with the budgets; five sequences of 1000 + 32, 140 regions,
+// 21.0 -> 15.9 us a call).  But they put more blocks on some SMs than on others, and a block has an SM's share of the memory
+// rate for 1.5 us.  So blocks are shared where all of one kind start beside the selection and not all of both (28 x 8 regions
+// of 300 + 32 tokens: 15.9 us apart, 12.8 shared), and where, beside a selection of one block an SM, there is less than a
+// text block for every SM that is free, yet one kept block more falls to some of them (28 x 2 of 1000 + 16: 11.7, 10.2).
+// Not with rows above 1 KB, whose text rows take twice as long (80 regions of 600 + 64 tokens: 20.3 apart, 23.4 shared).
+bool gather_shares_blocks(int64_t text, int64_t kept, int row_bytes, int select_blocks, int blocks_per_sm, int sms) {
+    if (row_bytes > 1024) return false;
+    // four gather blocks to an SM, fewer beside blocks of the selection
+    auto beside = [&](int n) { return n >= blocks_per_sm ? 0 : 4 - (4 * n + blocks_per_sm - 1) / blocks_per_sm; };
+    const int each = select_blocks / sms, more = select_blocks % sms;
+    const int64_t room = (int64_t)beside(each) * (sms - more) + (int64_t)beside(each + 1) * more;
+    if (text + kept > room) return (text > kept ? text : kept) <= room;
+    if (blocks_per_sm > 1) return false;
+    const int64_t free = sms - select_blocks;
+    return text <= free && (text + kept + free - 1) / free > (kept + free - 1) / free;
+}
+
 }  // namespace
 
 int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const float *scores,
@@ -450,11 +473,16 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
         return LB >= 2 * few && text_us > 9.0 * ((LB + few - 1) / few) ? few : LB;
     };
     cudaError_t e;
-    const int select_blocks = many && s->n_visual <= 256 * 16 ? blocks_of(256) : many && s->n_visual <= 512 * 16 ? blocks_of(512) : LB;
-    if (many && s->n_visual <= 256 * 16)
+    int blocks_per_sm = 1, select_blocks = LB;   // the most that an SM holds, and how many there are
+    if (many && s->n_visual <= 256 * 16) {
+        blocks_per_sm = 5;
+        select_blocks = blocks_of(256);
         e = select_blocks < LB ? launch_select<256, 16, true>(a, select_blocks, st) : launch_select<256, 16>(a, LB, st);
-    else if (many && s->n_visual <= 512 * 16) e = launch_select<512, 16, true>(a, select_blocks, st);
-    else if (s->n_visual <= 1024 * 8) e = launch_select<1024, 8>(a, LB, st);
+    } else if (many && s->n_visual <= 512 * 16) {
+        blocks_per_sm = 2;
+        select_blocks = blocks_of(512);
+        e = launch_select<512, 16, true>(a, select_blocks, st);
+    } else if (s->n_visual <= 1024 * 8) e = launch_select<1024, 8>(a, LB, st);
     else if (s->n_visual <= 1024 * 16) e = launch_select<1024, 16>(a, LB, st);
     else e = launch_select<1024, 0>(a, LB, st);
     AIRCACHE_CUDA_TRY(e);
@@ -471,11 +499,14 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
     p.Hc = cells_of(s);
     p.L = s->n_layers; p.B = s->batch; p.Hkv = s->n_kv_heads; p.d = s->head_dim;
     p.Nv = s->n_visual; p.Nt = s->n_text; p.slack = s->slack;
-    // One block per 32 rows, or more short ones (a grid limited to the resident blocks, each striding through the rows, measured 20 % slower on
-    // the large configurations).  The text rows' blocks come first and do not wait for the selection; at least one block does.
+    // One block per 32 rows, or more short ones (a grid limited to the resident blocks, each striding through the rows, measured
+    // 20 % slower on the large configurations).  At least one block waits for the selection.
     const int rows_per_block = kGatherThreads / 32 * kGatherRows * gather_rows_abreast(row_heads_of(s) * s->head_dim / 8);
-    p.text_blocks = (int)(((int64_t)LB * s->n_text + rows_per_block - 1) / rows_per_block);
-    const int64_t blocks = p.text_blocks + (kept_cap > 0 ? (kept_cap + rows_per_block - 1) / rows_per_block : 1);
+    const int64_t text = ((int64_t)LB * s->n_text + rows_per_block - 1) / rows_per_block;
+    const int64_t kept_blocks = kept_cap > 0 ? (kept_cap + rows_per_block - 1) / rows_per_block : 1;
+    p.text_blocks = (int)text;
+    const bool shared = gather_shares_blocks(text, kept_blocks, row_heads_of(s) * s->head_dim * 2, select_blocks, blocks_per_sm, sms);
+    const int64_t blocks = !shared ? text + kept_blocks : text > kept_blocks ? text : kept_blocks;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(kGatherThreads);
@@ -486,7 +517,7 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    AIRCACHE_CUDA_TRY(cudaLaunchKernelEx(&cfg, gather_kernel, p));
+    AIRCACHE_CUDA_TRY(shared ? cudaLaunchKernelEx(&cfg, gather_kernel<true>, p) : cudaLaunchKernelEx(&cfg, gather_kernel<false>, p));
     AIRCACHE_LAUNCH_CHECK();
     return AIRCACHE_OK;
 }

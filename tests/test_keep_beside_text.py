@@ -1,6 +1,7 @@
 """Copying of text rows beside the selection: selection by fewer blocks than regions (blocks of 256 and 512 threads that take
-two regions one after the other, and as many regions as blocks), and text rows beside it.  Lists and rows against a library
-sort and plain indexing (whole numbers and copies: equal)."""
+two regions one after the other, and as many regions as blocks), text rows by blocks of their own and by those of the kept rows,
+and short rows side by side in a warp.  Lists and rows against a library sort and plain indexing (whole numbers and copies:
+equal)."""
 import pytest
 import torch
 
@@ -50,3 +51,20 @@ def check_compaction(layers, batch, heads, d, n_visual, n_text, ratio, per_head=
     (37, 4, 64, 4500, 140)])    # 148 regions: a block of 1024 threads each
 def test_compaction_with_many_text_rows(layers, batch, d, n_visual, n_text):
     check_compaction(layers, batch, 8, d, n_visual, n_text, 0.07)
+
+
+@pytest.mark.parametrize("layers,batch,heads,d,n_visual,n_text,ratio,per_head", [
+    (28, 2, 4, 128, 1000, 16, 0.1, 0),     # shared: one kept block more on some SMs
+    (28, 2, 4, 128, 1000, 70, 0.1, 0),     # apart: more text blocks than free SMs
+    (28, 8, 4, 128, 300, 32, 0.1, 0),      # shared: either kind starts beside the selection, not both
+    (28, 8, 4, 128, 300, 3, 0.5, 0),       # many kept, few text blocks
+    (28, 8, 4, 128, 40, 64, 0.05, 0),      # few kept, many text blocks
+    (37, 4, 4, 128, 50, 3, 0.1, 0),        # no SM is free beside the selection
+    (3, 1, 4, 64, 77, 2, 0.02, 0),         # 32 vectors of a row: one row a warp
+    (5, 2, 1, 64, 97, 5, 0.2, 0),          # 8: four rows abreast
+    (7, 3, 2, 64, 333, 21, 0.3, 0),        # 16: two
+    (5, 2, 8, 64, 97, 5, 0.2, 1),          # the same with budgets per KV head
+    (9, 5, 4, 128, 301, 33, 0.1, 1),
+    (4, 1, 2, 64, 5, 2, 1.0, 0)])
+def test_text_and_kept_rows_in_one_block_or_two(layers, batch, heads, d, n_visual, n_text, ratio, per_head):
+    check_compaction(layers, batch, heads, d, n_visual, n_text, ratio, per_head)
