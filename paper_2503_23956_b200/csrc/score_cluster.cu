@@ -644,7 +644,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                             tmem_st_wait();
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                if (q < quads) {
+                                if (q < quads && __any_sync(0xffffffffu, fmaxf(fmaxf(x[4 * q], x[4 * q + 1]),
+                                                                               fmaxf(x[4 * q + 2], x[4 * q + 3])) > kRescale)) {
                                     float fac[4], raw[4];
                                     tmem_ld4(base + t * kRows + 4 * q, raw);
 #pragma unroll
