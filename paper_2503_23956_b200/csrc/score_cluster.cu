@@ -68,7 +68,7 @@ constexpr float kMiddle = 0.5f * (kRescale - 126.f);   // of the exponents that 
 constexpr float kFarDown = 7.888609052210118e-31f;   // 2^-100
 constexpr float kScaleUp = 18446744073709551616.f;   // 2^64
 constexpr int kPreloadRows = 128;     // window queries of a group that fit a ring stage
-constexpr int kFirstAhead = 5;        // tiles asked into L2 behind the first full ring
+constexpr int kFirstAhead = 5;        // tiles asked into L2 ahead of the wait, behind the first full ring
 
 struct ClusterSmem {   // small state behind the ring and the query block
     uint64_t full[kMaxStages], empty[kMaxStages];
@@ -220,9 +220,6 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
                     const int g = grp % p.Hkv, lb = grp / p.Hkv, l = lb / p.B, b = lb - l * p.B;
                     for (bool last = false; ok && !last; ++u) {
                         for (int t = 0; t < T; ++t, ++it) {
-                            if (it == (uint32_t)S - 1)   // the first query rows are some microseconds away: a few tiles more
-                                for (int t2 = t; t2 < T && t2 < S + kFirstAhead; ++t2)   // come as far as L2 meanwhile
-                                    prefetch_key_tile<D>(&tm_k, p, key0 + t2 * 128, g, b, l);
                             const uint32_t st = it % S;
                             ok = mbar_wait(smem_u32(&sm.empty[st]), ((it / S) & 1) ^ 1, abort_flag, p.status, 20) &&
                                  (it != (uint32_t)S - 1 || mbar_wait(smem_u32(&sm.q_taken), 0, abort_flag, p.status, 31));
