@@ -96,8 +96,56 @@ def test_candidates_at_the_threshold(oracle_mod, window, alpha):
         assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
         sides.add(int(ref["elite_mask"].reshape(-1)[0]))
     close = [abs(float(k[0, 0, -window + w, 0].double() @ last.double()) - top - wanted) for w in range(2, window, 3)]
-    norms = float(last.double().norm()) * max(float(k[0, 0, -window + w, 0].double().norm()) for w in range(window))
-    assert min(close) < 5.5e-6 * norms, "no candidate is as close as the fp32 decision's slack"
+    size = max(float((k[0, 0, -window + w, 0].double() * last.double()).abs().sum()) for w in range(window))
+    assert min(close) < 9e-6 * size, "no candidate is as close as the fp32 decision's slack"
+
+
+def logit_sum_fp32(q, k):
+    """The kernel's fp32 dot product: even and odd channels in element order, then one addition."""
+    sums = [np.float32(0), np.float32(0)]
+    for c, x in enumerate((q.double() * k.double()).tolist()):
+        sums[c & 1] = np.float32(float(sums[c & 1]) + x)
+    return np.float32(sums[0] + sums[1])
+
+
+@pytest.mark.parametrize("window", [8, 32, 33, 128])
+def test_candidates_that_cancel_at_the_threshold(oracle_mod, window):
+    """Candidates whose products are large and cancel, within some 1e-4 of the threshold on both sides: their fp32 sums are off by
+    more than that and decide several of them wrongly, the sum of the products' magnitudes (the slack, taken by shuffles up
+    to 32 candidates and by an atomic maximum beyond) has to send them to the fp64 sums."""
+    alpha, scale = 0.5, 0.09
+    wl = workload(1, (14, 2), 128, 1, 300, window, alpha, n_text=window + 3)
+    k, v, qw = gen_inputs(wl, "cpu")
+    gen = torch.Generator().manual_seed(window)
+    last = torch.randn(128, generator=gen).to(torch.bfloat16)
+    last[64:] = last[:64]
+    last[127], last[63] = 2.0 ** -5, 2.0 ** -14   # two channels to aim with, the others cancel
+    qw[:, :, -1] = last
+    q = last.double()
+    wanted = np.log(alpha) / scale   # below the best candidate's logit, which is zero
+    exact, rough = [], []
+    for w in range(window):
+        row = torch.zeros(128, dtype=torch.bfloat16)
+        if w:
+            row[:63] = (300 * torch.randn(63, generator=gen)).to(torch.bfloat16)
+            row[64:127] = -row[:63]
+            aim = wanted + (w - window / 2) * 2e-4 / window
+            for c in (127, 63):
+                row[c] = torch.tensor((aim - float(row.double() @ q)) / float(q[c])).to(torch.bfloat16)
+            exact.append(float(row.double() @ q) - wanted)
+            rough.append(float(logit_sum_fp32(last, row)) - wanted)
+            assert abs(exact[-1]) < 9e-6 * float((row.double() * q).abs().sum())
+        k[:, :, -window + w] = row
+    assert any((a > 0) != (b > 0) for a, b in zip(exact, rough)), "fp32 sums decide as the exact ones do"
+    assert min(exact) < 0 < max(exact)
+    dm = oracle_dims(oracle_mod, wl)
+    ref = oracle_mod.score(dm, u16(logical(k)), u16(qw), scale, alpha)
+    gp = GpuPath(wl, device=DEV)
+    gp.sh.scale = scale
+    gp.set_full(logical(k.to(DEV)), logical(v.to(DEV)))
+    gp.score(qw.to(DEV), alpha=alpha)
+    assert gp.status() == 0
+    assert np.array_equal(gp.mask.cpu().numpy().view(np.uint64), ref["elite_mask"])
 
 
 @pytest.mark.parametrize("heads,d,window,alpha,n_visual,per_head", [
