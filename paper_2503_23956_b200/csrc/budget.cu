@@ -10,7 +10,7 @@
 // across the lanes.  The CTA that finishes the last sequence scans the region sizes into offsets.
 //
 // A chain of latencies, most of it fp64.  With 512 threads, three reductions and a division per score it took 17.5 us for
-// 28 cells of 7290 scores and 47 us for 1792 of 2916; now 11 and 25 us.  (Five blocks of 256 threads to an SM instead of
+// 28 cells of 7290 scores and 47 us for 1792 of 2916; now 9.3 and 22 us.  (Five blocks of 256 threads to an SM instead of
 // four spill registers and gain nothing.)
 #include <math.h>
 

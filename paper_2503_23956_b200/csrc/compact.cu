@@ -240,7 +240,6 @@ struct GatherParams {
     int64_t s_layer, s_batch, s_head, s_token;
     uint16_t *k_out, *v_out;
     const int64_t *offsets;
-    const int32_t *lens;
     const int32_t *budgets;
     const int32_t *kept;
     int text_blocks;   // blocks of text rows; those behind them, or all, take the kept rows
@@ -254,7 +253,8 @@ struct GatherParams {
 
 constexpr int kGatherThreads = 256;
 constexpr int kGatherRows = 4;   // of a lane
-// Rows that lie side by side in a warp: a row of one or two heads has fewer 16-byte vectors (a power of two) than a warp lanes.
+// Rows that lie side by side in a warp: a row has heads x channels / 8 vectors of 16 bytes, a power of two from 8 to 128 (1, 2, 4
+// or 8 heads of 64 or 128 channels), and one of 8 or 16 leaves lanes to others.
 __host__ __device__ inline int gather_rows_abreast(int vec_per_row) { return vec_per_row < 32 ? 32 / vec_per_row : 1; }
 
 // Copies the rows of the ragged cache: for region r first the kept visual rows in ascending token order, then
@@ -491,7 +491,7 @@ int launch_compact(const aircache_shape_t *s, const aircache_full_t *f, const fl
     p.k = (const uint16_t *)f->k; p.v = (const uint16_t *)f->v;
     p.s_layer = f->stride_layer; p.s_batch = f->stride_batch; p.s_head = f->stride_head; p.s_token = f->stride_token;
     p.k_out = (uint16_t *)out->k; p.v_out = (uint16_t *)out->v;
-    p.offsets = out->offsets; p.lens = out->lens; p.budgets = budgets; p.kept = kept;
+    p.offsets = out->offsets; p.budgets = budgets; p.kept = kept;
     p.first_row = out->first_row;
     p.total_rows = out->total_rows;
     p.kept_cap = kept_cap;

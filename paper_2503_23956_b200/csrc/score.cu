@@ -801,7 +801,7 @@ int launch_group_sum(const ScoreParams &p, cudaStream_t st) {
 // Many KV groups of hardly a tile of keys: a cluster then spends its time on a group's elite rows, one unit of 16 after the
 // other, with two blocks to an SM; elite_kernel and the one-pass kernel hold six and five.  What there is of it grows with
 // the elite rows, of which a low alpha leaves many, and large groups fill the cluster kernel's units better.  Measured
-// (older kernels, cluster kernel; us a call):
+// (older kernels, cluster kernel, the latter when a one-layer call took it 17 us, 13.7 since; us a call):
 //   14336 groups of 4 heads, 64 channels, 16 window queries: alpha 0.9, 3 tokens 210, 270; 32 tokens 242, 277; 96 tokens 306,
 //   278.  alpha 0.1, 3 tokens 508, 944; 64 tokens 700, 939; 128 tokens 954, 961.  alpha 0.3, 16 tokens 346, 596.
 //   3584 groups of 2 heads: alpha 0.9, 32 tokens 64, 79; 128 tokens 92, 90 (alpha 0.5).  14336 groups of 1 head of 128 channels:

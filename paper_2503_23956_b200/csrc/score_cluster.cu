@@ -29,17 +29,18 @@
 // What it replaced (elite kernel, one-pass kernel on mma.sync with a wait between blocks, sum kernel) streamed keys
 // during half of a block's life and took three launches.  Measured, 28 layers of 28 query and 4 KV heads of 128
 // channels: 64 sequences of 2916 tokens 1196 -> 835 to 870 us by the box (6.2 TB/s of keys: at the memory's rate); one of
-// 7290 tokens 75 -> 41.4 us; four of 6272, a call per layer, 33 -> 13.9 us a call.  A call of one layer is a chain of latencies (us
-// behind the wait for what is before it in the stream): 1.4 until the rows of the first query block are staged, 4.2 until
-// the block is ready, 8.2 until the last tile has been multiplied, 12 at the end; then the sum over groups and the launches'
-// hand-over, 3.  What shortened it from 17: the first rows and tiles are asked into L2 and the addresses worked out ahead of
+// 7290 tokens 75 -> 41 us; four of 6272, a call per layer, 33 -> 13.7 us a call.  A call of one layer is a chain of latencies (us
+// behind the wait for what is before it in the stream, when a call took 13.9): 1.2 until the rows of the first query block are
+// staged, 4 until the block is ready, 8 until the last tile has been multiplied, 11.5 at the end; then the sum over groups
+// and the launches' hand-over, 2.4.  What shortened it from 17: the first rows and tiles are asked into L2 and the addresses worked out ahead of
 // the wait, an idle warp's lanes ask for the window's queries (one thread took 1 us for the 16 copies), the text columns'
 // statistics and the masks are written behind the query block, which does not need them, and no block waits for its
 // cluster at its end: 16.9 -> 15.5 us; image 47.6 -> 45.3.  A reference per warp (below) left no maxima to take behind the
 // last tile and the factors to one lane a row, and the first tile's exponentials come back beside the exchange: 14.6; 43.2.
 // (The next tile's beside the sums of one: 104 bytes of spills, image 53.)  The bound that decides whether a head needs its
 // fp64 sums comes out of the fp32 dot products themselves and no longer from norms taken while the rows were stored: 14.3 ->
-// 13.9; 42.4 -> 41.4.
+// 13.9; 42.4 -> 41.4.  (That bound is 1.08 times the one from norms at normally distributed rows: two chains of 64 products instead
+// of four of 32.)  The first tiles asked into L2 once, and not again by the producer: 13.8 -> 13.7; 41.4 -> 41.0.
 //
 // With up to eight tiles per block the tensor memory holds two units of work and the tensor core runs ahead of the
 // epilogue; with up to sixteen the other block of the SM fills the gap.  All waits are bounded.
@@ -92,6 +93,8 @@ struct ClusterCfg {
     static constexpr int Q_SUB = kRows * 128;
     static constexpr int Q_BYTES = D / 64 * Q_SUB;
     static constexpr int KS = D + 8;   // padded row of the staged candidate keys and last queries
+    // (W more words than the logits and sums take: without them 13 pairs of window and group of 128 channels would have room
+    // for a second ring stage and come here from the older kernels, 33 others for one stage more; neither was measured)
     static int tail_bytes(int W, int G) {
         return (int)sizeof(ClusterSmem) + (W + G) * KS * 2 + (G * W * 4 + (W + G) * 4 + 15) / 16 * 16;
     }
@@ -310,7 +313,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tm_k, ScoreParams p, Cl
         // Eq. 4, last row only: the logit of candidate w for head hl.  The decision of Eq. 5 is defined on fp64 dot
         // products in element order, rounded to fp32.  fp32 dot products settle it wherever the difference to the
         // threshold exceeds what the two can differ by; a head with a candidate closer than that is done again in fp64
-        // (about one group in 200).  The fp64 chain alone took 2-4 us of a one-layer call's 19.
+        // (about one group in 450).  The fp64 chain alone took 2-4 us of a one-layer call's 19.
         auto logit_fp32 = [&](int hl, int w, float &size) {   // size: the sum of the products' magnitudes
             const uint4 *q = reinterpret_cast<const uint4 *>(s_k + (p.W + hl) * C::KS);
             const uint4 *kk = reinterpret_cast<const uint4 *>(s_k + w * C::KS);
@@ -877,7 +880,7 @@ int launch_score_cluster_d(ScoreParams &p, const aircache_shape_t *s, const airc
     CUtensorMap tm;
     if (make_key_map(&tm, p, s, f) != AIRCACHE_OK) return AIRCACHE_OK;
 
-    // Cluster size and groups per item by estimated time (ns).  Measured on a B200: HBM delivers a tile of 128 keys by
+    // Cluster size and groups per item by estimated time (ns).  Measured on a B200, when a one-layer call took 17 us (13.7 since): HBM delivers a tile of 128 keys by
     // 128 channels in 5.3 ns over all SMs; a unit takes a block 0.6 us per tile plus the exchange (4 us where the tensor
     // memory holds one unit only, else hidden), and never less than the elite rows of the next group, 9 us.  A sum over
     // groups in a kernel of its own adds 2.5 us and 3 % of the traffic.
